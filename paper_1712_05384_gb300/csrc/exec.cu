@@ -1688,75 +1688,233 @@ __global__ void k_grad_reduce(const char *ws, const GradParam *gp, const uint64_
 }
 
 // ---------------------------------------------------------------------------
-// Cross-entropy statistics (App. B): FP64 sums of log p, N p and (N p)^2 over
-// the amplitudes, one block of 1024 threads.
-__global__ void __launch_bounds__(1024) k_xeb(const double2 *a, int64_t B, double N, double *sums) {
-  __shared__ double r0[1024], r1[1024], r2[1024];
-  double s0 = 0, s1 = 0, s2 = 0;
-  for (int64_t b = threadIdx.x; b < B; b += blockDim.x) {
+// Statistics of a computed set (App. B) and samples from it (App. C).
+//
+// Both are bound by FP64 arithmetic (about 2 FMA per clock and SM here), not
+// by the 16 bytes per amplitude, so work is spread over SMs and kept to a few
+// FP64 operations per amplitude.  Statistics of 65536 amplitudes and 10000
+// samples of them: 889 us with one CTA per sum and a logarithm per amplitude,
+// 65 us as below (k_xeb 27, the three k_cdf kernels 12, k_sample 8.5, the
+// rest the host's wait for the statistics).
+//
+// The statistics run as one thread-block cluster of SET_CTAS CTAs (the
+// largest portable cluster) whose partial results meet in distributed shared
+// memory: no scratch beyond the caller's four doubles, a fixed order of every
+// sum.  Sum of log p over the set = log of the product: each thread
+// multiplies the significands (renormalised to [1, 2) after every factor, a
+// relative rounding of 2^-53 each, below the rounding of adding logarithms)
+// and adds the binary exponents as integers; only the whole product's
+// logarithm (about 45 FP64 operations) is taken.
+constexpr int SET_CTAS = 8, SET_THREADS = 1024;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
+// This CTA's shared variable in CTA `rank` of the cluster
+__device__ __forceinline__ double cluster_peek(const double *v, uint32_t rank) {
+  uint32_t a;
+  double x;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(v)), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(a) : "memory");
+  return x;
+}
+
+// A positive value as m * 2^e with m in [1, 2)
+struct LogSum {
+  double m;
+  int64_t e;
+};
+
+__device__ __forceinline__ LogSum log_mul(LogSum a, LogSum b) {
+  const double m = a.m * b.m;  // in [1, 4)
+  const int64_t bits = __double_as_longlong(m);
+  const int64_t x = ((bits >> 52) & 0x7ff) - 1023;
+  return {__longlong_as_double(bits - (x << 52)), a.e + b.e + x};
+}
+
+// FP64 sums of log p, N p and (N p)^2 over the amplitudes.
+__global__ void __launch_bounds__(SET_THREADS) k_xeb(const double2 *a, int64_t B, double N, double *sums) {
+  __shared__ double wm[32], w1[32], w2[32], wx[32];
+  __shared__ int64_t we[32];
+  __shared__ double part[5];  // significand, exponent, irregular logs, N p, (N p)^2
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  LogSum L{1.0, 0};
+  double sx = 0, s1 = 0, s2 = 0;
+  for (int64_t b = (int64_t)blockIdx.x * SET_THREADS + tid; b < B; b += SET_CTAS * SET_THREADS) {
     const double p = a[b].x * a[b].x + a[b].y * a[b].y;
-    s0 += log(p);
+    const int64_t bits = __double_as_longlong(p);
+    const uint32_t x = (uint32_t)(bits >> 52);  // p >= 0 (or NaN): sign and exponent
+    if (x - 1u < 0x7feu) L = log_mul(L, {__longlong_as_double((bits & 0xfffffffffffffll) | (1023ll << 52)), (int64_t)x - 1023});
+    else sx += log(p);  // zero, subnormal, infinite or NaN
     s1 += N * p;
     s2 += (N * p) * (N * p);
   }
-  r0[threadIdx.x] = s0;
-  r1[threadIdx.x] = s1;
-  r2[threadIdx.x] = s2;
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) {
-      r0[threadIdx.x] += r0[threadIdx.x + h];
-      r1[threadIdx.x] += r1[threadIdx.x + h];
-      r2[threadIdx.x] += r2[threadIdx.x + h];
+  auto reduce = [&](int n) {
+    for (int o = n / 2; o > 0; o >>= 1) {
+      const LogSum q{__shfl_xor_sync(0xffffffffu, L.m, o), __shfl_xor_sync(0xffffffffu, L.e, o)};
+      L = log_mul(L, q);
+      sx += __shfl_xor_sync(0xffffffffu, sx, o);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
-    __syncthreads();
+  };
+  reduce(32);
+  if (lane == 0) {
+    wm[wid] = L.m;
+    we[wid] = L.e;
+    wx[wid] = sx;
+    w1[wid] = s1;
+    w2[wid] = s2;
   }
-  if (threadIdx.x == 0) {
-    sums[0] = r0[0];
-    sums[1] = r1[0];
-    sums[2] = r2[0];
+  __syncthreads();
+  if (wid == 0) {
+    L = {wm[lane], we[lane]};
+    sx = wx[lane];
+    s1 = w1[lane];
+    s2 = w2[lane];
+    reduce(32);
+    if (lane == 0) {
+      part[0] = L.m;
+      part[1] = (double)L.e;  // |e| <= 1074 B: exact
+      part[2] = sx;
+      part[3] = s1;
+      part[4] = s2;
+    }
   }
+  cluster_sync();
+  if (cluster_rank() == 0 && wid == 0) {
+    const bool have = lane < SET_CTAS;
+    L = {have ? cluster_peek(&part[0], lane) : 1.0, have ? (int64_t)cluster_peek(&part[1], lane) : 0};
+    sx = have ? cluster_peek(&part[2], lane) : 0.0;
+    s1 = have ? cluster_peek(&part[3], lane) : 0.0;
+    s2 = have ? cluster_peek(&part[4], lane) : 0.0;
+    reduce(32);
+    if (lane == 0) {
+      sums[0] = sx + (log(L.m) + (double)L.e * 0.693147180559945309417);
+      sums[1] = s1;
+      sums[2] = s2;
+    }
+  }
+  cluster_sync();  // a CTA's shared memory stays until it has been read
 }
 
-// Cumulative sums of p_j = |a_j|^2 (one block: each thread sums a contiguous
-// chunk, a block scan of the chunk totals, then each chunk is written out).
-__global__ void __launch_bounds__(1024) k_cumsum_p(const double2 *a, int64_t t, double *cdf) {
-  __shared__ double part[1024];
-  const int64_t chunk = (t + blockDim.x - 1) / blockDim.x;
-  const int64_t lo = threadIdx.x * chunk, hi = lo + chunk < t ? lo + chunk : t;
-  double s = 0;
-  for (int64_t j = lo; j < hi; ++j) s += a[j].x * a[j].x + a[j].y * a[j].y;
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int i = 1; i < (int)blockDim.x; ++i) part[i] += part[i - 1];
-  __syncthreads();
-  double run = threadIdx.x ? part[threadIdx.x - 1] : 0.0;
-  for (int64_t j = lo; j < hi; ++j) {
-    run += a[j].x * a[j].x + a[j].y * a[j].y;
-    cdf[j] = run;
+// Inclusive scan over a block of 256 of one value per thread; *sum = total.
+__device__ __forceinline__ double block_scan(double v, double *sum) {
+  __shared__ double wsum[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const double u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
   }
+  __syncthreads();  // the previous call's wsum is read
+  if (lane == 31) wsum[wid] = v;
+  __syncthreads();
+  double before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    before += w < wid ? wsum[w] : 0.0;
+    all += wsum[w];
+  }
+  *sum = all;
+  return before + v;
+}
+
+// Cumulative sums of p_j = |a_j|^2 over chunks of CDF_CHUNK values, one block
+// each, on all SMs (one cluster would be bound by its FP64 units): the
+// chunk's total goes to the chunk's first entry of cdf, one block turns these
+// into the sums before each chunk, and each block then reads its own and
+// writes its chunk.
+constexpr int CDF_CHUNK = 512;
+__device__ __forceinline__ double p_of(const double2 *a, int64_t j, int64_t t) {
+  return j < t ? a[j].x * a[j].x + a[j].y * a[j].y : 0.0;
+}
+__global__ void __launch_bounds__(256) k_cdf_totals(const double2 *a, int64_t t, double *cdf) {
+  const int64_t j = (int64_t)blockIdx.x * CDF_CHUNK + 2 * threadIdx.x;
+  double s = p_of(a, j, t) + p_of(a, j + 1, t), all;
+  block_scan(s, &all);
+  if (threadIdx.x == 0) cdf[(int64_t)blockIdx.x * CDF_CHUNK] = all;
+}
+__global__ void __launch_bounds__(256) k_cdf_before(int64_t n, double *cdf) {
+  double run = 0;
+  for (int64_t c0 = 0; c0 < n; c0 += 256) {
+    const int64_t c = c0 + threadIdx.x;
+    const double v = c < n ? cdf[c * CDF_CHUNK] : 0.0;
+    double all;
+    const double s = block_scan(v, &all);
+    if (c < n) cdf[c * CDF_CHUNK] = run + (s - v);
+    run += all;
+  }
+}
+__global__ void __launch_bounds__(256) k_cdf_chunks(const double2 *a, int64_t t, double *cdf) {
+  const int64_t j = (int64_t)blockIdx.x * CDF_CHUNK + 2 * threadIdx.x;
+  const double p0 = p_of(a, j, t), p1 = p_of(a, j + 1, t);
+  const double run = cdf[(int64_t)blockIdx.x * CDF_CHUNK];
+  double all;
+  const double s = run + block_scan(p0 + p1, &all);  // its barriers order the read before the writes
+  if (j < t) cdf[j] = s - p1;
+  if (j + 1 < t) cdf[j + 1] = s;
 }
 
 // Draw i: u = the i-th output of SplitMix64(seed) (counter form: the state
 // after i + 1 golden-ratio increments, then the two mixing rounds), top 53
-// bits; index = first j with cdf[j] / total > u.
-__global__ void k_sample(const double *cdf, int64_t t, int64_t m, uint64_t seed, int64_t *idx) {
+// bits; index = first j with cdf[j] / total > u.  The search runs on
+// cdf[j] > u * total, its first levels over SAMPLE_COARSE entries staged in
+// shared memory (a search in global memory is a chain of L2 latencies), and
+// the defining quotient is checked around the place found.
+constexpr int SAMPLE_COARSE = 512;
+__global__ void __launch_bounds__(256) k_sample(const double *cdf, int64_t t, int64_t m, uint64_t seed, int64_t *idx) {
+  __shared__ double coarse[SAMPLE_COARSE];
+  const int64_t stride = (t + SAMPLE_COARSE - 1) / SAMPLE_COARSE;
+  const int nc = (int)((t + stride - 1) / stride);  // coarse[c]: last entry of block c
+  for (int c = threadIdx.x; c < nc; c += blockDim.x) coarse[c] = cdf[((c + 1) * stride < t ? (c + 1) * stride : t) - 1];
+  __syncthreads();
+  const double total = coarse[nc - 1];
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     uint64_t z = seed + (uint64_t)(i + 1) * 0x9E3779B97F4A7C15ULL;
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     z ^= z >> 31;
     const double u = (double)(z >> 11) * (1.0 / 9007199254740992.0);
-    const double total = cdf[t - 1];
-    int64_t lo = 0, hi = t - 1;
+    const double v = u * total;
+    int c0 = 0, c1 = nc - 1;
+    while (c0 < c1) {
+      const int mid = (c0 + c1) >> 1;
+      if (coarse[mid] > v) c1 = mid;
+      else c0 = mid + 1;
+    }
+    int64_t lo = c0 * stride, hi = (c0 + 1) * stride < t ? (c0 + 1) * stride - 1 : t - 1;
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
-      if (cdf[mid] / total > u) hi = mid;
+      if (cdf[mid] > v) hi = mid;
       else lo = mid + 1;
     }
+    while (lo > 0 && cdf[lo - 1] / total > u) --lo;
+    while (lo < t - 1 && !(cdf[lo] / total > u)) ++lo;
     idx[i] = lo;
   }
+}
+
+// Launch of a one-cluster kernel of SET_CTAS CTAs
+template <typename... A>
+cudaError_t launch_set(void (*k)(A...), cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(SET_CTAS);
+  cfg.blockDim = dim3(SET_THREADS);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = SET_CTAS;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 // FP32 peak microbenchmark: independent FMA chains per thread (enough of
@@ -3178,8 +3336,7 @@ int qgm_xeb_stats(const double *d_amps, int64_t B, int n_qubits, double *d_scrat
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const double N = std::ldexp(1.0, n_qubits);
-  k_xeb<<<1, 1024, 0, st>>>(reinterpret_cast<const double2 *>(d_amps), B, N, d_scratch);
-  CK(cudaGetLastError());
+  CK(launch_set(k_xeb, st, reinterpret_cast<const double2 *>(d_amps), B, N, d_scratch));
   double h[3];
   CK(cudaMemcpyAsync(h, d_scratch, sizeof h, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -3200,7 +3357,15 @@ int qgm_sample_from_set(const double *d_amps, int64_t t, int64_t m, uint64_t see
   }
   if (m == 0) return QGM_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  k_cumsum_p<<<1, 1024, 0, st>>>(reinterpret_cast<const double2 *>(d_amps), t, d_scratch);
+  const double2 *amps = reinterpret_cast<const double2 *>(d_amps);
+  const int64_t chunks = (t + CDF_CHUNK - 1) / CDF_CHUNK;
+  if (chunks >= ((int64_t)1 << 31)) {
+    set_error("qgm_sample_from_set: more than 2^40 amplitudes");
+    return QGM_ERR_ARG;
+  }
+  k_cdf_totals<<<(unsigned)chunks, 256, 0, st>>>(amps, t, d_scratch);
+  k_cdf_before<<<1, 256, 0, st>>>(chunks, d_scratch);
+  k_cdf_chunks<<<(unsigned)chunks, 256, 0, st>>>(amps, t, d_scratch);
   const int64_t blocks = std::min<int64_t>((m + 255) / 256, 4096);
   k_sample<<<(unsigned)blocks, 256, 0, st>>>(d_scratch, t, m, seed, d_idx);
   CK(cudaGetLastError());

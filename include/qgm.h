@@ -277,8 +277,9 @@ int qgm_plan_get_steps(const qgm_plan *p, int32_t *out_rank, int32_t *k, int32_t
                        int32_t *batched, int64_t cap);
 /* Kernel that runs step s in the stepwise executor: 0 product-sum without a
  * batch axis, 1 batched product-sum, 2 batched with a register tile, 3 tiled
- * GEMM, 4 a small step without a batch axis run with its neighbours of the
- * same kind in one single-CTA launch. */
+ * GEMM, 4 a small step without a batch axis among neighbours of the same
+ * kind.  Small steps of any kind share a launch (a segment of the pass's step
+ * program); large ones run with the kernel named here. */
 int qgm_plan_get_step_kernels(const qgm_plan *p, int32_t *kind, int64_t cap);
 
 /* Algorithmic cost of step s: bytes[s] (inputs read once + output written,
@@ -306,7 +307,7 @@ int qgm_plan_get_tuning(const qgm_plan *p, int32_t *rec, float *ms, int64_t cap,
  * 0/1/2/4, in-kernel conversion 0/1, terms in flight 0/2/4/8, product-sum
  * form of a GEMM-shaped step 0/1 (only where no tensor of the step keeps its
  * batch entry outermost); a parameter that does not apply to the step is
- * ignored), e.g. to reuse a tuning saved
+ * ignored, as are all of a small step that shares a launch), e.g. to reuse a tuning saved
  * from an earlier bind without timing again.  After qgm_plan_bind (which
  * resets them); the next call re-captures its pass.  QGM_ERR_ARG on a bad
  * record (nothing changed). */

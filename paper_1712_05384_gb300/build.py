@@ -7,7 +7,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libqgm.so")
-SOURCES = ["host.cpp", "jit.cpp", "exec.cu"]
+SOURCES = ["host.cpp", "program.cpp", "jit.cpp", "exec.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

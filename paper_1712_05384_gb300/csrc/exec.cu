@@ -92,6 +92,12 @@ __device__ __forceinline__ float fmax_nan(float a, float b) { return (a > b || a
 
 __device__ __forceinline__ float absmax2(float2 a) { return fmax_nan(fabsf(a.x), fabsf(a.y)); }
 
+__device__ __forceinline__ uint64_t gtimer() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 // Block-wide max of non-negative floats, then one atomicMax on the slot
 // (non-negative IEEE floats order like their unsigned bit patterns).
 __device__ __forceinline__ void record_max(float v, Meta *meta, int slot) {
@@ -111,16 +117,19 @@ __device__ __forceinline__ void record_max(float v, Meta *meta, int slot) {
 
 // Leaf factors for the current slice and batch: base table entry chosen by
 // the leaf's internal row, the slice bits and the output bits of x_beta.
-// One block per leaf; block 0 also clears the intermediate metadata.
+// One block per leaf; block 0 also clears the intermediate metadata and the
+// step program's sync words.
 __global__ void k_build_leaves(char *ws, const LeafDesc *leaves, int n_leaves, Meta *meta,
                                int n_meta, const Header *hdr, const uint64_t *bits, int64_t B,
-                               int Bp) {
+                               int Bp, int32_t *sync, int n_sync) {
   const int li = blockIdx.x;
-  if (li == 0)
+  if (li == 0) {
     for (int i = threadIdx.x; i < n_meta; i += blockDim.x) {
       meta[i].maxbits = 0;
       meta[i].exp = 0;
     }
+    for (int i = threadIdx.x; i < n_sync; i += blockDim.x) sync[i] = 0;
+  }
   if (li >= n_leaves) return;
   const LeafDesc d = leaves[li];
   const int slice = hdr->slice_id;
@@ -645,98 +654,352 @@ __global__ void __launch_bounds__(256)
   record_max(lmax, meta, d.out_meta);
 }
 
-// A run of small product-sum steps without a batch axis in one launch of one
-// CTA: the steps run in plan order, each as in k_step_plain over a stride of
-// 256 rows, separated by block barriers (which make each step's outputs and
-// exponent visible to the next).  Tensors written inside the launch are read
-// with ordinary loads (not the read-only path); the recorded maximum of each
-// output is stored by thread 0 after a block reduction, and the metadata is
-// read through volatile loads, so no stale copy is used.
-__global__ void __launch_bounds__(256)
-    k_step_plain_group(char *ws, const StepDesc *descs, int first, int count, Meta *meta, Header *hdr) {
-  __shared__ int64_t rowtab[MAXIN][ROWTAB];
-  __shared__ int64_t etab[MAXIN][ETAB];
-  __shared__ float red[8];
+// ---------------------------------------------------------------------------
+// A segment of a step program: all small steps between two large ones in one
+// launch (see PStep, PTask and build_program).
+//
+// Bound: latency.  Most steps of a plan are a few thousand products; alone in
+// a launch each costs 5 us and more (its launch, then a chain of dependent
+// reads: descriptor, index runs, operand maxima, operands), and only one step
+// runs at a time although the elimination tree is wide.  Here CTAs take units
+// of work (a step, a part of one, or a chain of steps) from a ticket counter
+// and wait for the steps a unit reads on counters in memory, so a level of the
+// tree costs one wait and one signal through L2 (about 2 us) and independent
+// branches run side by side.  The index maps are evaluated per item from the
+// runs (a few shifts); only the summed bits' offsets, shared by all items, are
+// tabulated, in shared memory.  Four terms' loads are in flight per thread.
+// Passes before (a launch per step, or runs of batch-free steps in one CTA)
+// and now: 4x4 depth 10, all outputs 167 -> 47 us; 5x5 depth 20, 37
+// bitstrings with 6 open outputs 606 -> 100 us; 5x6 depth 30 in 8 slices 13.95
+// -> 4.8 ms; gradient of 6x6 depth 20, 256 bitstrings 8.3 -> 2.8 ms.
+//
+// Units are numbered producers first, and a CTA takes one unit at a time: the
+// unfinished unit of the lowest number never waits for an unfinished one, so
+// the segment always advances, whatever the number of resident CTAs.  Waits
+// are bounded all the same (one second); one that runs out raises the abort
+// word, every CTA leaves, and the status is QGM_ERR_TIMEOUT.
+//
+// Data written by other CTAs of the launch is read with ordinary loads after
+// an acquire of the counter (no read-only path).
+constexpr int PROG_THREADS = 256;
+
+__device__ __forceinline__ int ld_acquire(const int *p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ bool prog_wait(const int *done, int need, const int *abort_word) {
+  if (ld_acquire(done) >= need) return true;
+  const uint64_t t0 = gtimer();
+  while (ld_acquire(done) < need) {
+    __nanosleep(40);
+    if (gtimer() - t0 > 1000000000ull || *(const volatile int *)abort_word) return false;
+  }
+  return true;
+}
+
+__device__ __forceinline__ int run_index(const uint32_t *run, int n, uint32_t x) {
+  int r = 0;
+#pragma unroll 1
+  for (int q = 0; q < n; ++q) {
+    const uint32_t u = run[q];
+    r += (int)(((x >> (u & 255u)) & ((1u << ((u >> 8) & 255u)) - 1u)) << (u >> 16));
+  }
+  return r;
+}
+
+__device__ __forceinline__ float4 prog_load(const char *a, bool batched, bool pair) {
+  if (pair && batched) return *reinterpret_cast<const float4 *>(a);
+  const float2 v = *reinterpret_cast<const float2 *>(a);
+  return make_float4(v.x, v.y, v.x, v.y);
+}
+
+// An item's place: its row j and batch pair pr.
+template <bool PAIR>
+__device__ __forceinline__ void prog_place(const PStep &S, int it, uint32_t *j, uint32_t *pr) {
+  *j = PAIR ? (uint32_t)it / (uint32_t)S.pairs : (uint32_t)it;
+  *pr = PAIR ? (uint32_t)it - *j * (uint32_t)S.pairs : 0u;
+}
+
+// Sum over the lanes sharing an item (aligned groups of a warp), times comb,
+// stored by their first lane; returns the bits of max(|re|, |im|) stored.
+template <bool PAIR>
+__device__ __forceinline__ uint32_t prog_store(const PStep &S, char *ws, float4 acc, float comb, bool live, uint32_t j,
+                                               uint32_t pr, int Bp) {
+#pragma unroll 1
+  for (int q = 1; q < (1 << S.lg); q <<= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, q);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, q);
+    if (PAIR) {
+      acc.z += __shfl_xor_sync(0xffffffffu, acc.z, q);
+      acc.w += __shfl_xor_sync(0xffffffffu, acc.w, q);
+    }
+  }
+  if (!live || (threadIdx.x & ((1 << S.lg) - 1))) return 0u;
+  acc = make_float4(acc.x * comb, acc.y * comb, acc.z * comb, acc.w * comb);
+  uint32_t v = max(__float_as_uint(acc.x) & 0x7fffffffu, __float_as_uint(acc.y) & 0x7fffffffu);
+  if (PAIR) {
+    v = max(v, max(__float_as_uint(acc.z) & 0x7fffffffu, __float_as_uint(acc.w) & 0x7fffffffu));
+    *reinterpret_cast<float4 *>(ws + S.out_off + ((int64_t)j * Bp + 2 * (int64_t)pr) * 8) = acc;
+  } else {
+    *reinterpret_cast<float2 *>(ws + S.out_off + (int64_t)j * 8) = make_float2(acc.x, acc.y);
+  }
+  return v;
+}
+
+// An input's maximum and exponent (lane i of every warp: input i), read while
+// the operands are: its power-of-two scale, 2^-e, is only needed for the sum.
+struct ProgMeta {
+  uint32_t bits;
+  int exp;
+};
+
+__device__ __forceinline__ int prog_scale_exp(uint32_t bits) {
+  const int E = (int)((bits >> 23) & 0xff);
+  return E == 0xff || E == 0 ? 0 : (E - 126 > 126 ? 126 : E - 126);
+}
+
+// The factor on the sum: 2^-(e_1 + .. + e_m) gives the same values as scaling
+// every input (powers of two) while no product of unscaled inputs leaves
+// FP32's range; 0 where that is not sure (exponents above 60 in all).
+__device__ __forceinline__ float prog_comb(ProgMeta q) {
+  const int e = prog_scale_exp(q.bits);
+  const int es = __reduce_add_sync(0xffffffffu, e), big = __reduce_add_sync(0xffffffffu, e < 0 ? -e : e);
+  return big <= 60 ? __int_as_float((127 - es) << 23) : 0.f;
+}
+
+// Items [i0, i1) of a step of M inputs, U terms in flight per thread.  PAIR:
+// an item is two batch entries of a row (else a row).  Returns ~0u, with
+// nothing stored, when the sum cannot be scaled (prog_comb).
+template <int M, int U, bool PAIR>
+__device__ __forceinline__ uint32_t prog_items(const PStep &S, char *ws, const int *eoff, ProgMeta meta, int i0, int i1,
+                                               int Bp) {
+  float comb = 0.f;
+  const int tid = threadIdx.x, lg = S.lg, per = PROG_THREADS >> lg, g = tid & ((1 << lg) - 1);
+  const int K = 1 << S.k, Kt = K < 256 ? K : 256;
+  uint32_t lmax = 0;
+#pragma unroll 1
+  for (int b = i0; b < i1; b += per) {
+    const bool live = b + (tid >> lg) < i1;
+    uint32_t j, pr;
+    prog_place<PAIR>(S, live ? b + (tid >> lg) : i1 - 1, &j, &pr);
+    const char *a[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      const PIn &in = S.in[i];
+      const int64_t r = run_index(in.run, in.nrow, j);
+      a[i] = ws + in.off + (PAIR && in.batched ? r * Bp * 8 + (int)pr * 16 : r * 8);
+    }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int e0 = 0; e0 < K; e0 += 256) {
+      if (e0) {
+        // the table covers the 8 low summed bits: move on to the next block
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+          const PIn &in = S.in[i];
+          const int64_t r = run_index(in.run + in.nrow, in.nterm, e0) - run_index(in.run + in.nrow, in.nterm, e0 - 256);
+          a[i] += PAIR && in.batched ? r * Bp * 8 : r * 8;
+        }
+      }
+#pragma unroll 1
+      for (int e = g; e < Kt; e += U << lg) {
+        float4 v[U][M];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int i = 0; i < M; ++i) v[u][i] = prog_load(a[i] + eoff[i * 256 + e + (u << lg)], S.in[i].batched, PAIR);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float2 p0 = make_float2(v[u][0].x, v[u][0].y), p1 = make_float2(v[u][0].z, v[u][0].w);
+#pragma unroll
+          for (int i = 1; i < M; ++i) {
+            p0 = cmul(p0, make_float2(v[u][i].x, v[u][i].y));
+            if (PAIR) p1 = cmul(p1, make_float2(v[u][i].z, v[u][i].w));
+          }
+          acc.x += p0.x;
+          acc.y += p0.y;
+          if (PAIR) {
+            acc.z += p1.x;
+            acc.w += p1.y;
+          }
+        }
+      }
+    }
+    if (b == i0) {
+      comb = prog_comb(meta);
+      if (comb == 0.f) return ~0u;
+    }
+    lmax = max(lmax, prog_store<PAIR>(S, ws, acc, comb, live, j, pr, Bp));
+  }
+  return lmax;
+}
+
+// The same where the sum cannot be scaled: any number of inputs, one term at a
+// time, each value scaled as it is loaded.
+template <bool PAIR>
+__device__ __noinline__ uint32_t prog_items_any(const PStep &S, char *ws, const int *eoff, ProgMeta meta, int i0,
+                                                int i1, int Bp) {
+  const int e_in = prog_scale_exp(meta.bits);
+  float scale[MAXIN];
+#pragma unroll
+  for (int i = 0; i < MAXIN; ++i) scale[i] = __int_as_float((127 - __shfl_sync(0xffffffffu, e_in, i)) << 23);
+  const int tid = threadIdx.x, lg = S.lg, per = PROG_THREADS >> lg, g = tid & ((1 << lg) - 1);
+  const int K = 1 << S.k;
+  uint32_t lmax = 0;
+#pragma unroll 1
+  for (int b = i0; b < i1; b += per) {
+    const bool live = b + (tid >> lg) < i1;
+    uint32_t j, pr;
+    prog_place<PAIR>(S, live ? b + (tid >> lg) : i1 - 1, &j, &pr);
+    int a[MAXIN];  // byte offsets in the inputs (each below 2 GiB)
+#pragma unroll
+    for (int i = 0; i < MAXIN; ++i)
+      a[i] = i < S.m ? run_index(S.in[i].run, S.in[i].nrow, j) * (PAIR && S.in[i].batched ? Bp * 8 : 8) +
+                           (PAIR && S.in[i].batched ? (int)pr * 16 : 0)
+                     : 0;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int e = g; e < K; e += 1 << lg) {
+      float2 p0 = make_float2(1.f, 0.f), p1 = p0;
+#pragma unroll
+      for (int i = 0; i < MAXIN; ++i)
+        if (i < S.m) {
+          const PIn &in = S.in[i];
+          int o = a[i] + eoff[i * 256 + (e & 255)];
+          if (e >> 8) o += run_index(in.run + in.nrow, in.nterm, e & ~255) * (PAIR && in.batched ? Bp * 8 : 8);
+          const float4 v = prog_load(ws + in.off + o, in.batched, PAIR);
+          p0 = cmul(p0, make_float2(v.x * scale[i], v.y * scale[i]));
+          if (PAIR) p1 = cmul(p1, make_float2(v.z * scale[i], v.w * scale[i]));
+        }
+      acc.x += p0.x;
+      acc.y += p0.y;
+      acc.z += p1.x;
+      acc.w += p1.y;
+    }
+    lmax = max(lmax, prog_store<PAIR>(S, ws, acc, 1.f, live, j, pr, Bp));
+  }
+  return lmax;
+}
+
+template <int M, bool PAIR>
+__device__ __forceinline__ uint32_t prog_items_u(const PStep &S, char *ws, const int *eoff, ProgMeta meta, int i0, int i1,
+                                                 int Bp) {
+  const int tpt = S.k - S.lg;  // log2 of the terms per lane
+  if (tpt >= 2) return prog_items<M, M == 4 ? 2 : 4, PAIR>(S, ws, eoff, meta, i0, i1, Bp);
+  if (tpt == 1) return prog_items<M, 2, PAIR>(S, ws, eoff, meta, i0, i1, Bp);
+  return prog_items<M, 1, PAIR>(S, ws, eoff, meta, i0, i1, Bp);
+}
+
+__global__ void __launch_bounds__(PROG_THREADS, 2)
+    k_program(char *ws, const PStep *steps, const PTask *tasks, int n_tasks, int *sync, int ticket, int done0, Header *hdr,
+              int Bp) {
+  __shared__ PStep desc[2];
+  __shared__ int eoff[MAXIN * 256];
+  __shared__ uint32_t red[PROG_THREADS / 32];
+  __shared__ int s_task;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  volatile Meta *vm = meta;
-  for (int si = first; si < first + count; ++si) {
-    const StepDesc &d = descs[si];
-    build_tables(d, 8, 0, 1, rowtab, etab, tid, 256);
-    float scale[MAXIN];
-    int esum = 0;
-    int64_t rowb[MAXIN];
+  constexpr int WORDS = sizeof(PStep) / 4;
+  static_assert(sizeof(PStep) % 8 == 0 && WORDS <= 2 * PROG_THREADS, "descriptor copy");
+  for (;;) {
+    if (tid == 0) s_task = atomicAdd(sync + ticket, 1);
+    __syncthreads();
+    const int t = s_task;
+    if (t >= n_tasks) return;
+    const PTask task = tasks[t];
+    for (int w = tid; w < WORDS; w += PROG_THREADS)
+      reinterpret_cast<int *>(&desc[0])[w] = reinterpret_cast<const int *>(steps + task.step)[w];
+    for (int c = 0; c < task.count; ++c) {
+      __syncthreads();  // the descriptor is in; the previous step's outputs and maximum are visible
+      const PStep &S = desc[c & 1];
+      const int m = S.m, k = S.k;
+      // the chain's next descriptor, stored once this one's work is issued
+      int nd[2] = {0, 0};
+      const bool more = c + 1 < task.count;
+      if (more) {
+        const int *src = reinterpret_cast<const int *>(steps + task.step + c + 1);
 #pragma unroll
-    for (int i = 0; i < MAXIN; ++i) {
-      scale[i] = 1.f;
-      rowb[i] = 0;
-      if (i < d.m) {
-        const InDesc &in = d.in[i];
-        int e = 0;
-        if (in.meta >= 0) {
-          const uint32_t bits = vm[in.meta].maxbits;
-          const int E = (int)((bits >> 23) & 0xff);
-          if (E == 0xff) {
-            if (hdr && tid == 0) atomicCAS(&hdr->status, 0, QGM_ERR_NONFINITE);
-          } else if (E != 0) {
-            e = E - 126 > 126 ? 126 : E - 126;
-            scale[i] = __int_as_float((127 - e) << 23);
-          }
-          esum += e + vm[in.meta].exp;
+        for (int q = 0; q < 2; ++q)
+          if (tid + q * PROG_THREADS < WORDS) nd[q] = src[tid + q * PROG_THREADS];
+      }
+      bool ok = true;
+      if (wid == 0) {
+        if (lane < S.n_deps) ok = prog_wait(sync + done0 + S.dep[lane], S.dep_units[lane], sync);
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      const int Kt = k < 8 ? 1 << k : 256;
+      for (int i = 0; i < m; ++i) {
+        const PIn &in = S.in[i];
+        const int unit = in.batched ? Bp * 8 : 8;
+        for (int e = tid; e < Kt; e += PROG_THREADS) eoff[i * 256 + e] = run_index(in.run + in.nrow, in.nterm, e) * unit;
+      }
+      if (!__syncthreads_and(ok)) {
+        if (tid == 0) {
+          atomicExch(sync, 1);
+          atomicCAS(&hdr->status, 0, QGM_ERR_TIMEOUT);
         }
-        int64_t ri = 0;
-        for (int b = 0; b < 8 && b < d.w_out; ++b)
-          if ((tid >> b) & 1) ri += run_bit(in, b);
-        rowb[i] = in.off + ri * 8;
+        return;
+      }
+      const int i0 = task.unit * S.unit_items;
+      const int i1 = i0 + S.unit_items < S.items ? i0 + S.unit_items : S.items;
+      ProgMeta meta{0u, 0};
+      if (lane < m && S.in[lane].meta >= 0) {
+        meta.bits = __ldcg(reinterpret_cast<const uint32_t *>(ws + S.in[lane].meta));
+        meta.exp = __ldcg(reinterpret_cast<const int *>(ws + S.in[lane].meta) + 1);
+      }
+      uint32_t lmax = ~0u;
+      if (S.batched) {
+        switch (m) {
+          case 1: lmax = prog_items_u<1, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 2: lmax = prog_items_u<2, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 3: lmax = prog_items_u<3, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 4: lmax = prog_items_u<4, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 5: lmax = prog_items<5, 1, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 6: lmax = prog_items<6, 1, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 7: lmax = prog_items<7, 1, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+          default: lmax = prog_items<8, 1, true>(S, ws, eoff, meta, i0, i1, Bp); break;
+        }
+        if (lmax == ~0u) lmax = prog_items_any<true>(S, ws, eoff, meta, i0, i1, Bp);
+      } else {
+        switch (m) {
+          case 1: lmax = prog_items_u<1, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 2: lmax = prog_items_u<2, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 3: lmax = prog_items_u<3, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 4: lmax = prog_items_u<4, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 5: lmax = prog_items<5, 1, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 6: lmax = prog_items<6, 1, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          case 7: lmax = prog_items<7, 1, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+          default: lmax = prog_items<8, 1, false>(S, ws, eoff, meta, i0, i1, Bp); break;
+        }
+        if (lmax == ~0u) lmax = prog_items_any<false>(S, ws, eoff, meta, i0, i1, Bp);
+      }
+      if (wid == 0 && task.unit == 0) {
+        // the output's exponent; a non-finite input raises the status
+        if (((meta.bits >> 23) & 0xff) == 0xff) atomicCAS(&hdr->status, 0, QGM_ERR_NONFINITE);
+        const int ex = __reduce_add_sync(0xffffffffu, prog_scale_exp(meta.bits) + meta.exp);
+        if (lane == 0) *(reinterpret_cast<int *>(ws + S.out_meta) + 1) = ex;
+      }
+      lmax = __reduce_max_sync(0xffffffffu, lmax);
+      if (lane == 0) red[wid] = lmax;
+      if (more) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          if (tid + q * PROG_THREADS < WORDS) reinterpret_cast<int *>(&desc[(c + 1) & 1])[tid + q * PROG_THREADS] = nd[q];
+      }
+      __syncthreads();  // every output of the unit is stored
+      if (tid == 0) {
+        uint32_t v = red[0];
+#pragma unroll
+        for (int w = 1; w < PROG_THREADS / 32; ++w) v = max(v, red[w]);
+        if (v) atomicMax(reinterpret_cast<uint32_t *>(ws + S.out_meta), v);
+        if (S.signal) {
+          __threadfence();
+          atomicAdd(sync + done0 + (task.step + c), 1);
+        }
       }
     }
-    if (tid == 0) vm[d.out_meta].exp = esum;
-    __syncthreads();
-    const uint64_t rows = 1ull << d.w_out;
-    const int tcount = 1 << d.k;
-    float lmax = 0.f;
-    float2 *out = reinterpret_cast<float2 *>(ws + d.out_off);
-    uint64_t it = 0;
-    for (uint64_t j = tid; j < rows; j += 256, ++it) {
-      if (it) {
-        const int t = __ffsll((long long)it) - 1;
-#pragma unroll
-        for (int i = 0; i < MAXIN; ++i)
-          if (i < d.m) rowb[i] += rowtab[i][t];
-      }
-      float2 a = make_float2(0.f, 0.f);
-      int64_t eb[MAXIN];
-#pragma unroll
-      for (int i = 0; i < MAXIN; ++i) eb[i] = 0;
-      for (int jt = 0; jt < tcount; ++jt) {
-        if (jt) {
-          const int t = __ffs(jt) - 1;
-#pragma unroll
-          for (int i = 0; i < MAXIN; ++i)
-            if (i < d.m) eb[i] += etab[i][t];
-        }
-        float2 pr = make_float2(1.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < MAXIN; ++i) {
-          if (i < d.m) {
-            const float2 v = *reinterpret_cast<const float2 *>(ws + rowb[i] + eb[i]);
-            pr = cmul(pr, make_float2(v.x * scale[i], v.y * scale[i]));
-          }
-        }
-        a.x += pr.x;
-        a.y += pr.y;
-      }
-      out[j] = a;
-      lmax = fmax_nan(lmax, absmax2(a));
-    }
-    for (int o = 16; o > 0; o >>= 1) lmax = fmax_nan(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-    if (lane == 0) red[wid] = lmax;
-    __syncthreads();
-    if (tid == 0) {
-      float v = red[0];
-      for (int w = 1; w < 8; ++w) v = fmax_nan(v, red[w]);
-      if (v > 0.f || v != v) vm[d.out_meta].maxbits = __float_as_uint(v);
-    }
-    __syncthreads();
+    __syncthreads();  // s_task and the descriptors are free again
   }
 }
 
@@ -907,12 +1170,6 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ uint64_t gtimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
 }
 
 // Wait (about one second at most) for the completion of the mbarrier phase
@@ -2211,13 +2468,14 @@ extern "C" void qgm_exec_release(qgm_plan *p) {
   p->exec = nullptr;
 }
 
-static void launch_leaves(qgm_plan *p, const uint64_t *d_bits, int64_t B, cudaStream_t st) {
+static void launch_leaves(qgm_plan *p, const uint64_t *d_bits, int64_t B, cudaStream_t st, const Program *P = nullptr) {
   char *ws = p->exec->ws;
   const int nl = (int)p->leafdesc.size();
   k_build_leaves<<<std::max(nl, 1), 256, 0, st>>>(
       ws, reinterpret_cast<const LeafDesc *>(ws + p->off_leafdesc), nl,
       reinterpret_cast<Meta *>(ws + p->off_meta), p->n_meta,
-      reinterpret_cast<Header *>(ws + p->off_header), d_bits, B, p->Bp);
+      reinterpret_cast<Header *>(ws + p->off_header), d_bits, B, p->Bp,
+      P ? reinterpret_cast<int32_t *>(ws + P->off_sync) : nullptr, P ? (int)P->sync_words() : 0);
 }
 
 // Grid of one product-sum step: row strides are powers of two so that the
@@ -2505,6 +2763,7 @@ static int autotune(qgm_plan *p, cudaStream_t st) {
   for (size_t si = 0; si < p->steps.size(); ++si) {
     const StepDesc &d = p->steps[si];
     StepTune &tn = p->tune[si];
+    if (!program_alone(d, p->Bp)) continue;  // runs in the step program
     std::vector<StepTune> cand;
     if (d.gemm >= 0 && p->gemm_tc && tc_config(p->gemms[d.gemm], p->Bp, p->tc_planes).ok) {
       const TcCfg tcc = tc_config(p->gemms[d.gemm], p->Bp, p->tc_planes);
@@ -2569,37 +2828,43 @@ static int autotune(qgm_plan *p, cudaStream_t st) {
   return QGM_OK;
 }
 
-static void launch_accumulate(qgm_plan *p, double2 *d_out, int64_t n_out, cudaStream_t st) {
+static void launch_accumulate(qgm_plan *p, double2 *d_out, int64_t n_out, int64_t final_off, cudaStream_t st) {
   char *ws = p->exec->ws;
   const int64_t blocks = std::min<int64_t>((n_out + 255) / 256, (int64_t)p->exec->sms * 8);
   // the fixed-gate tables had 2^{-1/2} pulled out half_pow_total times
   const cd c = p->constant * std::pow(2.0, -0.5 * p->half_pow_total);
   k_accumulate<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, st>>>(
-      ws, p->final_off, p->final_meta, p->final_batched,
+      ws, final_off, p->final_meta, p->final_batched,
       p->output_mode == QGM_OUT_OPEN ? 1 : (p->open_in_batch ? 2 : 0), n_out, d_out,
       reinterpret_cast<const Meta *>(ws + p->off_meta), reinterpret_cast<Header *>(ws + p->off_header), c.real(),
       c.imag(), p->open_in_batch, p->Bp);
 }
 
+// Enqueue a step program: its segments, and its large steps on their own (with
+// the tuner's parameters for the forward pass).
+static void launch_program(qgm_plan *p, const Program &P, cudaStream_t st) {
+  char *ws = p->exec->ws;
+  Meta *meta = reinterpret_cast<Meta *>(ws + p->off_meta);
+  Header *hdr = reinterpret_cast<Header *>(ws + p->off_header);
+  int ticket = 1;  // sync word 0 is the abort word
+  for (const ProgramOp &op : P.ops) {
+    if (op.big >= 0) {
+      launch_step_ws(ws, p->exec->sms, p->Bp, P.all[op.big], P.gemms.data(), meta, hdr, st, p->gemm_tc, p->off_planes,
+                     p->tc_planes, nullptr, &P == &p->fprog ? &p->tune[op.big] : nullptr);
+    } else {
+      k_program<<<std::min(op.tasks, 2 * p->exec->sms), PROG_THREADS, 0, st>>>(
+          ws, reinterpret_cast<const PStep *>(ws + P.off_steps), reinterpret_cast<const PTask *>(ws + P.off_tasks) + op.task0,
+          op.tasks, reinterpret_cast<int *>(ws + P.off_sync), ticket++, (int)P.done_word(), hdr, p->Bp);
+    }
+  }
+}
+
 // Enqueue one slice: leaves, steps, accumulation.
 static int enqueue_slice(qgm_plan *p, const uint64_t *d_bits, int64_t B, double2 *d_out,
                          int64_t n_out, cudaStream_t st) {
-  launch_leaves(p, d_bits, B, st);
-  char *ws = p->exec->ws;
-  for (size_t s = 0; s < p->steps.size();) {
-    const int32_t g = s < p->plain_group.size() ? p->plain_group[s] : 0;
-    if (g >= 2) {
-      // a run of small batch-free steps: one launch of one CTA
-      k_step_plain_group<<<1, 256, 0, st>>>(ws, reinterpret_cast<const StepDesc *>(ws + p->off_sdesc), (int)s, g,
-                                            reinterpret_cast<Meta *>(ws + p->off_meta),
-                                            reinterpret_cast<Header *>(ws + p->off_header));
-      s += (size_t)g;
-    } else {
-      launch_step(p, p->steps[s], st);
-      ++s;
-    }
-  }
-  launch_accumulate(p, d_out, n_out, st);
+  launch_leaves(p, d_bits, B, st, &p->fprog);
+  launch_program(p, p->fprog, st);
+  launch_accumulate(p, d_out, n_out, p->f_final_off, st);
   return QGM_OK;
 }
 
@@ -2786,9 +3051,11 @@ int qgm_plan_bind(qgm_plan *p, void *d_workspace, size_t ws_bytes, void *stream)
   if (!p->leafdesc.empty())
     CK(cudaMemcpyAsync(x->ws + p->off_leafdesc, p->leafdesc.data(), p->leafdesc.size() * sizeof(LeafDesc),
                        cudaMemcpyHostToDevice, st));
-  if (!p->steps.empty())
-    CK(cudaMemcpyAsync(x->ws + p->off_sdesc, p->steps.data(), p->steps.size() * sizeof(StepDesc),
-                       cudaMemcpyHostToDevice, st));
+  for (const Program *P : {&p->fprog, &p->gprog}) {
+    if (P->tasks.empty()) continue;
+    CK(cudaMemcpyAsync(x->ws + P->off_steps, P->steps.data(), P->steps.size() * sizeof(PStep), cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(x->ws + P->off_tasks, P->tasks.data(), P->tasks.size() * sizeof(PTask), cudaMemcpyHostToDevice, st));
+  }
   if (p->grad && !p->gparams.empty())
     CK(cudaMemcpyAsync(x->ws + p->off_gparams, p->gparams.data(), p->gparams.size() * sizeof(GradParam),
                        cudaMemcpyHostToDevice, st));
@@ -3093,26 +3360,20 @@ int qgm_amplitudes_report(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, 
   rep->bytes = p->sim.bytes * (double)rep->slices;
   rep->flops = p->sim.flops * (double)rep->slices;
   if (x->kind == QGM_EXEC_STEPWISE) {
-    // per slice: leaves, accumulation, and per step one launch (a run of
-    // small batch-free steps: one for the run), a tensor-core step adding
-    // its split passes (one when its streamed operand is converted in the
-    // product kernel, else two)
+    // per slice: leaves, accumulation, a launch per segment of the step
+    // program and per large step, a tensor-core step adding its split passes
+    // (one when its streamed operand is converted in the product kernel,
+    // else two)
     int64_t per = 2;
-    for (size_t si = 0; si < p->steps.size();) {
-      const int32_t g = si < p->plain_group.size() ? p->plain_group[si] : 0;
-      if (g >= 2) {
-        per += 1;
-        si += (size_t)g;
-        continue;
-      }
-      const StepDesc &d = p->steps[si];
-      const StepTune *tn = si < p->tune.size() ? &p->tune[si] : nullptr;
+    for (const ProgramOp &op : p->fprog.ops) {
       per += 1;
-      if (d.gemm >= 0 && p->gemm_tc && !(tn && tn->ps)) {
-        const TcCfg c = tc_config(p->gemms[d.gemm], p->Bp, p->tc_planes, tn && tn->nt_cap ? tn->nt_cap : 256);
-        if (c.ok) per += tn && tn->conv && c.fold ? 1 : 2;
+      if (op.big < 0) continue;
+      const StepDesc &d = p->fprog.all[op.big];
+      const StepTune &tn = p->tune[op.big];
+      if (d.gemm >= 0 && p->gemm_tc && !tn.ps) {
+        const TcCfg c = tc_config(p->gemms[d.gemm], p->Bp, p->tc_planes, tn.nt_cap ? tn.nt_cap : 256);
+        if (c.ok) per += tn.conv && c.fold ? 1 : 2;
       }
-      ++si;
     }
     rep->launches = per * rep->slices + 1;
   } else {
@@ -3163,7 +3424,7 @@ int qgm_plan_profile(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, doubl
     launch_step(p, p->steps[s], st);
     CK(cudaEventRecord(ev[2 + s], st));
   }
-  launch_accumulate(p, reinterpret_cast<double2 *>(d_out), B << p->open_in_batch, st);
+  launch_accumulate(p, reinterpret_cast<double2 *>(d_out), B << p->open_in_batch, p->final_off, st);
   CK(cudaEventRecord(ev[n], st));
   CK(cudaGetLastError());
   CK(cudaEventSynchronize(ev[n]));
@@ -3206,7 +3467,7 @@ int qgm_plan_profile_gemm(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, 
     CK(cudaEventRecord(e[2], st));
     for (auto &x : e) ev.push_back(x);
   }
-  launch_accumulate(p, reinterpret_cast<double2 *>(d_out), B << p->open_in_batch, st);
+  launch_accumulate(p, reinterpret_cast<double2 *>(d_out), B << p->open_in_batch, p->final_off, st);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
   for (size_t c = 0; c < ev.size() / 3; ++c) {
@@ -3453,13 +3714,13 @@ static void enqueue_grad(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, c
   // pass of that slice; the per-gate reduction adds each slice's share
   const int64_t nslices = (int64_t)1 << p->slice_vars.size();
   for (int64_t s = 0; s < nslices; ++s) {
-    launch_leaves(p, d_bitstrings, B, st);
-    for (const StepDesc &d : p->gfwd) launch_step(p, d, st);
-    k_accumulate<<<(unsigned)std::max<int64_t>(iblocks, 1), 256, 0, st>>>(
-        ws, p->g_final_off, p->g_final_meta, 1, 0, B, amp, meta, hdr, c.real(), c.imag(), 0, p->Bp);
+    launch_leaves(p, d_bitstrings, B, st, &p->gprog);
     k_seed<<<(p->Bp + 255) / 256, 256, 0, st>>>(reinterpret_cast<float2 *>(ws + p->g_seed_off), p->Bp, meta,
                                                  p->g_seed_meta);
-    for (const StepDesc &d : p->gbwd) launch_step(p, d, st);
+    // the adjoint steps of a tensor run beside forward steps of others
+    launch_program(p, p->gprog, st);
+    k_accumulate<<<(unsigned)std::max<int64_t>(iblocks, 1), 256, 0, st>>>(
+        ws, p->g_final_off, p->g_final_meta, 1, 0, B, amp, meta, hdr, c.real(), c.imag(), 0, p->Bp);
     if (n_gates > 0)
       k_grad_reduce<<<2 * n_gates, 256, 0, st>>>(ws, reinterpret_cast<const GradParam *>(ws + p->off_gparams),
                                                  d_bitstrings, B, p->Bp,
@@ -3518,7 +3779,7 @@ void static_slice(const qgm_plan *p, char *ws, int sms, const uint64_t *d_bits, 
   Header *hdr = reinterpret_cast<Header *>(ws + p->off_header);
   const int nl = (int)p->leafdesc.size();
   k_build_leaves<<<std::max(nl, 1), 256, 0, st>>>(ws, reinterpret_cast<const LeafDesc *>(ws + p->off_leafdesc),
-                                                   nl, meta, p->n_meta, hdr, d_bits, B, p->Bp);
+                                                   nl, meta, p->n_meta, hdr, d_bits, B, p->Bp, nullptr, 0);
   for (const StepDesc &d : p->steps) launch_step_ws(ws, sms, p->Bp, d, p->gemms.data(), meta, hdr, st);
   const int64_t blocks = std::min<int64_t>((B + 255) / 256, (int64_t)sms * 8);
   const cd c = p->constant * std::pow(2.0, -0.5 * p->half_pow_total);

@@ -1298,6 +1298,87 @@ int plan_set_params(qgm_plan *p, const double *params) {
   return QGM_OK;
 }
 
+// The forward pass as a step program.  Small steps run in any order their
+// inputs allow, so their outputs leave the arena (whose reuse of memory
+// assumes the plan's order) for a region of their own, where a block is only
+// reused along a tensor's descent: what step s frees goes to the one step
+// that reads s's output, which cannot start before s is done.
+static void forward_program(qgm_plan *p) {
+  const SimResult &S = p->sim;
+  const int n = (int)p->steps.size();
+  Program &P = p->fprog;
+  P.all = p->steps;
+  P.gemms = p->gemms;
+  P.prod.assign(n, {});
+  std::vector<int> producer(S.tensors.size(), -1);
+  for (int s = 0; s < n; ++s) producer[S.steps[s].out] = s;
+  using Block = std::pair<int64_t, int64_t>;  // size, offset
+  std::vector<std::vector<Block>> pool(n);
+  std::vector<int64_t> off(S.tensors.size());
+  std::vector<char> moved(S.tensors.size(), 0);
+  for (size_t t = 0; t < S.tensors.size(); ++t) off[t] = S.tensors[t].off;
+  int64_t top = p->ws_bytes - 256;
+  for (int s = 0; s < n; ++s) {
+    const StepRec &st = S.steps[s];
+    StepDesc &d = P.all[s];
+    for (size_t i = 0; i < st.inputs.size(); ++i) {
+      const int q = producer[st.inputs[i]];
+      P.prod[s].push_back(q);
+      d.in[i].off = off[st.inputs[i]];
+      if (q >= 0) {
+        pool[s].insert(pool[s].end(), pool[q].begin(), pool[q].end());
+        pool[q].clear();
+      }
+    }
+    if (!program_alone(d, p->Bp)) {
+      const int64_t bytes = (S.tensors[st.out].entries * 8 + 255) & ~int64_t(255);
+      int best = -1;
+      for (int b = 0; b < (int)pool[s].size(); ++b)
+        if (pool[s][b].first >= bytes && (best < 0 || pool[s][b].first < pool[s][best].first)) best = b;
+      if (best >= 0) {
+        off[st.out] = pool[s][best].second;
+        pool[s][best].first -= bytes;
+        pool[s][best].second += bytes;
+      } else {
+        off[st.out] = top;
+        top += bytes;
+      }
+      moved[st.out] = 1;
+      d.out_off = off[st.out];
+    }
+    for (int id : st.inputs)
+      if (moved[id]) pool[s].push_back({(S.tensors[id].entries * 8 + 255) & ~int64_t(255), off[id]});
+    if (d.gemm >= 0) {
+      GemmDesc &g = P.gemms[d.gemm];
+      g.a_off = off[st.inputs[0]];
+      g.b_off = off[st.inputs[1]];
+    }
+  }
+  p->f_final_off = off[S.final_tensor];
+  build_program(P, p->Bp, p->off_meta, std::vector<char>(n, 0));
+  p->ws_bytes = place_program(P, top) + 256;
+}
+
+// The gradient pass (forward keeping every intermediate, then the adjoint
+// steps) as a step program: no memory is reused, so a tensor's producer is
+// found by its offset.
+static void gradient_program(qgm_plan *p) {
+  Program &P = p->gprog;
+  P.all = p->gfwd;
+  P.all.insert(P.all.end(), p->gbwd.begin(), p->gbwd.end());
+  P.prod.assign(P.all.size(), {});
+  std::map<int64_t, int> producer;
+  for (size_t s = 0; s < P.all.size(); ++s) {
+    for (int i = 0; i < P.all[s].m; ++i) {
+      auto it = producer.find(P.all[s].in[i].off);
+      P.prod[s].push_back(it == producer.end() ? -1 : it->second);
+    }
+    producer[P.all[s].out_off] = (int)s;
+  }
+  build_program(P, p->Bp, p->off_meta, std::vector<char>(P.all.size(), 0));
+  p->ws_bytes = place_program(P, p->ws_bytes - 256) + 256;
+}
+
 int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
   p->model = m;
   p->opts = o;
@@ -1614,7 +1695,6 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
                          (int64_t)(p->leaves.size() + 1) * sizeof(RLeaf) + (njobs + 1) * sizeof(RJob) +
                          ((int64_t)S.steps.size() * RES_WARPS + RES_WARPS + 8) * 4);
   }
-  p->off_sdesc = take((int64_t)(S.steps.size() + 1) * (int64_t)sizeof(StepDesc));
   p->off_arena = take(0);
   for (SymTensor &t : S.tensors)
     if (t.leaf < 0) t.off += p->off_arena;
@@ -1755,8 +1835,7 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
   }
   p->tune.assign(p->steps.size(), StepTune{});
   // runs of at least two consecutive small batch-free product-sum steps (at
-  // most 2^12 outputs and 2^16 products each): a launch of their own would
-  // cost more than the work
+  // most 2^12 outputs and 2^16 products each), as step reports list them
   p->plain_group.assign(p->steps.size(), 0);
   for (size_t s0 = 0; s0 < p->steps.size();) {
     auto small = [&](size_t s) {
@@ -1778,6 +1857,7 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
     }
   p->off_planes = p->ws_bytes - 256;
   p->ws_bytes = p->off_planes + p->planes_bytes + 256;
+  forward_program(p);
   build_resident(p);
   if (p->grad) {
     // ------------------------------------------- adjoint elimination layout
@@ -1898,6 +1978,7 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
     p->off_gparams = gtake((int64_t)std::max<size_t>(p->gparams.size(), 1) * sizeof(GradParam));
     p->n_meta = next_meta;
     p->ws_bytes = goff + 256;
+    gradient_program(p);
   }
   if (o.executor < 0 || o.executor > 3) {
     set_error("qgm_plan_order: bad executor %d", o.executor);
@@ -2301,7 +2382,7 @@ int qgm_plan_get_step_kernels(const qgm_plan *p, int32_t *kind, int64_t cap) {
     const StepDesc &d = p->steps[s];
     kind[s] = d.gemm >= 0 ? 3 : (d.tile_t > 0 ? 2 : (d.batched_out ? 1 : 0));
   }
-  // steps inside a run of small batch-free steps share one single-CTA launch
+  // steps inside a run of small batch-free steps
   for (size_t s = 0; s < p->plain_group.size(); ++s)
     for (int32_t j = 0; j < p->plain_group[s] && (int64_t)(s + j) < cap; ++j) kind[s + j] = 4;
   return QGM_OK;

@@ -187,6 +187,66 @@ inline bool gemm_tc_eligible(const GemmDesc &g, int Bp) { return tc_config(g, Bp
 // not used.
 inline bool gemm_fp32_ok(const GemmDesc &g) { return g.nk >= 4 && g.nm >= 6 && g.nn >= 5; }
 
+// ------------------------------------------------------------- step program
+// Most steps of a plan are small: alone in a launch they cost its latency and
+// the setup of its index tables (5 to 8 us a step).  They run instead as
+// segments of a program: one launch takes all small steps between two large
+// ones, cut into units of one CTA's work, which CTAs take in the order of a
+// ticket counter; a unit waits for the units of the steps it reads (counters
+// in the workspace).  Units are numbered so that a step's producers come
+// first, so a unit only ever waits for units taken before it.
+constexpr int PMAXRUN = 2 * MAXRUN;
+
+// One input: index = the row's and the term's bits by contiguous runs, each
+// packed as source bit | length << 8 | destination bit << 16 (row runs first).
+struct PIn {
+  int64_t off;       // byte offset of the tensor in the workspace (below 2 GiB in size)
+  int64_t meta;      // byte offset of its Meta, -1 for leaves
+  int32_t batched;
+  int16_t nrow, nterm;
+  uint32_t run[PMAXRUN];
+};
+
+struct PStep {
+  int32_t m, k, w_out, batched;
+  int64_t out_off, out_meta;  // byte offsets
+  int32_t lg;                 // 2^lg lanes share an item's terms
+  int32_t items, pairs;       // items = rows x batch pairs (1 without a batch axis)
+  int32_t unit_items, n_units;
+  int32_t n_deps, signal;     // steps waited for; 1: another task waits for this one
+  int32_t dep[MAXIN], dep_units[MAXIN];
+  PIn in[MAXIN];
+};
+
+// One ticket: unit `unit` of step `step`, or (count > 1) the one-unit steps
+// step .. step + count - 1, each reading the one before it, run in turn by
+// the same CTA.
+struct PTask {
+  int32_t step, unit, count, pad_;
+};
+
+struct ProgramOp {
+  int32_t big;          // >= 0: index of a step launched on its own; -1: a segment
+  int32_t task0, tasks; // the segment's tasks
+};
+
+struct Program {
+  std::vector<StepDesc> all;     // every step, offsets as the program uses them
+  std::vector<GemmDesc> gemms;
+  std::vector<std::vector<int>> prod;  // producer step of each input (-1: a leaf or another pass's tensor)
+  std::vector<PStep> steps;
+  std::vector<PTask> tasks;
+  std::vector<ProgramOp> ops;
+  int32_t n_segments = 0, n_tmp = 0;  // segments; temporary tensors of split sums
+  int64_t tmp_bytes = 0;
+  // workspace layout: sync words (abort, a ticket per segment, a counter per
+  // step), the temporaries' Meta (both cleared with the leaves), descriptors
+  int64_t off_sync = 0, off_steps = 0, off_tasks = 0, off_tmp = 0;
+  int64_t done_word() const { return 1 + n_segments; }
+  int64_t meta_word() const { return (done_word() + (int64_t)steps.size() + 1) & ~int64_t(1); }
+  int64_t sync_words() const { return meta_word() + 2 * n_tmp; }
+};
+
 // Leaf factor built on the device per slice: base table over
 // (internal vars | slice vars | output vars), MSB first.
 struct LeafDesc {
@@ -411,11 +471,11 @@ struct qgm_plan {
   int64_t planes_bytes = 0; // its size (the largest tensor-core step's two operands)
   int64_t ws_fwd_bytes = 0; // workspace the forward pass needs without that region
   std::vector<qgm::StepTune> tune;  // per step of `steps` (autotuner choices)
-  // runs of consecutive small steps without a batch axis, run by one CTA in
-  // one launch: plain_group[s] = steps in the run starting at s (0: none);
-  // their descriptors are copied to the workspace at off_sdesc
+  // runs of consecutive small steps without a batch axis:
+  // plain_group[s] = steps in the run starting at s (0: none)
   std::vector<int32_t> plain_group;
-  int64_t off_sdesc = 0;
+  qgm::Program fprog, gprog;  // the forward and the gradient pass as step programs
+  int64_t f_final_off = 0;    // the forward program's final tensor
   // per leaf: table layout (internal | slice | output variables), offset of
   // its base table and of its derivative tables (floats), its RXY member
   std::vector<std::vector<int>> leaf_layout;
@@ -429,6 +489,13 @@ struct qgm_plan {
 namespace qgm {
 int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p);
 int plan_set_params(qgm_plan *p, const double *params);
+// Cut P.all into segments of small steps and large steps launched on their
+// own (program.cpp).  alone[s]: launch step s on its own whatever its size.
+void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char> &alone);
+// Whether a step is launched on its own by its size and form.
+bool program_alone(const StepDesc &d, int Bp);
+// Sizes of the program's workspace region, laid out from `off` on; returns its end.
+int64_t place_program(Program &P, int64_t off);
 // CUDA source of the resident kernel specialised to one layout (jit.cpp):
 // the whole pass, its batched part, or its bitstring-independent part
 enum { RES_WHOLE = 0, RES_MAIN = 1, RES_PRE = 2 };

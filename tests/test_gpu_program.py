@@ -1,0 +1,89 @@
+"""Stepwise passes run as step programs (small steps in shared launches, taken
+as units by CTAs that wait for one another's tensors) against the FP64 oracle,
+at the sizes where the cutting into units changes: one bitstring, batches that
+fill no pair or no pass of 256 lanes, long sums over few outputs (more than 8
+summed variables, split sums), several segments around large steps, slices,
+open outputs, and the adjoint pass."""
+import numpy as np
+import pytest
+
+import errmeasure
+import qgm_inputs as qi
+from oracle import statevector as sv
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5  # the parity tests' bound for complex64
+
+
+@pytest.fixture(scope="module")
+def q():
+    from paper_1712_05384_gb300 import build
+    build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1712_05384_gb300 as q
+    return q
+
+
+@pytest.mark.parametrize("rows,cols,depth,B,kw", [
+    (2, 2, 6, 1, {}), (3, 3, 8, 1, {}), (3, 3, 16, 2, {}), (3, 4, 14, 5, {"max_fuse": 16}), (3, 4, 24, 3, {"max_fuse": 16}),
+    (4, 4, 16, 37, {}), (4, 4, 24, 130, {"max_fuse": 12}), (4, 5, 20, 127, {"max_fuse": 1}), (3, 4, 30, 1000, {}),
+    (4, 5, 24, 1024, {}), (4, 5, 24, 16, {"div": 6}), (4, 5, 28, 9, {"div": 3, "precision": "fp32"})])
+def test_program_matches_state_vector(q, rows, cols, depth, B, kw):
+    kw = dict(kw)
+    c = qi.grid_circuit(rows, cols, depth, 2)
+    m = q.Model(q.Circuit.grid(rows, cols, depth, 2))
+    div = kw.pop("div", 0)
+    if div:
+        kw["mem_budget_bytes"] = q.Plan(m, batch=B, executor=q.EXEC_STEPWISE, **kw).info.arena_bytes // div
+    p = q.Plan(m, batch=B, executor=q.EXEC_STEPWISE, **kw).bind()
+    assert not div or p.info.n_slices > 1
+    bits = qi.bitstrings(c.n, B, 5)
+    ref = sv.amplitudes(c, bits)
+    for _ in range(2):  # a second pass starts from the first one's workspace
+        a = p.amplitudes_host(bits)
+        assert p.status() == 0
+        e = errmeasure.measures(a, ref, c.n)
+        assert e["rel"] < TOL and e["abs"] < TOL, e
+
+
+@pytest.mark.parametrize("B,k", [(1, 1), (5, 4), (37, 7)])
+def test_program_with_open_outputs(q, B, k):
+    c = qi.grid_circuit(3, 4, 16, 4)
+    p = q.Plan(q.Model(q.Circuit.grid(3, 4, 16, 4)), batch=B, open_mask=(1 << k) - 1).bind()
+    bits = qi.bitstrings(12, B, 1)
+    a = p.amplitudes_host(bits)
+    full = (bits & ~np.uint64((1 << k) - 1))[:, None] + np.arange(1 << k, dtype=np.uint64)[None, :]
+    ref = sv.amplitudes(c, full.reshape(-1)).reshape(B, 1 << k)
+    assert p.status() == 0 and np.max(np.abs(a - ref)) * 2.0 ** 6 < TOL
+
+
+@pytest.mark.parametrize("rows,cols,depth,B", [(3, 3, 10, 1), (3, 4, 20, 6), (4, 4, 20, 3)])
+def test_program_gradients(q, rows, cols, depth, B):
+    # the deeper plans sum more than 8 variables into a gate's adjoint
+    c = qi.grid_circuit(rows, cols, depth, 1, param=True)
+    p = q.Plan(q.Model(q.Circuit.grid(rows, cols, depth, 1, True)), batch=B, gradients=True, executor=q.EXEC_STEPWISE).bind()
+    bits = qi.bitstrings(c.n, B, 3)
+    amps = sv.amplitudes(c, bits)
+    n = 2 * len(c.param_gates)
+    g_out = torch.zeros(n, dtype=torch.float64, device="cuda")
+    # L = sum |a|^2 2^n: g_b = a_b 2^n (Wirtinger derivative to conj(a_b))
+    w = amps * 2.0 ** c.n
+    d_g = torch.from_numpy(np.ascontiguousarray(w).view(np.float64)).cuda()
+    p.amplitude_grad(torch.from_numpy(bits.astype(np.int64)).cuda(), d_g, g_out)
+    assert p.status() == 0
+    got = g_out.cpu().numpy()
+    eps, theta = 1e-5, np.array([[c.gates[g].theta, c.gates[g].phi] for g in c.param_gates])
+
+    def loss(t):
+        return 2.0 ** c.n * np.sum(np.abs(sv.amplitudes(c.with_angles(t[:, 0], t[:, 1]), bits)) ** 2)
+
+    for i in np.unique(np.linspace(0, n - 1, 9).astype(int)):
+        t = theta.copy().reshape(-1)
+        t[i] += eps
+        up = loss(t.reshape(-1, 2))
+        t[i] -= 2 * eps
+        fd = (up - loss(t.reshape(-1, 2))) / (2 * eps)
+        assert abs(got[i] - fd) <= 1e-3 * max(abs(fd), 1e-2 * np.max(np.abs(got))), i

@@ -259,8 +259,10 @@ typedef struct {
   int32_t n_tile_steps;       /* batched steps run with a register tile */
   int32_t n_nested_steps;     /* steps whose compiled form sums some variables
                                  in an inner loop over part of the inputs */
-  int32_t n_gemm_tc_steps;    /* of the GEMM steps, those run on the tensor
-                                 cores (qgm_plan_opts.gemm_precision) */
+  int32_t n_gemm_tc_steps;    /* of the GEMM steps, those with a tensor-core
+                                 form (qgm_plan_opts.gemm_precision); short
+                                 products may run on the FP32 cores all the
+                                 same, where that is faster */
 } qgm_plan_info;
 
 /* Elimination order, slicing, step list and memory layout (Sec. IV, App. A).
@@ -297,7 +299,8 @@ int qgm_plan_get_step_inputs(const qgm_plan *p, int32_t step, int32_t *rec, int6
  * folded tensor-core step converts its streamed operand inside the product
  * kernel (instead of a separate split pass), product-sum terms in flight
  * per thread (4 or 8, or 0/2 for two), 1 when a GEMM-shaped step runs with the
- * product-sum kernels instead of a GEMM kernel, and
+ * product-sum kernels (register-tiled where their form applies and neither
+ * term groups nor terms in flight are set) instead of a GEMM kernel, and
  * ms[2c], ms[2c+1] = milliseconds with the fixed rules and with the choice.
  * *n = the number of tuned steps; rec/ms may be NULL to query it. */
 int qgm_plan_get_tuning(const qgm_plan *p, int32_t *rec, float *ms, int64_t cap, int64_t *n);
@@ -317,7 +320,7 @@ int qgm_plan_set_tuning(qgm_plan *p, const int32_t *rec, int64_t n);
  * operands sharing every summed variable): for the c-th such step, c < cap,
  * rec[12c .. 12c+11] = step index, nm, nn, nk, ns (variables private to A, to
  * B, summed, shared and kept), A batched, B batched, output batched, 1 when
- * the step runs on the tensor cores, 1 when its output is stored with the
+ * the step has a tensor-core form, 1 when its output is stored with the
  * batch entry outermost, 1 when an operand is (both for tensor-core steps
  * only: a product per batch entry read by another tensor-core step), and 1
  * when the tensor-core step folds its batch entries into M, so that the

@@ -26,6 +26,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -91,6 +92,10 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 __device__ __forceinline__ float fmax_nan(float a, float b) { return (a > b || a != a) ? a : b; }
 
 __device__ __forceinline__ float absmax2(float2 a) { return fmax_nan(fabsf(a.x), fabsf(a.y)); }
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
 
 __device__ __forceinline__ uint64_t gtimer() {
   uint64_t t;
@@ -580,6 +585,368 @@ __global__ void __launch_bounds__(STEP_THREADS)
       }
     }
   }
+  record_max(lmax, meta, d.out_meta);
+}
+
+// Index from packed runs (see PIn).
+__device__ __forceinline__ int64_t run_index64(const uint32_t *run, int n, uint32_t x) {
+  int64_t r = 0;
+#pragma unroll 1
+  for (int q = 0; q < n; ++q) {
+    const uint32_t u = run[q];
+    r += (int64_t)((x >> (u & 255u)) & ((1u << ((u >> 8) & 255u)) - 1u)) << (u >> 16);
+  }
+  return r;
+}
+
+// ---------------------------------------------------------------------------
+// Large batched product-sum step of two inputs with a register tile (RegStep).
+//
+// Bound: memory (few summed entries, or one large operand).  One load per
+// input, term and output, as k_step_batched does, re-reads each value of an
+// input once for every output bit it lacks.  Here a thread forms 2^(TM + TN)
+// outputs of one batch entry from 2^TM + 2^TN loads a term, the next term's in
+// flight.  6x6 depth 25, 1000 bitstrings: 2^15 outputs from (19, 14)-variable
+// operands over 16 terms 1.55 -> 0.90 ms (4.2 GB), 2^13 from (7, 13) over 4
+// 0.091 -> 0.045.  For longer sums L2 binds (18 to 22 TFLOP/s): k_step_mm.
+template <int TM, int TN, bool SC>
+__device__ __forceinline__ float reg_items(const RegStep &d, char *ws, const int64_t *tab, const float *scale, float comb,
+                                           int Bp) {
+  constexpr int NM = 1 << TM, NN = 1 << TN;
+  const int n = 1 << d.k;
+  const int64_t *eA = tab, *eB = eA + n, *oO = eB + n;  // byte offsets: terms of A and B, tile outputs
+  const int64_t total = ((int64_t)d.nblk << (d.lb + d.wr));
+  const int64_t uA = d.in[0].batched ? (int64_t)Bp * 8 : 8, uB = d.in[1].batched ? (int64_t)Bp * 8 : 8;
+  int64_t tA[TM ? TM : 1], tB[TN ? TN : 1];
+#pragma unroll
+  for (int b = 0; b < TM; ++b) tA[b] = d.in[0].tile[b] * uA;
+#pragma unroll
+  for (int b = 0; b < TN; ++b) tB[b] = d.in[1].tile[REG_TM + b] * uB;
+  float lmax = 0.f;
+  for (int64_t idx = (int64_t)blockIdx.x * STEP_THREADS + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * STEP_THREADS) {
+    const int bl = (int)(idx & ((1 << d.lb) - 1));
+    const int64_t rest = idx >> (d.lb + d.rl);
+    const int beta0 = (int)(rest % d.nblk) * (1 << d.lb) + bl;
+    const uint32_t row = (uint32_t)((rest / d.nblk) << d.rl) | ((uint32_t)(idx >> d.lb) & ((1u << d.rl) - 1u));
+    const bool live = beta0 < Bp;
+    const int64_t b8 = live ? beta0 * 8 : 0;
+    const char *a = ws + d.in[0].off + run_index64(d.in[0].run, d.in[0].nrow, row) * uA + (d.in[0].batched ? b8 : 0);
+    const char *b = ws + d.in[1].off + run_index64(d.in[1].run, d.in[1].nrow, row) * uB + (d.in[1].batched ? b8 : 0);
+    float2 acc[NM][NN];
+#pragma unroll
+    for (int i = 0; i < NM; ++i)
+#pragma unroll
+      for (int j = 0; j < NN; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    auto load = [&](const char *pa, const char *pb, float2 (&va)[NM], float2 (&vb)[NN]) {
+#pragma unroll
+      for (int i = 0; i < NM; ++i) {
+        int64_t o = 0;
+#pragma unroll
+        for (int t = 0; t < TM; ++t) o += (i >> t) & 1 ? tA[t] : 0;
+        va[i] = __ldg(reinterpret_cast<const float2 *>(pa + o));
+        if (SC) va[i] = make_float2(va[i].x * scale[0], va[i].y * scale[0]);
+      }
+#pragma unroll
+      for (int j = 0; j < NN; ++j) {
+        int64_t o = 0;
+#pragma unroll
+        for (int t = 0; t < TN; ++t) o += (j >> t) & 1 ? tB[t] : 0;
+        vb[j] = __ldg(reinterpret_cast<const float2 *>(pb + o));
+        if (SC) vb[j] = make_float2(vb[j].x * scale[1], vb[j].y * scale[1]);
+      }
+    };
+    float2 va[NM], vb[NN];
+    load(a + eA[0], b + eB[0], va, vb);
+#pragma unroll 1
+    for (int q = 0; q < n; ++q) {
+      float2 na[NM], nb[NN];
+      if (q + 1 < n) load(a + eA[q + 1], b + eB[q + 1], na, nb);
+#pragma unroll
+      for (int i = 0; i < NM; ++i)
+#pragma unroll
+        for (int j = 0; j < NN; ++j) {
+          acc[i][j].x = fmaf(va[i].x, vb[j].x, fmaf(-va[i].y, vb[j].y, acc[i][j].x));
+          acc[i][j].y = fmaf(va[i].x, vb[j].y, fmaf(va[i].y, vb[j].x, acc[i][j].y));
+        }
+#pragma unroll
+      for (int i = 0; i < NM; ++i) va[i] = na[i];
+#pragma unroll
+      for (int j = 0; j < NN; ++j) vb[j] = nb[j];
+    }
+    if (live) {
+      char *o = ws + d.out_off + run_index64(d.orun, d.norun, row) * Bp * 8 + b8;
+#pragma unroll
+      for (int i = 0; i < NM; ++i)
+#pragma unroll
+        for (int j = 0; j < NN; ++j) {
+          const float2 v = SC ? acc[i][j] : make_float2(acc[i][j].x * comb, acc[i][j].y * comb);
+          *reinterpret_cast<float2 *>(o + oO[i * NN + j]) = v;
+          lmax = fmax_nan(lmax, absmax2(v));
+        }
+    }
+  }
+  return lmax;
+}
+
+template <int TM, int TN>
+__global__ void __launch_bounds__(STEP_THREADS, 3)
+    k_step_reg(char *ws, const __grid_constant__ RegStep d, Meta *meta, Header *hdr, int Bp) {
+  constexpr int NC = 1 << (TM + TN);
+  extern __shared__ __align__(16) int64_t tab[];
+  const int tid = threadIdx.x, n = 1 << d.k;
+  for (int x = tid; x < 2 * n; x += STEP_THREADS) {
+    const RegIn &in = d.in[x >> d.k];
+    tab[x] = run_index64(in.run + in.nrow, in.nterm, x & (n - 1)) * (in.batched ? (int64_t)Bp * 8 : 8);
+  }
+  int64_t *oO = tab + 2 * n;
+  for (int c = tid; c < NC; c += STEP_THREADS) {
+    int64_t v = 0;  // c = cm * 2^TN + cn
+    for (int b = 0; b < TM; ++b) v += (c >> (TN + b)) & 1 ? d.otile[b] : 0;
+    for (int b = 0; b < TN; ++b) v += (c >> b) & 1 ? d.otile[REG_TM + b] : 0;
+    oO[c] = v * Bp * 8;
+  }
+  float scale[2];
+  int e[2];
+  operand_scale(meta, d.in[0].meta, hdr, &scale[0], &e[0]);
+  operand_scale(meta, d.in[1].meta, hdr, &scale[1], &e[1]);
+  if (blockIdx.x == 0 && tid == 0)
+    meta[d.out_meta].exp = e[0] + e[1] + (d.in[0].meta >= 0 ? meta[d.in[0].meta].exp : 0) +
+                           (d.in[1].meta >= 0 ? meta[d.in[1].meta].exp : 0);
+  __syncthreads();
+  // one factor on each sum, as prog_comb
+  const bool one = (e[0] < 0 ? -e[0] : e[0]) + (e[1] < 0 ? -e[1] : e[1]) <= 60;
+  const float lmax = one ? reg_items<TM, TN, false>(d, ws, tab, scale, __int_as_float((127 - e[0] - e[1]) << 23), Bp)
+                         : reg_items<TM, TN, true>(d, ws, tab, scale, 1.f, Bp);
+  record_max(lmax, meta, d.out_meta);
+}
+
+// ---------------------------------------------------------------------------
+// The same step with the pair's operands staged in shared memory (MmStep).
+//
+// Bound: FP32 arithmetic.  The register tile alone (k_step_reg) waits for L2:
+// a row is re-read by every column tile.  Here a CTA copies 2^(3 + MGB) rows
+// of A and 2^(2 + NGB) of B for 2^lb batch entries, MM_KC summed entries a
+// stage, three stages ahead (cp.async, 16 bytes = two batch entries), and each
+// of its 256 threads forms 8 x 4 outputs of one entry: 12 shared-memory loads
+// for 32 complex products.  The rows of a thread lie MG (columns NG) apart,
+// so that a warp's loads are contiguous (no bank conflicts, and the same
+// values broadcast).  Further inputs (NEST) multiply the inner sum once per
+// outer term.  43 to 50 TFLOP/s of the 77 measured: 2^24 outputs x 4 entries,
+// three inputs, 256 terms 21.1 (k_step_batched) -> 4.8 ms; 64 x 32 x 16 per
+// entry, 256 shared indices, 1000 entries 6.6 (k_gemm) -> 2.2 ms.
+template <int MGB, int NGB, bool NEST, bool SC>
+__device__ __forceinline__ float mm_tiles(const MmStep &d, char *ws, char *stage, const int64_t *tab, const float *scale,
+                                          float comb, int Bp) {
+  constexpr int MG = 1 << MGB, NG = 1 << NGB, NM = 1 << MM_TM, NN = 1 << MM_TN;
+  constexpr int LA = 256 >> NGB, LN = 256 >> MGB;        // A and B values per (summed entry, thread row or column)
+  constexpr int KA = NM * LA * 8, KB = NN * LN * 8;      // bytes per summed entry
+  constexpr int STAGES = 3, SBYTES = MM_KC * (KA + KB);
+  constexpr int SLOTS = NM * LA / 2 + NN * LN / 2, NS = (SLOTS + 255) / 256;
+  const int tid = threadIdx.x, lb = d.lb, LB = 1 << lb;
+  const int n1 = 1 << d.k1, n2 = 1 << d.k2, nst = n1 * n2 / MM_KC;
+  const int64_t *mA = tab, *nB = mA + NM * MG, *mO = nB + NN * NG, *nO = mO + NM * MG, *e2 = nO + NN * NG, *e1 = e2 + 2 * n2,
+                *xt = e1 + (2 + d.nx) * n1;
+  const int beta = tid & (LB - 1), ng = (tid >> lb) & (NG - 1), mg = (tid >> (lb + NGB)) & (MG - 1),
+            r = tid >> (lb + NGB + MGB);
+  const int64_t tiles = (int64_t)d.nblk << (d.wr - d.rb);
+  const uint32_t st0 = smem_u32(stage);
+  float lmax = 0.f;
+  for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const uint32_t p0 = (uint32_t)(tile & ((1ll << d.wp) - 1));
+    const int64_t rest = tile >> d.wp;
+    const int b0 = (int)(rest % d.nblk) << lb;
+    const uint32_t row0 = ((uint32_t)(rest / d.nblk) << d.wp | p0) << d.rb;
+    // this thread's copies: slot = (row or column, its lanes' pair)
+    const char *src[NS];
+    uint32_t dst[NS];
+    int kind[NS];  // 0: none, 1: 16 bytes, 2: one value for every entry; + 4: operand B
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+      const int s = tid + 256 * q;
+      const bool isA = s < NM * LA / 2;
+      const int u = isA ? s : s - NM * LA / 2, half = isA ? LA / 2 : LN / 2;
+      const int i = u / half, l = 2 * (u % half);  // thread row (column) and first lane
+      const int bb = l & (LB - 1), g = (l >> lb) & (isA ? MG - 1 : NG - 1), rr = l >> (lb + (isA ? MGB : NGB));
+      const MmIn &in = d.in[isA ? 0 : 1];
+      const int64_t unit = in.batched ? (int64_t)Bp * 8 : 8;
+      kind[q] = s >= SLOTS || b0 + bb >= Bp ? 0 : (in.batched ? 1 : 2) + (isA ? 0 : 4);
+      src[q] = ws + in.off + run_index64(in.run, in.nrow, row0 + rr) * unit + (in.batched ? (int64_t)(b0 + bb) * 8 : 0) +
+               (s < SLOTS ? (isA ? mA[i * MG + g] : nB[i * NG + g]) : 0);
+      dst[q] = st0 + (isA ? (i * LA + l) * 8 : MM_KC * KA + (i * LN + l) * 8);
+    }
+    auto issue = [&](int s) {
+      if (s < nst) {
+        const int q1 = (s * MM_KC) >> d.k2, q2 = (s * MM_KC) & (n2 - 1);
+        const uint32_t base = (uint32_t)(s % STAGES) * SBYTES;
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+          const bool isB = kind[q] & 4;
+          const int64_t *e = e2 + (isB ? n2 : 0) + q2;
+          const char *a = src[q] + e1[(isB ? n1 : 0) + q1];
+#pragma unroll
+          for (int kk = 0; kk < MM_KC; ++kk) {
+            const uint32_t t = dst[q] + base + kk * (isB ? KB : KA);
+            if ((kind[q] & 3) == 1)
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(t), "l"(a + e[kk]) : "memory");
+            else if ((kind[q] & 3) == 2) {
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(t), "l"(a + e[kk]) : "memory");
+              asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(t + 8), "l"(a + e[kk]) : "memory");
+            }
+          }
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float2 acc[NM][NN], in[NEST ? NM : 1][NEST ? NN : 1];
+#pragma unroll
+    for (int i = 0; i < NM; ++i)
+#pragma unroll
+      for (int j = 0; j < NN; ++j) {
+        acc[i][j] = make_float2(0.f, 0.f);
+        if (NEST) in[NEST ? i : 0][NEST ? j : 0] = make_float2(0.f, 0.f);
+      }
+    const uint32_t row = row0 + r;
+    const bool live = b0 + beta < Bp;
+    const int64_t b8 = live ? (int64_t)(b0 + beta) * 8 : 0;
+#pragma unroll
+    for (int s = 0; s < STAGES - 1; ++s) issue(s);
+#pragma unroll 1
+    for (int s = 0; s < nst; ++s) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+      __syncthreads();  // stage s is in, and the one before it is consumed
+      issue(s + STAGES - 1);
+      const char *sa = stage + (s % STAGES) * SBYTES + (beta + LB * (mg + MG * r)) * 8;
+      const char *sb = stage + (s % STAGES) * SBYTES + MM_KC * KA + (beta + LB * (ng + NG * r)) * 8;
+#pragma unroll
+      for (int kk = 0; kk < MM_KC; ++kk) {
+        float2 va[NM], vb[NN];
+#pragma unroll
+        for (int i = 0; i < NM; ++i) {
+          va[i] = *reinterpret_cast<const float2 *>(sa + kk * KA + i * LA * 8);
+          if (SC) va[i] = make_float2(va[i].x * scale[0], va[i].y * scale[0]);
+        }
+#pragma unroll
+        for (int j = 0; j < NN; ++j) {
+          vb[j] = *reinterpret_cast<const float2 *>(sb + kk * KB + j * LN * 8);
+          if (SC) vb[j] = make_float2(vb[j].x * scale[1], vb[j].y * scale[1]);
+        }
+#pragma unroll
+        for (int i = 0; i < NM; ++i)
+#pragma unroll
+          for (int j = 0; j < NN; ++j) {
+            float2 &t = NEST ? in[NEST ? i : 0][NEST ? j : 0] : acc[i][j];
+            t.x = fmaf(va[i].x, vb[j].x, fmaf(-va[i].y, vb[j].y, t.x));
+            t.y = fmaf(va[i].x, vb[j].y, fmaf(va[i].y, vb[j].x, t.y));
+          }
+      }
+      if (NEST && (((s + 1) * MM_KC) & (n2 - 1)) == 0) {
+        // the outer term's further inputs, entry by entry of the tile
+        const int q1 = (s * MM_KC) >> d.k2;
+#pragma unroll
+        for (int y = 0; y < MM_MAXX; ++y)
+          if (y < d.nx) {
+            const MmIn &X = d.in[2 + y];
+            const char *x = ws + X.off + run_index64(X.run, X.nrow, row) * (X.batched ? (int64_t)Bp * 8 : 8) +
+                            (X.batched ? b8 : 0) + e1[(2 + y) * n1 + q1];
+            const int64_t *xm = xt + y * (NM * MG + NN * NG), *xn = xm + NM * MG;
+#pragma unroll
+            for (int i = 0; i < NM; ++i)
+#pragma unroll
+              for (int j = 0; j < NN; ++j) {
+                float2 v = __ldg(reinterpret_cast<const float2 *>(x + xm[i * MG + mg] + xn[j * NG + ng]));
+                if (SC) v = make_float2(v.x * scale[2 + y], v.y * scale[2 + y]);
+                float2 &t = in[NEST ? i : 0][NEST ? j : 0];
+                t = cmul(t, v);
+              }
+          }
+#pragma unroll
+        for (int i = 0; i < NM; ++i)
+#pragma unroll
+          for (int j = 0; j < NN; ++j) {
+            float2 &t = in[NEST ? i : 0][NEST ? j : 0];
+            acc[i][j].x += t.x;
+            acc[i][j].y += t.y;
+            t = make_float2(0.f, 0.f);
+          }
+      }
+    }
+    if (live) {
+      char *o = ws + d.out_off + run_index64(d.orun, d.norun, row) * Bp * 8 + b8;
+#pragma unroll
+      for (int i = 0; i < NM; ++i)
+#pragma unroll
+        for (int j = 0; j < NN; ++j) {
+          const float2 v = SC ? acc[i][j] : make_float2(acc[i][j].x * comb, acc[i][j].y * comb);
+          *reinterpret_cast<float2 *>(o + mO[i * MG + mg] + nO[j * NG + ng]) = v;
+          lmax = fmax_nan(lmax, absmax2(v));
+        }
+    }
+    __syncthreads();  // the last stage is consumed
+  }
+  return lmax;
+}
+
+__host__ __device__ constexpr int mm_stage_bytes(int mgb, int ngb) {
+  return 3 * MM_KC * ((8 << MM_TM) * (256 >> ngb) + (8 << MM_TN) * (256 >> mgb));
+}
+
+template <int MGB, int NGB, bool NEST>
+__global__ void __launch_bounds__(256, NEST ? 1 : 2)
+    k_step_mm(char *ws, const __grid_constant__ MmStep d, Meta *meta, Header *hdr, int Bp) {
+  constexpr int NMR = 1 << (MM_TM + MGB), NNR = 1 << (MM_TN + NGB);
+  extern __shared__ __align__(16) char mms[];
+  int64_t *tab = reinterpret_cast<int64_t *>(mms + mm_stage_bytes(MGB, NGB));
+  const int tid = threadIdx.x, m = 2 + d.nx;
+  const int n1 = 1 << d.k1, n2 = 1 << d.k2;
+  auto unit = [&](int i) { return d.in[i].batched ? (int64_t)Bp * 8 : (int64_t)8; };
+  // byte offsets: A's rows, B's columns, the output's, inner terms, outer
+  // terms, the further inputs' rows and columns
+  auto linear = [&](const int64_t *t, int bits, int x) {
+    int64_t v = 0;
+    for (int b = 0; b < bits; ++b) v += (x >> b) & 1 ? t[b] : 0;
+    return v;
+  };
+  int64_t *mA = tab, *nB = mA + NMR, *mO = nB + NNR, *nO = mO + NMR, *e2 = nO + NNR, *e1 = e2 + 2 * n2, *xt = e1 + m * n1;
+  for (int x = tid; x < NMR; x += 256) {
+    mA[x] = linear(d.in[0].tile, MM_TM + MGB, x) * unit(0);
+    mO[x] = linear(d.otile, MM_TM + MGB, x) * (int64_t)Bp * 8;
+  }
+  for (int x = tid; x < NNR; x += 256) {
+    nB[x] = linear(d.in[1].tile + MM_MBITS, MM_TN + NGB, x) * unit(1);
+    nO[x] = linear(d.otile + MM_MBITS, MM_TN + NGB, x) * (int64_t)Bp * 8;
+  }
+  for (int x = tid; x < 2 * n2; x += 256) {
+    const int i = x >> d.k2;
+    e2[x] = run_index64(d.in[i].run + d.in[i].nrow, d.in[i].nterm, x & (n2 - 1)) * unit(i);
+  }
+  for (int x = tid; x < m * n1; x += 256) {
+    const int i = x >> d.k1;
+    e1[x] = run_index64(d.in[i].run + d.in[i].nrow, d.in[i].nterm, (uint32_t)(x & (n1 - 1)) << d.k2) * unit(i);
+  }
+  for (int x = tid; x < d.nx * (NMR + NNR); x += 256) {
+    const int y = x / (NMR + NNR), c = x % (NMR + NNR);
+    xt[x] = (c < NMR ? linear(d.in[2 + y].tile, MM_TM + MGB, c) : linear(d.in[2 + y].tile + MM_MBITS, MM_TN + NGB, c - NMR)) *
+            unit(2 + y);
+  }
+  float scale[2 + MM_MAXX];
+  int esum = 0, es = 0, big = 0;
+#pragma unroll
+  for (int i = 0; i < 2 + MM_MAXX; ++i) {
+    scale[i] = 1.f;
+    if (i < m) {
+      int e;
+      operand_scale(meta, d.in[i].meta, hdr, &scale[i], &e);
+      esum += e + (d.in[i].meta >= 0 ? meta[d.in[i].meta].exp : 0);
+      es += e;
+      big += e < 0 ? -e : e;
+    }
+  }
+  if (blockIdx.x == 0 && tid == 0) meta[d.out_meta].exp = esum;
+  __syncthreads();
+  // one factor on each sum, as prog_comb
+  float lmax;
+  if (big <= 60) lmax = mm_tiles<MGB, NGB, NEST, false>(d, ws, mms, tab, scale, __int_as_float((127 - es) << 23), Bp);
+  else lmax = mm_tiles<MGB, NGB, NEST, true>(d, ws, mms, tab, scale, 1.f, Bp);
   record_max(lmax, meta, d.out_meta);
 }
 
@@ -1156,10 +1523,6 @@ __global__ void __launch_bounds__(256) k_gemm(char *ws, const GemmDesc g, Meta *
 // Shared-memory matrix descriptor, K-major without swizzle: start address,
 // leading byte offset (the next 8 summed entries: 128 B), stride byte offset
 // (the next 8-row group: 256 B), descriptor version 1.
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
 __device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
          (1ull << 46);
@@ -2590,6 +2953,26 @@ static void launch_gemm_tc(char *ws, int sms, int Bp, GemmDesc g, const TcCfg &c
 #undef QGM_TC_LAUNCH
 }
 
+// Raise the dynamic shared-memory limit of the staged product-sum kernels
+// (three stages and tables).
+static cudaError_t mm_set_smem(int device) {
+  static std::atomic<bool> done[128];  // per device, for the life of the process
+  if (device >= 0 && device < 128 && done[device]) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+#define QGM_MM_ATTR(MG_, NG_)                                                                                        \
+  for (int q = 0; q < 2 && e == cudaSuccess; ++q)                                                                    \
+    e = cudaFuncSetAttribute(q ? (const void *)k_step_mm<MG_, NG_, true> : (const void *)k_step_mm<MG_, NG_, false>, \
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, mm_stage_bytes(MG_, NG_) + 24 * 1024);
+  QGM_MM_ATTR(3, 3)
+  QGM_MM_ATTR(2, 3)
+  QGM_MM_ATTR(2, 2)
+  QGM_MM_ATTR(1, 2)
+  QGM_MM_ATTR(1, 1)
+#undef QGM_MM_ATTR
+  if (e == cudaSuccess && device >= 0 && device < 128) done[device] = true;
+  return e;
+}
+
 // Raise the dynamic shared-memory limit of every tensor-core kernel.
 static cudaError_t tc_set_smem() {
   cudaError_t e = cudaSuccess;
@@ -2621,19 +3004,56 @@ static cudaError_t tc_set_smem() {
   return e;
 }
 
+// Whether a GEMM-shaped step runs on the tensor cores, and its form there.  By
+// rule all that have one do, but short products stay on the FP32 cores
+// (k_step_mm): with fewer than 16 summed entries most of a chunk is padding,
+// and per batch entry with the batch innermost a product's stores fill 8 of
+// every 32 bytes and its operands are read and written once more as planes,
+// which the tensor cores make up for from 128 summed entries on (512 x 64 x 64
+// per entry, 4 shared indices, 1000 entries: 2.97 ms, k_step_mm 1.54; 128 x 64
+// x 128, 16 shared, 16 entries: 0.058 against 0.064).  An N tile set by the
+// tuner or by hand asks for the tensor cores.
+static bool tc_step(const StepDesc &d, const GemmDesc *gemms, int Bp, int planes, bool bound, const StepTune *tn, TcCfg *c) {
+  if (d.gemm < 0 || (tn && tn->ps)) return false;
+  const GemmDesc &g = gemms[d.gemm];
+  *c = tc_config(g, Bp, planes, tn && tn->nt_cap ? tn->nt_cap : 256);
+  if (!c->ok) return false;
+  MmStep mm;
+  const bool outer = g.a_bout || g.b_bout || g.o_bout, forced = tn && tn->nt_cap;
+  return outer || forced || !bound || !(g.nk <= 3 || (c->perbeta && g.nk <= 6)) || !mm_step(d, Bp, mm);
+}
+
 static void launch_step_ws(char *ws, int sms, int Bp, const StepDesc &d, const GemmDesc *gemms, Meta *meta,
                            Header *hdr, cudaStream_t st, bool tc = false, int64_t planes_off = 0,
-                           int planes = 4, cudaEvent_t mid = nullptr, const StepTune *tn = nullptr) {
+                           int planes = 4, cudaEvent_t mid = nullptr, const StepTune *tn = nullptr, bool bound = true) {
   const uint64_t rows = 1ull << d.w_out;
-  const bool as_ps = tn && tn->ps;  // a GEMM-shaped step the tuner runs as a product-sum
-  if (d.gemm >= 0 && gemms && tc && !as_ps) {
-    const TcCfg c = tc_config(gemms[d.gemm], Bp, planes, tn && tn->nt_cap ? tn->nt_cap : 256);
-    if (c.ok) {
-      launch_gemm_tc(ws, sms, Bp, gemms[d.gemm], c, planes_off, planes, meta, hdr, st, mid, tn && tn->conv);
-      return;
-    }
+  TcCfg c;
+  if (gemms && tc && tc_step(d, gemms, Bp, planes, bound, tn, &c)) {
+    launch_gemm_tc(ws, sms, Bp, gemms[d.gemm], c, planes_off, planes, meta, hdr, st, mid, tn && tn->conv);
+    return;
   }
-  if (d.gemm >= 0 && gemms && gemm_fp32_ok(gemms[d.gemm]) && !as_ps) {
+  // register-tiled forms, unless the tuner or the user set the batched
+  // kernel's own parameters
+  const bool tuned = tn && (tn->T || tn->U);
+  MmStep mm;  // (its shared-memory limit is raised at bind)
+  if (bound && !tuned && mm_step(d, Bp, mm)) {
+    const int64_t tiles = (int64_t)mm.nblk << (mm.wr - mm.rb);
+    const unsigned blocks = (unsigned)std::min<int64_t>(tiles, (int64_t)sms * 8);
+    const size_t sm = (size_t)mm_stage_bytes(mm.mgb, mm.ngb) +
+                      8u * (size_t)((2 + mm.nx) * ((1 << (MM_TM + mm.mgb)) + (1 << (MM_TN + mm.ngb))) + 2 * (1 << mm.k2) +
+                                    (2 + mm.nx) * (1 << mm.k1));
+#define QGM_MM(MG_, NG_)                                                                              \
+  if (mm.nx) k_step_mm<MG_, NG_, true><<<blocks, 256, sm, st>>>(ws, mm, meta, hdr, Bp);               \
+  else k_step_mm<MG_, NG_, false><<<blocks, 256, sm, st>>>(ws, mm, meta, hdr, Bp);
+    if (mm.mgb == 3) { QGM_MM(3, 3) }
+    else if (mm.mgb == 2 && mm.ngb == 3) { QGM_MM(2, 3) }
+    else if (mm.mgb == 2) { QGM_MM(2, 2) }
+    else if (mm.ngb == 2) { QGM_MM(1, 2) }
+    else { QGM_MM(1, 1) }
+#undef QGM_MM
+    return;
+  }
+  if (d.gemm >= 0 && gemms && gemm_fp32_ok(gemms[d.gemm]) && !(tn && tn->ps)) {
     const GemmDesc &g = gemms[d.gemm];
     const dim3 grid(1u << ((g.nm - 6) + (g.nn - (g.nn >= 6 ? 6 : 5))), g.o_bat ? Bp : 1, 1u << g.ns);
     if (g.nn >= 6) {
@@ -2643,6 +3063,18 @@ static void launch_step_ws(char *ws, int sms, int Bp, const StepDesc &d, const G
       if (g.nk >= 5) k_gemm<32, 32><<<grid, 256, 0, st>>>(ws, g, meta, hdr, Bp);
       else k_gemm<16, 32><<<grid, 256, 0, st>>>(ws, g, meta, hdr, Bp);
     }
+    return;
+  }
+  RegStep rg;
+  if (!tuned && reg_step(d, Bp, rg)) {
+    const int64_t total = (int64_t)rg.nblk << (rg.lb + rg.wr);
+    const unsigned blocks = (unsigned)std::min<int64_t>((total + STEP_THREADS - 1) / STEP_THREADS, (int64_t)sms * 64);
+    const size_t sm = (size_t)(2 * (1 << rg.k) + (2 << (rg.tm + rg.tn))) * 8;
+    if (rg.tm == 3 && rg.tn == 2) k_step_reg<3, 2><<<blocks, STEP_THREADS, sm, st>>>(ws, rg, meta, hdr, Bp);
+    else if (rg.tm == 3 && rg.tn == 1) k_step_reg<3, 1><<<blocks, STEP_THREADS, sm, st>>>(ws, rg, meta, hdr, Bp);
+    else if (rg.tm == 3) k_step_reg<3, 0><<<blocks, STEP_THREADS, sm, st>>>(ws, rg, meta, hdr, Bp);
+    else if (rg.tn == 2) k_step_reg<2, 2><<<blocks, STEP_THREADS, sm, st>>>(ws, rg, meta, hdr, Bp);
+    else k_step_reg<2, 0><<<blocks, STEP_THREADS, sm, st>>>(ws, rg, meta, hdr, Bp);
     return;
   }
   auto pow2_floor = [](uint64_t v) {
@@ -2776,17 +3208,15 @@ static int autotune(qgm_plan *p, cudaStream_t st) {
             cand.push_back(t);
           }
     }
-    if (d.gemm >= 0 && d.batched_out && d.tile_t == 0) {
-      // a GEMM-shaped step may also run as a product-sum (batch axis
-      // innermost everywhere: coalesced across batch entries)
+    if (d.gemm >= 0 && d.batched_out) {
+      // a GEMM-shaped step may also run on the FP32 cores (batch axis
+      // innermost everywhere)
       const GemmDesc &g = p->gemms[d.gemm];
-      if (!g.a_bout && !g.b_bout && !g.o_bout)
-        for (int U : {2, 4}) {
-          StepTune t;
-          t.ps = 1;
-          t.U = U;
-          cand.push_back(t);
-        }
+      if (!g.a_bout && !g.b_bout && !g.o_bout) {
+        StepTune t;
+        t.ps = 1;
+        cand.push_back(t);
+      }
     } else if (d.gemm < 0 && d.batched_out && d.tile_t == 0) {
       for (int U : {2, 4, 8})
         for (int T : {1, 2, 4})
@@ -3042,6 +3472,7 @@ int qgm_plan_bind(qgm_plan *p, void *d_workspace, size_t ws_bytes, void *stream)
   CK(cudaDeviceGetAttribute(&x->sms, cudaDevAttrMultiProcessorCount, x->device));
   x->ws = static_cast<char *>(d_workspace);
   if (p->gemm_tc && !p->gemms.empty()) CK(tc_set_smem());
+  CK(mm_set_smem(x->device));
   x->ws_bytes = ws_bytes;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   CK(cudaMemsetAsync(x->ws + p->off_header, 0, 256, st));
@@ -3368,12 +3799,10 @@ int qgm_amplitudes_report(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, 
     for (const ProgramOp &op : p->fprog.ops) {
       per += 1;
       if (op.big < 0) continue;
-      const StepDesc &d = p->fprog.all[op.big];
+      TcCfg c;
       const StepTune &tn = p->tune[op.big];
-      if (d.gemm >= 0 && p->gemm_tc && !tn.ps) {
-        const TcCfg c = tc_config(p->gemms[d.gemm], p->Bp, p->tc_planes, tn.nt_cap ? tn.nt_cap : 256);
-        if (c.ok) per += tn.conv && c.fold ? 1 : 2;
-      }
+      if (p->gemm_tc && tc_step(p->fprog.all[op.big], p->fprog.gemms.data(), p->Bp, p->tc_planes, true, &tn, &c))
+        per += tn.conv && c.fold ? 1 : 2;
     }
     rep->launches = per * rep->slices + 1;
   } else {
@@ -3461,7 +3890,8 @@ int qgm_plan_profile_gemm(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, 
     cudaEvent_t e[3];
     for (auto &x : e) CK(cudaEventCreate(&x));
     CK(cudaEventRecord(e[0], st));
-    const bool tc = p->gemm_tc && tc_config(p->gemms[d.gemm], p->Bp, p->tc_planes).ok;
+    TcCfg tcc;
+    const bool tc = p->gemm_tc && tc_step(d, p->gemms.data(), p->Bp, p->tc_planes, true, tune_of(p, d), &tcc);
     if (!tc) CK(cudaEventRecord(e[1], st));  // no split pass: all of it is the product
     launch_step(p, d, st, tc ? e[1] : nullptr);
     CK(cudaEventRecord(e[2], st));
@@ -3780,7 +4210,7 @@ void static_slice(const qgm_plan *p, char *ws, int sms, const uint64_t *d_bits, 
   const int nl = (int)p->leafdesc.size();
   k_build_leaves<<<std::max(nl, 1), 256, 0, st>>>(ws, reinterpret_cast<const LeafDesc *>(ws + p->off_leafdesc),
                                                    nl, meta, p->n_meta, hdr, d_bits, B, p->Bp, nullptr, 0);
-  for (const StepDesc &d : p->steps) launch_step_ws(ws, sms, p->Bp, d, p->gemms.data(), meta, hdr, st);
+  for (const StepDesc &d : p->steps) launch_step_ws(ws, sms, p->Bp, d, p->gemms.data(), meta, hdr, st, false, 0, 4, nullptr, nullptr, false);
   const int64_t blocks = std::min<int64_t>((B + 255) / 256, (int64_t)sms * 8);
   const cd c = p->constant * std::pow(2.0, -0.5 * p->half_pow_total);
   k_accumulate<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, st>>>(

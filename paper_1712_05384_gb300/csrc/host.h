@@ -247,6 +247,59 @@ struct Program {
   int64_t sync_words() const { return meta_word() + 2 * n_tmp; }
 };
 
+// --------------------------------------------------- register-tiled step
+// A large batched product-sum step of two inputs,
+//   out[c] = sum_e A[e, cm] B[e, cn]
+// for the tile c = (cm, cn) of outputs one thread forms for one batch entry:
+// cm runs over output bits only A holds, cn over bits only B holds, so each
+// loaded value serves a row or a column of the tile.
+constexpr int REG_TM = 3, REG_TN = 2;  // most tile bits of either kind
+struct RegIn {
+  int64_t off;
+  int32_t meta, batched;
+  int32_t nrow, nterm;
+  uint32_t run[PMAXRUN];               // row runs, then term runs (as PIn)
+  int64_t tile[REG_TM + REG_TN];       // index steps of the tile bits (0: not held), cm first
+};
+struct RegStep {
+  int32_t k, tm, tn;                   // summed variables; tile bits
+  int32_t wr, rl;                      // row bits outside the tile; of them below the batch block
+  int32_t lb, nblk;                    // batch entries per block (log2), blocks per row
+  int32_t out_meta, norun;
+  int64_t out_off;
+  uint32_t orun[PMAXRUN];
+  int64_t otile[REG_TM + REG_TN];
+  RegIn in[2];
+};
+
+// A step of two to five inputs as
+//   out[c] = sum_{e1} prod_{i >= 2} F_i[e1, c] * sum_{e2} A[e1, e2, cm] B[e1, e2, cn]
+// with the pair's operands staged in shared memory: e2 are the summed
+// variables the pair (A, B) alone holds; a CTA of 256 threads forms tiles of
+// 2^(3 + mgb) x 2^(2 + ngb) outputs (cm and cn as in RegStep) for 2^lb batch
+// entries and 2^rb rows, a thread 8 x 4 of them.
+constexpr int MM_MAXX = 3;                                  // most further inputs
+constexpr int MM_TM = 3, MM_TN = 2, MM_KC = 4;  // thread tile (log2); summed entries per stage
+constexpr int MM_MBITS = MM_TM + 3, MM_NBITS = MM_TN + 3;
+struct MmIn {
+  int64_t off;
+  int32_t meta, batched;
+  int32_t nrow, nterm;
+  uint32_t run[PMAXRUN];
+  int64_t tile[MM_MBITS + MM_NBITS];  // index steps of the tile bits (0: not held), rows (m) first
+};
+struct MmStep {
+  int32_t nx, k1, k2;      // further inputs; summed variables outside and inside
+  int32_t mgb, ngb, rb;    // thread groups along m and n, rows of a CTA (log2)
+  int32_t lb, nblk;        // batch entries of a CTA (log2), blocks
+  int32_t wr, wp;          // row bits outside the tile; of them, above the rb lowest, held by A or B alone
+  int32_t out_meta, norun;
+  int64_t out_off;
+  uint32_t orun[PMAXRUN];
+  int64_t otile[MM_MBITS + MM_NBITS];
+  MmIn in[2 + MM_MAXX];
+};
+
 // Leaf factor built on the device per slice: base table over
 // (internal vars | slice vars | output vars), MSB first.
 struct LeafDesc {
@@ -494,6 +547,10 @@ int plan_set_params(qgm_plan *p, const double *params);
 void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char> &alone);
 // Whether a step is launched on its own by its size and form.
 bool program_alone(const StepDesc &d, int Bp);
+// The register-tiled form of a step, where it has one that pays.
+bool reg_step(const StepDesc &d, int Bp, RegStep &r);
+// Its form with operands staged in shared memory, likewise.
+bool mm_step(const StepDesc &d, int Bp, MmStep &r);
 // Sizes of the program's workspace region, laid out from `off` on; returns its end.
 int64_t place_program(Program &P, int64_t off);
 // CUDA source of the resident kernel specialised to one layout (jit.cpp):

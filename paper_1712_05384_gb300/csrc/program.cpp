@@ -258,6 +258,247 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
   }
 }
 
+namespace {
+
+// Runs of an index that is linear in the bits of x: bit b of x has value
+// 2^pos[b] (pos < 0: absent).
+int runs_of(const std::vector<int> &pos, uint32_t *run) {
+  int n = 0;
+  for (size_t b = 0; b < pos.size();) {
+    if (pos[b] < 0) {
+      ++b;
+      continue;
+    }
+    size_t l = 1;
+    while (b + l < pos.size() && pos[b + l] == pos[b] + (int)l) ++l;
+    if (n == PMAXRUN) return -1;
+    run[n++] = (uint32_t)(b | l << 8 | (size_t)pos[b] << 16);
+    b += l;
+  }
+  return n;
+}
+
+}  // namespace
+
+bool reg_step(const StepDesc &d, int Bp, RegStep &r) {
+  const int w = d.w_out, k = d.k;
+  if (!d.batched_out || d.m != 2 || k > 8 || w < 3) return false;
+  // position of each union bit in each input
+  std::vector<std::vector<int>> pos(2, std::vector<int>(w + k, -1));
+  for (int i = 0; i < 2; ++i)
+    for (int q = 0; q < d.in[i].nruns; ++q)
+      for (int l = 0; l < d.in[i].len[q]; ++l) pos[i][d.in[i].src[q] + l] = d.in[i].dst[q] + l;
+  int pa = 0, pb = 0;
+  for (int u = 0; u < w; ++u) {
+    pa += pos[0][u] >= 0 && pos[1][u] < 0;
+    pb += pos[1][u] >= 0 && pos[0][u] < 0;
+  }
+  const int A = pa >= pb ? 0 : 1, B = 1 - A;
+  int tm = std::min(std::max(pa, pb), REG_TM), tn = std::min(std::min(pa, pb), REG_TN);
+  // enough threads: smaller tiles while the step would leave SMs idle
+  while (tm + tn > 2 && (w - tm - tn < 1 || std::ldexp((double)Bp, w - tm - tn) < 65536.0)) {
+    if (tm > tn && tm > 2) --tm;
+    else if (tn > 0) --tn;
+    else break;
+  }
+  if (tm == 2 && tn == 1) tn = 0;  // forms compiled: 3+2, 3+1, 3+0, 2+2, 2+0
+  if (tm < 2 || w - tm - tn < 1) return false;
+  // an output with no bit A lacks, and a gate table for B: nothing to reuse;
+  // only short sums gain (several rows' loads in flight; 2^25 outputs, one
+  // term 0.51 -> 0.44 ms; 2^9 outputs x 1000 entries, 64 terms 0.068 -> 0.096)
+  if (tn == 0 && !d.in[B].batched && k > 2) return false;
+  r = RegStep{};
+  r.k = k;
+  r.tm = tm;
+  r.tn = tn;
+  r.out_off = d.out_off;
+  r.out_meta = d.out_meta;
+  // batch entries per block: lanes of a warp along the batch, as many as
+  // waste few on the last block
+  r.lb = 5;
+  while (r.lb > 2 && (((Bp + (1 << r.lb) - 1) >> r.lb) << r.lb) * 8 > Bp * 9) --r.lb;
+  r.nblk = (Bp + (1 << r.lb) - 1) >> r.lb;
+  // tile bits: the highest private bits (the low ones stay neighbours in a row)
+  std::vector<int> tile, row;
+  std::vector<char> is_tile(w, 0);
+  auto pick = [&](int x, int y, int n) {
+    for (int u = w - 1; u >= 0 && n > 0; --u)
+      if (!is_tile[u] && pos[x][u] >= 0 && pos[y][u] < 0) {
+        is_tile[u] = 1;
+        tile.push_back(u);
+        --n;
+      }
+  };
+  pick(A, B, tm);
+  pick(B, A, tn);
+  // row bits: with whole warps along the batch, one bit of either kind below
+  // the batch block, so that the warps of a CTA share their operands in L1
+  if (r.lb == 5)
+    for (int side = 0; side < 2; ++side)
+      for (int u = 0; u < w; ++u)
+        if (!is_tile[u] && std::find(row.begin(), row.end(), u) == row.end() && pos[side ? B : A][u] >= 0 &&
+            pos[side ? A : B][u] < 0) {
+          row.push_back(u);
+          break;
+        }
+  r.rl = r.lb == 5 ? (int)row.size() : std::min(w - tm - tn, 7 - r.lb);
+  for (int u = 0; u < w; ++u)
+    if (!is_tile[u] && std::find(row.begin(), row.end(), u) == row.end()) row.push_back(u);
+  r.wr = (int)row.size();
+  std::vector<int> term;
+  for (int u = w; u < w + k; ++u) term.push_back(u);
+  auto at = [&](const std::vector<int> &p, const std::vector<int> &bits) {
+    std::vector<int> v;
+    for (int u : bits) v.push_back(p[u]);
+    return v;
+  };
+  for (int q = 0; q < 2; ++q) {
+    const int i = q ? B : A;
+    RegIn &x = r.in[q];
+    x.off = d.in[i].off;
+    x.meta = d.in[i].meta;
+    x.batched = d.in[i].batched;
+    x.nrow = runs_of(at(pos[i], row), x.run);
+    if (x.nrow < 0) return false;
+    uint32_t tr[PMAXRUN];
+    x.nterm = runs_of(at(pos[i], term), tr);
+    if (x.nterm < 0 || x.nrow + x.nterm > PMAXRUN) return false;
+    std::copy(tr, tr + x.nterm, x.run + x.nrow);
+    for (size_t b = 0; b < tile.size(); ++b) {
+      const int ps = pos[i][tile[b]];
+      x.tile[(int)b < tm ? b : REG_TM + b - tm] = ps < 0 ? 0 : (int64_t)1 << ps;
+    }
+  }
+  r.norun = runs_of(row, r.orun);
+  if (r.norun < 0) return false;
+  for (size_t b = 0; b < tile.size(); ++b) r.otile[(int)b < tm ? b : REG_TM + b - tm] = (int64_t)1 << tile[b];
+  return true;
+}
+
+bool mm_step(const StepDesc &d, int Bp, MmStep &r) {
+  const int w = d.w_out, k = d.k, m = d.m;
+  if (!d.batched_out || m < 2 || m > 2 + MM_MAXX || k < 2 || k > 16) return false;
+  std::vector<std::vector<int>> pos(m, std::vector<int>(w + k, -1));
+  for (int i = 0; i < m; ++i)
+    for (int q = 0; q < d.in[i].nruns; ++q)
+      for (int l = 0; l < d.in[i].len[q]; ++l) pos[i][d.in[i].src[q] + l] = d.in[i].dst[q] + l;
+  // batch entries per CTA: 8 unless that wastes lanes (64-byte copies, and
+  // the fewer the entries the larger the tile, so the fewer re-reads)
+  const int lb = Bp % 8 == 0 || Bp > 32 ? 3 : 2;
+  // the pair: least work per output; its tile: as many tile rows and columns
+  // as the pair's private bits and 256 threads allow
+  double best = 1e300;
+  int A = -1, B = -1, mgb = 0, ngb = 0, k2 = 0;
+  for (int a = 0; a < m; ++a)
+    for (int b = 0; b < m; ++b) {
+      if (a == b) continue;
+      int pa = 0, pb = 0, in2 = 0;
+      for (int u = 0; u < w; ++u) {
+        pa += pos[a][u] >= 0 && pos[b][u] < 0;
+        pb += pos[b][u] >= 0 && pos[a][u] < 0;
+      }
+      for (int u = w; u < w + k; ++u) {
+        bool out = false;
+        for (int i = 0; i < m; ++i) out = out || (i != a && i != b && pos[i][u] >= 0);
+        in2 += !out;
+      }
+      if (pa < MM_TM || pb < MM_TN || in2 < 2 || in2 > 8 || k - in2 > 8) continue;
+      // forms compiled: thread groups 3+3, 2+3, 2+2, 1+2, 1+1
+      static const int form[5][2] = {{3, 3}, {2, 3}, {2, 2}, {1, 2}, {1, 1}};
+      int f = 0;
+      while (f < 5 && (form[f][0] + MM_TM > pa || form[f][1] + MM_TN > pb || form[f][0] + form[f][1] + lb > 8)) ++f;
+      if (f == 5) continue;
+      const double cost = std::ldexp(1.0, k - in2) * (std::ldexp(1.0, in2) + 3.0 * (m - 2)) * (1.0 + 0.05 * f);
+      if (cost < best) {
+        best = cost;
+        A = a;
+        B = b;
+        mgb = form[f][0];
+        ngb = form[f][1];
+        k2 = in2;
+      }
+    }
+  if (A < 0) return false;
+  r = MmStep{};
+  r.nx = m - 2;
+  r.k1 = k - k2;
+  r.k2 = k2;
+  r.mgb = mgb;
+  r.ngb = ngb;
+  r.lb = lb;
+  r.nblk = (Bp + (1 << lb) - 1) >> lb;
+  r.out_off = d.out_off;
+  r.out_meta = d.out_meta;
+  std::vector<int> tile, row;
+  std::vector<char> used(w, 0);
+  auto priv = [&](int x, int y, int u) { return !used[u] && pos[x][u] >= 0 && pos[y][u] < 0; };
+  auto pick = [&](int x, int y, int n) {
+    for (int u = 0; u < w && n > 0; ++u)
+      if (priv(x, y, u)) {
+        used[u] = 1;
+        tile.push_back(u);
+        --n;
+      }
+  };
+  pick(A, B, MM_TM + mgb);
+  pick(B, A, MM_TN + ngb);
+  // rows: the rb lowest share a CTA; then the pair's other private bits (CTAs
+  // that run together re-read the pair's operands from L2), then the rest
+  const int wr = w - (int)tile.size();
+  r.wr = wr;
+  r.rb = std::min(wr, 8 - lb - mgb - ngb);
+  if (r.rb != 8 - lb - mgb - ngb) return false;  // a CTA's threads are all in use
+  for (int u = 0; u < w && (int)row.size() < r.rb; ++u)
+    if (!used[u]) {
+      used[u] = 1;
+      row.push_back(u);
+    }
+  for (int pass = 0; pass < 2; ++pass)
+    for (int u = 0; u < w; ++u)
+      if (!used[u] && (pass || priv(A, B, u) || priv(B, A, u))) {
+        used[u] = 1;
+        row.push_back(u);
+        r.wp += pass == 0;
+      }
+  std::vector<int> term;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int u = w; u < w + k; ++u) {
+      bool out = false;
+      for (int i = 0; i < m; ++i) out = out || (i != A && i != B && pos[i][u] >= 0);
+      if (out == (pass == 1)) term.push_back(u);
+    }
+  auto at = [&](const std::vector<int> &p, const std::vector<int> &bits) {
+    std::vector<int> v;
+    for (int u : bits) v.push_back(p[u]);
+    return v;
+  };
+  std::vector<int> order = {A, B};
+  for (int i = 0; i < m; ++i)
+    if (i != A && i != B) order.push_back(i);
+  const int mb = MM_TM + mgb;
+  for (int q = 0; q < m; ++q) {
+    const InDesc &in = d.in[order[q]];
+    MmIn &x = r.in[q];
+    x.off = in.off;
+    x.meta = in.meta;
+    x.batched = in.batched;
+    x.nrow = runs_of(at(pos[order[q]], row), x.run);
+    if (x.nrow < 0) return false;
+    uint32_t tr[PMAXRUN];
+    x.nterm = runs_of(at(pos[order[q]], term), tr);
+    if (x.nterm < 0 || x.nrow + x.nterm > PMAXRUN) return false;
+    std::copy(tr, tr + x.nterm, x.run + x.nrow);
+    for (int b = 0; b < (int)tile.size(); ++b) {
+      const int ps = pos[order[q]][tile[b]];
+      x.tile[b < mb ? b : MM_MBITS + b - mb] = ps < 0 ? 0 : (int64_t)1 << ps;
+    }
+  }
+  r.norun = runs_of(row, r.orun);
+  if (r.norun < 0) return false;
+  for (int b = 0; b < (int)tile.size(); ++b) r.otile[b < mb ? b : MM_MBITS + b - mb] = (int64_t)1 << tile[b];
+  return true;
+}
+
 int64_t place_program(Program &P, int64_t off) {
   auto take = [&](int64_t bytes) {
     const int64_t o = off;

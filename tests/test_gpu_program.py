@@ -87,3 +87,26 @@ def test_program_gradients(q, rows, cols, depth, B):
         t[i] -= 2 * eps
         fd = (up - loss(t.reshape(-1, 2))) / (2 * eps)
         assert abs(got[i] - fd) <= 1e-3 * max(abs(fd), 1e-2 * np.max(np.abs(got))), i
+
+
+@pytest.mark.parametrize("rows,cols,depth,B,kw", [
+    (4, 4, 32, 1000, {}), (4, 4, 32, 37, {"max_fuse": 16, "gemm": False}), (4, 6, 30, 4, {"order_kind": 1}),
+    (4, 5, 31, 12, {"order_kind": 1, "max_fuse": 16, "gemm": False}), (5, 5, 28, 20, {"gemm": False}),
+    (5, 6, 28, 16, {"gemm": False}), (6, 6, 25, 37, {}), (4, 6, 34, 6, {"order_kind": 1}), (5, 5, 20, 64, {"open_mask": 7}),
+    (4, 5, 36, 33, {"precision": "fp32"})])
+def test_register_tiled_steps_match_the_general_kernel(q, rows, cols, depth, B, kw):
+    # a pass step by step runs every step with the kernel of its own launch,
+    # small ones too: each form of tile (rows, columns, batch entries per CTA,
+    # further inputs) against the same steps on the general product-sum kernel
+    p = q.Plan(q.Model(q.Circuit.grid(rows, cols, depth, 1)), batch=B, executor=q.EXEC_STEPWISE, **kw).bind()
+    bits = torch.from_numpy(qi.bitstrings(rows * cols, B, 2).astype(np.int64)).cuda()
+    n = 2 * (B << p.n_open)
+    a, b = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2))
+    p.profile(bits, a)
+    assert p.status() == 0
+    outer = {g["step"]: g["o_bout"] or g["in_bout"] for g in p.gemm_shapes()}
+    p.set_tuning([{"step": s, "T": 1, "U": 2, "ps": int(s in outer and not outer[s])} for s in range(p.info.n_steps)])
+    p.profile(bits, b)
+    assert p.status() == 0
+    # two FP32 evaluations of the same sums, each within 1e-5 of the largest
+    assert torch.max(torch.abs(a - b)).item() <= 2e-5 * torch.max(torch.abs(b)).item()

@@ -3402,9 +3402,10 @@ static int check_bound(qgm_plan *p, const char *fn) {
   return QGM_OK;
 }
 
-// Initial shared memory of the compiled resident kernel: zeros (tensor
-// metadata included) with the bitstring-independent leaf rows in place and
-// the recorded maxima of the steps with a static bound (2^k, exponent 0).
+// Initial shared memory of the compiled resident kernel: the tensor metadata
+// (zeros, and the maxima and exponents known beforehand) and the
+// bitstring-independent leaf rows, as the chunks that hold something and
+// their places.
 static int upload_image(qgm_plan *p, const ResidentLayout &L, int smem, cudaStream_t st) {
   const int64_t shift = worklist_bytes(L);
   std::vector<float> img((size_t)smem / 4, 0.f);
@@ -3415,12 +3416,16 @@ static int upload_image(qgm_plan *p, const ResidentLayout &L, int smem, cudaStre
     img[d + 1] = p->base_tables[s2 + 1];
   }
   for (const auto &sb : static_bounds(L)) {
-    const uint32_t bits = (uint32_t)(127 + sb.second.first) << 23;
-    const int32_t ex = sb.second.second;
+    const uint32_t bits = (uint32_t)(127 + sb.second.k) << 23;
+    const int32_t ex = sb.second.exp_known ? sb.second.exp : 0;
     std::memcpy(&img[2 * (size_t)sb.first], &bits, 4);
     std::memcpy(&img[2 * (size_t)sb.first + 1], &ex, 4);
   }
-  CK(cudaMemcpyAsync(p->exec->ws + p->off_image, img.data(), img.size() * 4, cudaMemcpyHostToDevice, st));
+  const std::vector<uint32_t> at = image_chunks(p, L);
+  std::vector<float> out(at.size() * 5);
+  for (size_t i = 0; i < at.size(); ++i) std::memcpy(&out[4 * i], &img[4 * (size_t)at[i]], 16);
+  std::memcpy(&out[4 * at.size()], at.data(), at.size() * 4);
+  CK(cudaMemcpyAsync(p->exec->ws + p->off_image, out.data(), out.size() * 4, cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));
   return QGM_OK;
 }

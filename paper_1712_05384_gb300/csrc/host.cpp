@@ -1199,8 +1199,9 @@ static void build_resident(qgm_plan *p) {
     int64_t image = 0;
     for (const ResidentLayout &L : p->resident) image = std::max(image, compiled_smem(L));
     if (image > 0) {
+      // the chunks that hold something, and their places (4 bytes each)
       p->off_image = p->ws_bytes - 256;
-      p->ws_bytes += (image + 255) & ~int64_t(255);
+      p->ws_bytes += (image + image / 4 + 512) & ~int64_t(255);
     }
   }
   // bitstring-independent outputs read by batched steps (the same tensors and

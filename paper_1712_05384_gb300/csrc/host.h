@@ -11,6 +11,8 @@
 
 #include "qgm.h"
 
+struct qgm_plan;
+
 namespace qgm {
 
 using cd = std::complex<double>;
@@ -195,7 +197,9 @@ inline bool gemm_fp32_ok(const GemmDesc &g) { return g.nk >= 4 && g.nm >= 6 && g
 // ticket counter; a unit waits for the units of the steps it reads (counters
 // in the workspace).  Units are numbered so that a step's producers come
 // first, so a unit only ever waits for units taken before it.
-constexpr int PMAXRUN = 2 * MAXRUN;
+// (a descriptor's runs: a map's, one split between rows and terms, one more
+// where a long sum is cut in two)
+constexpr int PMAXRUN = MAXRUN + 2;
 
 // One input: index = the row's and the term's bits by contiguous runs, each
 // packed as source bit | length << 8 | destination bit << 16 (row runs first).
@@ -393,16 +397,24 @@ struct ResidentLayout {
 // the tensors (the compiled kernel has no work lists and drops them).
 inline int64_t worklist_bytes(const ResidentLayout &L) { return ((int64_t)L.wlist.size() * 4 + 15) & ~int64_t(15); }
 // Steps of the compiled resident kernel with a static bound on their output:
-// every input is a leaf (gate tables: entries of modulus at most 1) or the
-// output of such a step, scaled by the consumer to maxima at most 1/2, so
-// |out| <= 2^k for k summed variables.  That bound, placed in the kernel's
-// initial shared-memory image, serves as the recorded maximum (no run-time
-// reduction); chains of such steps stop after three levels, so that the
-// headroom a loose bound gives away stays far from FP32's range, and the
-// final tensor is always measured (non-finite values reach it and set the
-// status there).  Returns metadata slot -> (k, exponent), the exponent being
-// the sum of the inputs' exponents and scale exponents, as at run time.
-std::map<int, std::pair<int, int>> static_bounds(const ResidentLayout &L);
+// inputs are scaled to maxima at most 1 (gate tables have entries of modulus
+// at most 1), so |out| <= 2^k for k summed variables.  That bound serves as
+// the recorded maximum (no run-time reduction, and a constant scale in the
+// consumer).  Powers of two cost no precision; what a loose bound gives away
+// is headroom towards FP32's smallest values, so it is counted (k bits and one
+// per scaled input, added along the tree) and a step whose bound may be more
+// than 2^48 above its values is measured instead, as is always the final
+// tensor (non-finite values reach it and set the status there).
+struct StaticBound {
+  int k = 0;               // |out| <= 2^k
+  bool exp_known = false;  // every input's exponent is known too:
+  int exp = 0;             //   the output's, else it is formed at run time
+};
+std::map<int, StaticBound> static_bounds(const ResidentLayout &L);  // by metadata slot
+// 16-byte chunks of the compiled resident kernel's initial shared memory that
+// hold something (tensor metadata, bitstring-independent leaf rows); the
+// others are written before they are read
+std::vector<uint32_t> image_chunks(const qgm_plan *p, const ResidentLayout &L);
 // Dynamic shared memory of the compiled resident kernel (16-byte multiple).
 inline int64_t compiled_smem(const ResidentLayout &L) { return (L.smem_bytes - worklist_bytes(L) + 15) & ~int64_t(15); }
 

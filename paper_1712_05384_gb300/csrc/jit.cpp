@@ -15,10 +15,18 @@
 // Arithmetic follows the generic kernel: per-tensor power-of-two exponents
 // (the producer records max |re|,|im|; the consumer scales by 2^-e), one
 // combined scale per output entry when the inputs' exponents sum to a
-// representable power of two, the inputs rescaled in place otherwise.  Two
-// additions: short chains of steps over gate tables take a static bound as
-// their recorded maximum (static_bounds), and shared memory starts from a
-// plan image built at bind.
+// representable power of two, the inputs rescaled in place otherwise.  Three
+// additions.  Most steps take a static bound as their recorded maximum
+// (static_bounds): their consumers' scales are constants and nothing is
+// measured.  In wide steps a thread forms two or four entries that share
+// loads and addresses (emit_tile).  Shared memory starts from the chunks of a
+// plan image that hold something, built at bind.
+//
+// What bounds it: one CTA alone, the chain of dependency levels (5x5 depth 20:
+// 17 levels, 16.6 us before these additions, 10.4 now; 4x4 depth 12: 3.9 and
+// 2.4 us); a full SM (7 CTAs, shared memory), instruction issue: 1024
+// bitstrings of 5x5 depth 20 26.9 -> 21.0 M warp instructions, 47% of them
+// FP32 arithmetic, 37.2 -> 28.5 us (20 -> 26 TFLOP/s).
 #include <cuda_runtime.h>
 #include <dlfcn.h>
 
@@ -121,6 +129,137 @@ void emit_term(std::ostringstream &o, const std::vector<std::string> &f, const s
   o << ind << "  cmac(" << acc << ", p, " << f.back() << "); }\n";
 }
 
+// Wide steps (every thread forms T = 2 or 4 entries): the T entries of a
+// thread differ in item bits J chosen so that the fewest values are loaded
+// (an input is loaded once for all entries that agree in the bits it holds),
+// with constant offsets between them: one address per input, and loads, not
+// index arithmetic, for the other entries.
+void emit_tile(std::ostringstream &o, const ResidentLayout &L, const RStep &r, const StepRec &st,
+               const std::vector<std::vector<int64_t>> &v, int w, int k, int lb, int nw, int64_t n_iter, int64_t shift,
+               bool track_max) {
+  const int m = (int)v.size(), W = w + lb;
+  const int jt = n_iter >= 4 ? 2 : 1, T = 1 << jt;
+  auto log2i = [](int64_t x) { return 63 - __builtin_clzll((unsigned long long)x); };
+  const int lt = log2i(32 * nw), lo = log2i(n_iter) - jt;  // thread bits, loop bits
+  // value of item bit p in input i (bits below lb: the batch entry)
+  auto val = [&](int i, int p) -> int64_t { return p < lb ? (r.in[i].batched ? (int64_t)1 << p : 0) : v[i][p - lb]; };
+  // nested evaluation, as in emit_body
+  const int k2 = st.k_inner, k1 = k - k2;
+  const bool nested = k2 > 0 && k2 <= 4 && (int)st.inner.size() == m;
+  // the bits J: item bits of whole warps (from 5 on, the batch entry below)
+  std::vector<int> J;
+  double best = 1e300;
+  for (int a = std::max(5, lb); a < W; ++a)
+    for (int b = jt == 2 ? a + 1 : a; b < (jt == 2 ? W : a + 1); ++b) {
+      double c = 0;
+      for (int i = 0; i < m; ++i) {
+        int h = val(i, a) != 0;
+        if (jt == 2) h += val(i, b) != 0;
+        c += std::ldexp(nested && !st.inner[i] ? std::ldexp(1.0, -k2) : 1.0, h);
+      }
+      if (c < best) {
+        best = c;
+        J = jt == 2 ? std::vector<int>{a, b} : std::vector<int>{a};
+      }
+    }
+  std::vector<int> tb, ob;
+  for (int p = 0; p < W; ++p)
+    if (std::find(J.begin(), J.end(), p) == J.end()) ((int)tb.size() < lt ? tb : ob).push_back(p);
+  auto expr = [&](const char *x, const std::vector<int> &bits, int i) {  // i < 0: the output
+    std::vector<int64_t> a;
+    for (int p : bits) a.push_back(i < 0 ? (int64_t)1 << p : val(i, p));
+    return bit_map_expr(x, a, 0, (int)a.size());
+  };
+  auto jval = [&](int i, int c) {
+    int64_t x = 0;
+    for (int q = 0; q < jt; ++q)
+      if ((c >> q) & 1) x += i < 0 ? (int64_t)1 << J[q] : val(i, J[q]);
+    return x;
+  };
+  if (track_max) o << "    unsigned lmax = 0u;\n";
+  if (lo) o << "#pragma unroll 1\n    for (int j = 0; j < " << (1 << lo) << "; ++j) {\n";
+  else o << "    {\n";
+  for (int i = 0; i < m; ++i) {
+    o << "      const int b" << i << " = " << ((r.in[i].soff - shift) / 8) << " + " << expr("gt", tb, i);
+    if (lo) o << " + " << expr("j", ob, i);
+    o << ";\n";
+  }
+  o << "      const int bo = " << ((r.out_soff - shift) / 8) << " + " << expr("gt", tb, -1);
+  if (lo) o << " + " << expr("j", ob, -1);
+  o << ";\n";
+  for (int c = 0; c < T; ++c) o << "      float2 a" << c << " = make_float2(0.f, 0.f);\n";
+  // inputs that hold fewer of J first: their products are shared
+  std::vector<int> in_order(m);
+  for (int i = 0; i < m; ++i) in_order[i] = i;
+  std::stable_sort(in_order.begin(), in_order.end(), [&](int a, int b) {
+    int ha = 0, hb = 0;
+    for (int p : J) {
+      ha += val(a, p) != 0;
+      hb += val(b, p) != 0;
+    }
+    return ha < hb;
+  });
+  // one term: the values each entry needs (an entry's value named after the
+  // first entry with the same one), then the T products
+  auto term = [&](int64_t e, bool inner_only, bool outer_only, const std::string &acc, const std::string &lead,
+                  const std::string &base, const std::string &ind) {
+    o << ind << "{\n";
+    std::vector<std::vector<std::string>> f(T);
+    if (!lead.empty())
+      for (int c = 0; c < T; ++c) f[c].push_back(lead + std::to_string(c));
+    for (int i : in_order) {
+      if ((inner_only && !st.inner[i]) || (outer_only && st.inner[i])) continue;
+      std::map<int64_t, int> seen;
+      for (int c = 0; c < T; ++c) {
+        const int64_t x = jval(i, c);
+        auto it = seen.find(x);
+        if (it == seen.end()) {
+          it = seen.emplace(x, c).first;
+          o << ind << "  const float2 x" << i << "_" << c << " = F[" << base << i << " + "
+            << (bit_map_value(e, v[i], w, k) + x) << "];\n";
+        }
+        f[c].push_back("x" + std::to_string(i) + "_" + std::to_string(it->second));
+      }
+    }
+    for (int c = 0; c < T; ++c) emit_term(o, f[c], acc + std::to_string(c), ind + "  ");
+    o << ind << "}\n";
+  };
+  if (nested) {
+    const int u2n = 1 << k2;
+    const int u1_log = std::min(k1, std::max(0, 4 - k2 - jt)), blk_log = k1 - u1_log;
+    if (blk_log) o << "#pragma unroll 1\n      for (int blk = 0; blk < " << (1 << blk_log) << "; ++blk) {\n";
+    else o << "      {\n";
+    for (int i = 0; i < m; ++i)
+      o << "        const int c" << i << " = b" << i << " + "
+        << (blk_log ? bit_map_expr("blk", v[i], w + k2 + u1_log, blk_log) : std::string("0")) << ";\n";
+    for (int u1 = 0; u1 < (1 << u1_log); ++u1) {
+      o << "        {\n";
+      for (int c = 0; c < T; ++c) o << "          float2 i" << c << " = make_float2(0.f, 0.f);\n";
+      for (int u2 = 0; u2 < u2n; ++u2) term(((int64_t)u1 << k2) | u2, true, false, "i", "", "c", "          ");
+      term((int64_t)u1 << k2, false, true, "a", "i", "c", "          ");
+      o << "        }\n";
+    }
+    o << "      }\n";
+  } else {
+    const int unr_log = std::min(k, std::max(0, 4 - jt)), blk_log = k - unr_log;
+    if (blk_log) o << "#pragma unroll 1\n      for (int blk = 0; blk < " << (1 << blk_log) << "; ++blk) {\n";
+    else o << "      {\n";
+    for (int i = 0; i < m; ++i)
+      o << "        const int c" << i << " = b" << i << " + "
+        << (blk_log ? bit_map_expr("blk", v[i], w + unr_log, blk_log) : std::string("0")) << ";\n";
+    for (int u = 0; u < (1 << unr_log); ++u) term(u, false, false, "a", "", "c", "        ");
+    o << "      }\n";
+  }
+  for (int c = 0; c < T; ++c) {
+    o << "      a" << c << " = make_float2(a" << c << ".x * comb, a" << c << ".y * comb); F[bo + " << jval(-1, c) << "] = a" << c
+      << ";\n";
+    if (track_max)
+      o << "      lmax = max(lmax, max(__float_as_uint(a" << c << ".x) & 0x7fffffffu, __float_as_uint(a" << c
+        << ".y) & 0x7fffffffu));\n";
+  }
+  o << "    }\n";
+}
+
 // One step's body for the threads of its warps (gt = thread index in the
 // group): every item's product-sum with raw operand values, times `comb`
 // (2^-es, the inputs' combined scale) per entry.  Shared-memory offsets are
@@ -149,6 +288,10 @@ void emit_body(std::ostringstream &o, const qgm_plan *p, const ResidentLayout &L
   const int k2 = st.k_inner, k1 = k - k2;
   const bool nested = k2 > 0 && k2 <= 4 && lg <= k1 && (int)st.inner.size() == m;
   const int glo = nested ? w + k2 : w;  // union bit of the lane index's bit 0
+  if (lg == 0 && n_iter >= 2 && always_live && (n_iter & (n_iter - 1)) == 0 && w + lb >= 7) {
+    emit_tile(o, L, r, st, v, w, k, lb, nw, n_iter, shift, track_max);
+    return;
+  }
   if (track_max) o << "    unsigned lmax = 0u;\n";
   if (lg) {
     o << "    const int g = gt & " << (tpi - 1) << ";\n";
@@ -228,28 +371,44 @@ void emit_body(std::ostringstream &o, const qgm_plan *p, const ResidentLayout &L
 
 }  // namespace
 
-std::map<int, std::pair<int, int>> static_bounds(const ResidentLayout &L) {
-  std::map<int, std::pair<int, int>> bound;  // metadata slot -> (k, exponent)
-  std::map<int, int> depth;                  // chain depth
+std::map<int, StaticBound> static_bounds(const ResidentLayout &L) {
+  constexpr int kMost = 48;  // bits a bound may lie above the values
+  std::map<int, StaticBound> bound;
+  std::map<int, int> loose;  // metadata slot -> bits
   for (const RStep &r : L.steps) {
-    if (r.out_meta == L.final_meta) continue;
-    int dp = 1, ex = 0;
-    bool ok = true;
-    for (int i = 0; i < r.m && ok; ++i) {
+    StaticBound s;
+    s.k = r.k;
+    s.exp_known = true;
+    int bits = r.k;
+    for (int i = 0; i < r.m; ++i) {
       if (r.in[i].meta < 0) continue;
+      bits += 1;
       auto it = bound.find(r.in[i].meta);
-      if (it == bound.end()) ok = false;
-      else {
-        dp = std::max(dp, depth[r.in[i].meta] + 1);
-        ex += it->second.first + 1 + it->second.second;  // scale exponent k+1, recorded exponent
+      if (it == bound.end()) {
+        s.exp_known = false;  // measured at run time
+        continue;
       }
+      bits += loose[r.in[i].meta];
+      s.exp_known = s.exp_known && it->second.exp_known;
+      s.exp += it->second.k + 1 + it->second.exp;  // scale exponent k+1, recorded exponent
     }
-    if (ok && dp <= 3) {
-      bound[r.out_meta] = {r.k, ex};
-      depth[r.out_meta] = dp;
-    }
+    if (r.out_meta == L.final_meta || bits > kMost) continue;
+    bound[r.out_meta] = s;
+    loose[r.out_meta] = bits;
   }
   return bound;
+}
+
+std::vector<uint32_t> image_chunks(const qgm_plan *p, const ResidentLayout &L) {
+  std::vector<char> used((size_t)(compiled_smem(L) / 16), 0);
+  const int64_t shift = worklist_bytes(L);
+  for (int64_t b = 0; b < (int64_t)p->n_meta_fwd * 8; b += 16) used[b / 16] = 1;
+  for (const RJob &j : L.jobs)
+    if (!j.batched) used[(j.dst - shift) / 16] = 1;
+  std::vector<uint32_t> at;
+  for (size_t c = 0; c < used.size(); ++c)
+    if (used[c]) at.push_back((uint32_t)c);
+  return at;
 }
 
 // CUDA source of the resident kernel specialised to layout L of plan p.
@@ -274,17 +433,18 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
   o << "  const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;\n";
   o << "  const long long b0 = (long long)blockIdx.x * " << L.chunk << ";\n";
   if (pre) o << "  asm volatile(\"griddepcontrol.launch_dependents;\");\n";
-  // shared memory starts as the plan's image: zeros (tensor metadata
-  // included) with the bitstring-independent leaf rows in place
-  const int64_t smem = compiled_smem(L);
+  // shared memory starts with the plan's image (image_chunks)
+  const size_t n_img = image_chunks(p, L).size();
   o << "  {\n    const uint4 *img = reinterpret_cast<const uint4 *>(ws + " << p->off_image << ");\n";
+  o << "    const unsigned *at = reinterpret_cast<const unsigned *>(img + " << n_img << ");\n";
   o << "    uint4 *S = reinterpret_cast<uint4 *>(sm);\n";
-  o << "#pragma unroll 4\n    for (int i = tid; i < " << smem / 16 << "; i += 256) S[i] = __ldg(img + i);\n  }\n";
+  o << "#pragma unroll 2\n    for (int i = tid; i < " << n_img << "; i += 256) S[__ldg(at + i)] = __ldg(img + i);\n  }\n";
   int n_batched = 0;
   for (const RJob &j : L.jobs) n_batched += j.batched != 0;
   if (!pre && n_batched) {
-    // leaf rows that depend on the output bits of x_beta (listed first)
-    o << "  __syncthreads();\n";
+    // leaf rows that depend on the output bits of x_beta (listed first); no
+    // tensor shares a 16-byte chunk with another, so they need not wait for
+    // the image
     o << "  const float2 *wsf = reinterpret_cast<const float2 *>(ws);\n";
     if (L.chunk == 1) o << "  const u64 x1 = b0 < B ? __ldg(bits + b0) : 0ull;\n";
     o << "  for (int t = tid; t < " << (n_batched << logBc) << "; t += 256) {\n";
@@ -317,7 +477,7 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
   }
   o << "  __syncthreads();\n";
   // recorded maxima known before the run: steps with a static bound
-  const std::map<int, std::pair<int, int>> static_k = static_bounds(L);  // slot -> (k of 2^k, exponent)
+  const std::map<int, StaticBound> static_k = static_bounds(L);
   // steps in level order; inside a level grouped by first warp, so that
   // each warp's code for the level is contiguous
   std::vector<size_t> emit_order(L.steps.size());
@@ -341,25 +501,28 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
     o << "  if (wid >= " << w0 << " && wid < " << (w0 + nw) << ") {\n";
     o << "    const int gt = tid - " << (32 * w0) << ";\n";
     // inputs whose producer has a static bound 2^k' get the constant scale
-    // 2^-(k'+1) (exponent k'+1, recorded exponent 0); the others read theirs
+    // 2^-(k'+1) (exponent k'+1); the others read theirs
     int es_static = 0, esum_static = 0;
     bool any_dynamic = false;
+    std::string esum_late;  // recorded exponents read by the thread that records the output's
     for (int i = 0; i < d.m; ++i)
       if (r.in[i].meta >= 0) {
         auto it = static_k.find(r.in[i].meta);
-        if (it != static_k.end()) {
-          es_static += it->second.first + 1;
-          esum_static += it->second.first + 1 + it->second.second;
-        } else {
+        if (it == static_k.end()) {
           any_dynamic = true;
+          continue;
         }
+        es_static += it->second.k + 1;
+        esum_static += it->second.k + 1;
+        if (it->second.exp_known) esum_static += it->second.exp;
+        else esum_late += " + meta[" + std::to_string(r.in[i].meta) + "].exp";
       }
     o << "    int es = " << es_static << ", esum = " << esum_static << ";\n";
     for (int i = 0; i < d.m; ++i) {
       if (r.in[i].meta < 0) continue;
       auto it = static_k.find(r.in[i].meta);
       if (it != static_k.end())
-        o << "    const float s" << i << " = __int_as_float(" << (126 - it->second.first) << " << 23);\n";
+        o << "    const float s" << i << " = __int_as_float(" << (126 - it->second.k) << " << 23);\n";
       else
         o << "    float s" << i << "; { int e; opscale(meta, " << r.in[i].meta << ", s" << i
           << ", e, esum); es += e; }\n";
@@ -386,7 +549,8 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
       else o << "      __syncwarp();\n";
       o << "    }\n";
     }
-    const bool track = static_k.count(r.out_meta) == 0;
+    auto bound = static_k.find(r.out_meta);
+    const bool track = bound == static_k.end();
     {
       std::ostringstream b;
       emit_body(b, p, L, q, shift, track);
@@ -399,8 +563,10 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
       o << "    lm = __reduce_max_sync(0xffffffffu, lm);\n";
       o << "    if (lane == 0) {\n";
       o << "      if (lm) atomicMax(&meta[" << r.out_meta << "].maxbits, lm);\n";
-      o << "      if (wid == " << w0 << ") meta[" << r.out_meta << "].exp = esum;\n";
+      o << "      if (wid == " << w0 << ") meta[" << r.out_meta << "].exp = esum" << esum_late << ";\n";
       o << "    }\n";
+    } else if (!bound->second.exp_known) {
+      o << "    if (gt == 0) meta[" << r.out_meta << "].exp = esum" << esum_late << ";\n";
     }
     o << "  }\n";
   }

@@ -305,6 +305,7 @@ class Plan:
         self.batch = batch
         self.output_mode = output_mode
         self.gradients = bool(gradients)
+        self.params_set = 0  # calls of set_params so far
         self._ws = None
 
     def order(self):
@@ -495,6 +496,7 @@ class Plan:
     def set_params(self, params, stream=None):
         """New (theta, phi) of the RXY gates (flat, 2 per gate) without re-planning."""
         a = np.ascontiguousarray(np.asarray(params, dtype=np.float64).reshape(-1))
+        self.params_set += 1
         check(lib().qgm_plan_set_params(self._h, a.ctypes.data_as(C.POINTER(C.c_double)), a.size, _stream(stream)))
 
     def amplitude_grad(self, d_bits, d_dL_dconja, d_grad, d_amp=None, B=None, stream=None):

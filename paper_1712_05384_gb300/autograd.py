@@ -30,6 +30,7 @@ class AmplitudeFunction(torch.autograd.Function):
         out = torch.empty(2 * B, dtype=torch.float64, device=d_bits.device)
         plan.amplitudes(d_bits, out, B=B)
         ctx.plan = plan
+        ctx.tables = plan.params_set
         ctx.save_for_backward(params, d_bits)
         return torch.view_as_complex(out.view(B, 2))
 
@@ -37,8 +38,9 @@ class AmplitudeFunction(torch.autograd.Function):
     def backward(ctx, grad_a):
         params, d_bits = ctx.saved_tensors
         plan = ctx.plan
-        # the tables of these angles (a later forward may have changed them)
-        plan.set_params(params.detach().to("cpu", torch.float64).numpy())
+        # the tables of these angles, where a later call has set others
+        if plan.params_set != ctx.tables:
+            plan.set_params(params.detach().to("cpu", torch.float64).numpy())
         g = torch.view_as_real((grad_a / 2).to(torch.complex128).contiguous()).reshape(-1).to(d_bits.device)
         d_grad = torch.empty(params.numel(), dtype=torch.float64, device=d_bits.device)
         plan.amplitude_grad(d_bits, g, d_grad, B=d_bits.numel())

@@ -30,6 +30,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -2810,6 +2811,8 @@ struct qgm_exec_state {
   cudaKernel_t jit = nullptr;  // compiled resident kernel (QGM_EXEC_COMPILED)
   cudaKernel_t jit_pre = nullptr;  // its bitstring-independent part, when split off
   std::string jit_error;       // why the compiled kernel is not used, if so
+  std::vector<float> image;    // the compiled kernel's initial shared memory, as uploaded,
+  std::vector<std::pair<int64_t, int64_t>> image_leaf;  // its leaf rows: place in it, in base_tables (floats)
 };
 
 static int cuda_fail(cudaError_t e, const char *what) {
@@ -3406,26 +3409,32 @@ static int check_bound(qgm_plan *p, const char *fn) {
 // (zeros, and the maxima and exponents known beforehand) and the
 // bitstring-independent leaf rows, as the chunks that hold something and
 // their places.
-static int upload_image(qgm_plan *p, const ResidentLayout &L, int smem, cudaStream_t st) {
-  const int64_t shift = worklist_bytes(L);
-  std::vector<float> img((size_t)smem / 4, 0.f);
-  for (const RJob &j : L.jobs) {
-    if (j.batched) continue;
-    const int64_t d = (j.dst - shift) / 4, s2 = 2 * (int64_t)j.src - p->off_base / 4;
-    img[d] = p->base_tables[s2];
-    img[d + 1] = p->base_tables[s2 + 1];
+static int upload_image(qgm_plan *p, const ResidentLayout &L, cudaStream_t st) {
+  qgm_exec_state *x = p->exec;
+  if (x->image.empty()) {
+    const std::vector<uint32_t> at = image_chunks(p, L);
+    std::map<uint32_t, size_t> place;
+    for (size_t i = 0; i < at.size(); ++i) place[at[i]] = i;
+    x->image.assign(at.size() * 5, 0.f);
+    std::memcpy(&x->image[4 * at.size()], at.data(), at.size() * 4);
+    const int64_t shift = worklist_bytes(L);
+    for (const RJob &j : L.jobs) {
+      if (j.batched) continue;
+      const int64_t d = j.dst - shift;
+      x->image_leaf.push_back({4 * (int64_t)place[(uint32_t)(d / 16)] + d % 16 / 4, 2 * (int64_t)j.src - p->off_base / 4});
+    }
+    for (const auto &sb : static_bounds(L)) {
+      const uint32_t bits = (uint32_t)(127 + sb.second.k) << 23;
+      const int32_t ex = sb.second.exp_known ? sb.second.exp : 0;
+      std::memcpy(&x->image[2 * (size_t)sb.first], &bits, 4);  // (the metadata's chunks come first)
+      std::memcpy(&x->image[2 * (size_t)sb.first + 1], &ex, 4);
+    }
   }
-  for (const auto &sb : static_bounds(L)) {
-    const uint32_t bits = (uint32_t)(127 + sb.second.k) << 23;
-    const int32_t ex = sb.second.exp_known ? sb.second.exp : 0;
-    std::memcpy(&img[2 * (size_t)sb.first], &bits, 4);
-    std::memcpy(&img[2 * (size_t)sb.first + 1], &ex, 4);
+  for (const auto &lf : x->image_leaf) {
+    x->image[lf.first] = p->base_tables[lf.second];
+    x->image[lf.first + 1] = p->base_tables[lf.second + 1];
   }
-  const std::vector<uint32_t> at = image_chunks(p, L);
-  std::vector<float> out(at.size() * 5);
-  for (size_t i = 0; i < at.size(); ++i) std::memcpy(&out[4 * i], &img[4 * (size_t)at[i]], 16);
-  std::memcpy(&out[4 * at.size()], at.data(), at.size() * 4);
-  CK(cudaMemcpyAsync(p->exec->ws + p->off_image, out.data(), out.size() * 4, cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(x->ws + p->off_image, x->image.data(), x->image.size() * 4, cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));
   return QGM_OK;
 }
@@ -3570,7 +3579,7 @@ int qgm_plan_bind(qgm_plan *p, void *d_workspace, size_t ws_bytes, void *stream)
         if (kp) CK(cudaKernelSetAttributeForDevice(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, smem, x->device));
         int rc = upload(L);
         if (rc) return rc;
-        rc = upload_image(p, L, smem, st);
+        rc = upload_image(p, L, st);
         if (rc) return rc;
         x->jit = k;
         x->jit_pre = kp;
@@ -3633,7 +3642,7 @@ int qgm_plan_set_params(qgm_plan *p, const double *params, int64_t n, void *stre
                        cudaMemcpyHostToDevice, st));
   if (p->exec->kind == QGM_EXEC_COMPILED) {
     const ResidentLayout &L = p->resident[p->exec->layout];
-    return upload_image(p, L, (int)compiled_smem(L), st);
+    return upload_image(p, L, st);
   }
   CK(cudaStreamSynchronize(st));
   return QGM_OK;

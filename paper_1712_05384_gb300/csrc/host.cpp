@@ -885,6 +885,17 @@ static SimResult simulate(const qgm_plan *p, const std::vector<int> &order_in,
 
 static int64_t pow2(int r) { return (int64_t)1 << r; }
 
+// d/dtheta (which = 0) or d/dphi (1) of RXY's table
+// [[c, -i e^{-i phi} s], [-i e^{i phi} s, c]].
+static void rxy_derivative(const qgm_gate &g, int which, cd t[4]) {
+  const cd I(0.0, 1.0);
+  const double c = std::cos(g.theta / 2), sn = std::sin(g.theta / 2);
+  const cd e = std::exp(I * g.phi), ec = std::conj(e);
+  t[0] = t[3] = which == 0 ? -0.5 * sn : 0.0;
+  t[1] = which == 0 ? -I * ec * (0.5 * c) : -ec * sn;
+  t[2] = which == 0 ? -I * e * (0.5 * c) : e * sn;
+}
+
 // Table of model factor fi (inputs substituted by 0) on `scope`, optionally
 // with the RXY table replaced by its derivative (which = 0: theta, 1: phi).
 static std::vector<cd> member_table(const Model &m, int fi, const std::vector<int> &scope,
@@ -892,22 +903,7 @@ static std::vector<cd> member_table(const Model &m, int fi, const std::vector<in
   const MFactor &f = m.factors[fi];
   cd t[4];
   for (int i = 0; i < 4; ++i) t[i] = f.t[i];
-  if (deriv_which >= 0) {
-    const qgm_gate &g = m.gates[f.gate];
-    const cd I(0.0, 1.0);
-    const double c = std::cos(g.theta / 2), sn = std::sin(g.theta / 2);
-    if (deriv_which == 0) {  // d/dtheta of [[c, -i e^{-i phi} s], [-i e^{i phi} s, c]]
-      t[0] = -0.5 * sn;
-      t[1] = -I * std::exp(-I * g.phi) * (0.5 * c);
-      t[2] = -I * std::exp(I * g.phi) * (0.5 * c);
-      t[3] = -0.5 * sn;
-    } else {  // d/dphi
-      t[0] = 0.0;
-      t[1] = -std::exp(-I * g.phi) * sn;
-      t[2] = std::exp(I * g.phi) * sn;
-      t[3] = 0.0;
-    }
-  }
+  if (deriv_which >= 0) rxy_derivative(m.gates[f.gate], deriv_which, t);
   std::vector<char> is_in(m.n_vars, 0);
   for (int v : m.inputs) is_in[v] = 1;
   std::vector<int> keep;
@@ -1265,11 +1261,44 @@ static void fill_tables(qgm_plan *p) {
   }
 }
 
+// The leaves new angles change, with the place of every table entry in its
+// members' tables (a factor's inputs fixed to 0).
+static void find_param_leaves(qgm_plan *p) {
+  const Model &m = p->model;
+  std::vector<char> is_in(m.n_vars, 0), is_param(m.factors.size(), 0);
+  for (int v : m.inputs) is_in[v] = 1;
+  for (int f : m.param_factor) is_param[f] = 1;
+  p->param_leaf.clear();
+  for (size_t li = 0; li < p->leaves.size(); ++li) {
+    const LeafFactor &L = p->leaves[li];
+    bool any = false;
+    for (int fi : L.members) any = any || is_param[fi];
+    if (!any) continue;
+    const std::vector<int> &layout = p->leaf_layout[li];
+    const int r = (int)layout.size();
+    qgm_plan::ParamLeaf q;
+    q.leaf = (int)li;
+    for (int fi : L.members) {
+      const MFactor &f = m.factors[fi];
+      std::vector<uint8_t> at((size_t)1 << r, 0);
+      for (int a = 0; a < f.nv; ++a) {
+        if (is_in[f.v[a]]) continue;
+        const int w = (int)(std::find(layout.begin(), layout.end(), f.v[a]) - layout.begin());
+        for (size_t i = 0; i < at.size(); ++i)
+          if ((i >> (r - 1 - w)) & 1) at[i] |= (uint8_t)(1 << (f.nv - 1 - a));
+      }
+      q.factor.push_back(fi);
+      q.entry.push_back(at);
+    }
+    p->param_leaf.push_back(q);
+  }
+}
+
 // New angles for the RXY gates of the plan's circuit (params: theta_p at 2p,
-// phi_p at 2p+1, the order of qgm_circuit_param_gates): the gate tables,
-// the merged leaf tables and the constant are recomputed on the host; the
-// variable structure -- and so the order, the steps and the layout -- does
-// not depend on the angles.
+// phi_p at 2p+1, the order of qgm_circuit_param_gates): their gate tables and
+// the merged tables of the leaves that hold them (and their derivatives) are
+// recomputed on the host; the variable structure -- and so the order, the
+// steps and the layout -- does not depend on the angles.
 int plan_set_params(qgm_plan *p, const double *params) {
   Model &m = p->model;
   for (size_t q = 0; q < m.param_factor.size(); ++q) {
@@ -1279,23 +1308,30 @@ int plan_set_params(qgm_plan *p, const double *params) {
     g.phi = params[2 * q + 1];
     gate_table(g, f.t, &f.half_pow);
   }
-  std::vector<LeafFactor> leaves;
-  cd constant;
-  int hp = 0;
-  reduce_factors(m, leaves, constant, hp);
-  if (leaves.size() != p->leaves.size() || hp != p->half_pow_total) {
-    set_error("qgm_plan_set_params: the leaf structure changed");
-    return QGM_ERR_ARG;
+  std::vector<cd> tab;
+  for (const qgm_plan::ParamLeaf &q : p->param_leaf) {
+    const size_t n = q.entry[0].size();
+    auto put = [&](int64_t at, const cd *swapped) {
+      // product of the members' tables, the RXY gate's replaced by `swapped`
+      tab.assign(n, 1.0);
+      for (size_t c = 0; c < q.factor.size(); ++c) {
+        const cd *t = swapped && q.factor[c] == p->rxy_member[q.leaf] ? swapped : m.factors[q.factor[c]].t;
+        for (size_t i = 0; i < n; ++i) tab[i] *= t[q.entry[c][i]];
+      }
+      for (size_t i = 0; i < n; ++i) {
+        p->base_tables[at + 2 * i] = (float)tab[i].real();
+        p->base_tables[at + 2 * i + 1] = (float)tab[i].imag();
+      }
+    };
+    put(p->base_at[q.leaf], nullptr);
+    p->leaves[q.leaf].table = expand_table(p->leaf_layout[q.leaf], tab, p->leaves[q.leaf].scope);
+    if (p->grad && p->rxy_member[q.leaf] >= 0)
+      for (int which = 0; which < 2; ++which) {
+        cd t[4];
+        rxy_derivative(m.gates[m.factors[p->rxy_member[q.leaf]].gate], which, t);
+        put(p->dbase_at[q.leaf] + 2 * which * (int64_t)n, t);
+      }
   }
-  for (size_t li = 0; li < leaves.size(); ++li) {
-    if (leaves[li].scope != p->leaves[li].scope || leaves[li].members != p->leaves[li].members) {
-      set_error("qgm_plan_set_params: the leaf structure changed");
-      return QGM_ERR_ARG;
-    }
-    p->leaves[li].table = leaves[li].table;
-  }
-  p->constant = constant;
-  fill_tables(p);
   return QGM_OK;
 }
 
@@ -1672,6 +1708,7 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
     p->leafdesc.push_back(d);
   }
   fill_tables(p);
+  find_param_leaves(p);
   p->off_leaf = take(leaf_bytes);
   for (size_t li = 0; li < p->leafdesc.size(); ++li) {
     p->leafdesc[li].out_off += p->off_leaf;

@@ -546,6 +546,14 @@ struct qgm_plan {
   std::vector<std::vector<int>> leaf_layout;
   std::vector<int64_t> base_at, dbase_at;
   std::vector<int> rxy_member;
+  // leaves holding an RXY gate (qgm_plan_set_params): per member its factor
+  // and, per entry of the leaf's base table, the entry of the factor's table
+  struct ParamLeaf {
+    int leaf;
+    std::vector<int> factor;
+    std::vector<std::vector<uint8_t>> entry;
+  };
+  std::vector<ParamLeaf> param_leaf;
   bool trees_ok = false;    // buckets of three or more inputs may run as contraction trees
   bool nest_ok = true;      // buckets may be marked for nested evaluation
   qgm_exec_state *exec = nullptr;

@@ -519,7 +519,7 @@ def main():
             ach = g_flops / (g_ms / 1e3) / 1e12
             roof = {"bound": "tensor", "achieved": ach, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
                     "frac": ach / pk["bf16_tflops"], "traffic": NCU_TRAFFIC.get((args.workload, exec_hash())),
-                    "kernel": f"k_gemm_tc / k_gemm_tc_conv with their operand split k_split (GEMM-shaped steps, "
+                    "kernel": f"k_gemm_tc with its operand split k_split (GEMM-shaped steps, "
                               f"split {'FP16' if args.precision == 'fp16' else 'BF16'} on tcgen05; algorithmic flops "
                               f"8*M*N*K per complex product, split terms not counted)",
                     "frac_sustained": ach / pk["bf16_tflops_sustained"], "peak_source": pk["source"] + " (bf16 burst)",

@@ -1504,22 +1504,28 @@ __global__ void __launch_bounds__(256) k_gemm(char *ws, const GemmDesc g, Meta *
 // from the instruction's negate-A bit), im += Ar Bi + Ai Br -- so a chunk of
 // 16 summed entries is 12 (FP16) or 24 (BF16) MMAs of 128 x NT x 16.
 //
-// Product.  One CTA of 128 threads per 128 x NT output tile of one instance.
-// Warp 0 (one lane) streams the tile's plane blocks, one chunk per stage, with
-// bulk asynchronous copies (cp.async.bulk, the TMA unit) into a ring of
-// shared-memory stages, each completing a "full" mbarrier by its byte count;
-// warp 1 (one lane) waits for a stage, issues its MMAs and commits them to the
-// stage's "empty" mbarrier, which frees the stage for the next copy; after the
-// last chunk it commits to "done".  D_re sits in tensor-memory columns
-// [0, NT), D_im in [NT, 2 NT), tile row r in lane r; the four warps then read
-// their 32 lanes back (tcgen05.ld), undo the terms' scale, store through the
-// output's bit maps and record the maximum for the rescale.
+// Product.  One CTA per SM walks over 128 x NT output tiles of the instances
+// (k_gemm_tc).  Its warps have roles that overlap from tile to tile: warp 0
+// (one lane) streams plane blocks, one chunk per stage, with bulk asynchronous
+// copies (cp.async.bulk, the TMA unit) into a ring of shared-memory stages,
+// each completing a "full" mbarrier by its byte count; warp 1 (one lane) waits
+// for a stage, issues its MMAs and commits them to the stage's "empty"
+// mbarrier, which frees the stage, and after a tile's last chunk to the
+// accumulator's "full" barrier; the epilogue warps read the accumulator
+// (tcgen05.ld), undo the terms' scale, store through the output's bit maps,
+// record the maximum for the rescale and arrive on the accumulator's "empty"
+// barrier.  D_re sits in tensor-memory columns [0, NT) of an accumulator, D_im
+// in [NT, 2 NT), tile row r in lane r; with NT <= 128 there are two
+// accumulators, so that a tile's epilogue runs beside the next tile's MMAs
+// (with NT = 256 tensor memory holds one, and the next tile's operands are
+// loaded meanwhile).
 //
 // Every wait is bounded (about one second of %globaltimer).  A wait runs out
-// only if a copy or an MMA never completes; the kernel then stops issuing,
-// records QGM_ERR_TIMEOUT, and still ends with the MMA thread's final commit
-// (tcgen05.commit tracks every MMA that thread issued), which the epilogue
-// waits for before the tensor memory is released.
+// only if a copy or an MMA never completes; every role then leaves its loop
+// (an abort flag in shared memory), the status becomes QGM_ERR_TIMEOUT, and
+// the kernel still ends with the MMA thread's final commit (tcgen05.commit
+// tracks every MMA that thread issued), which that thread waits for before
+// the tensor memory is released.
 
 // Shared-memory matrix descriptor, K-major without swizzle: start address,
 // leading byte offset (the next 8 summed entries: 128 B), stride byte offset
@@ -1701,6 +1707,7 @@ struct TcArgs {
   int32_t s_fast;                 // shared index fastest in the grid (its bits share output sectors)
   int32_t nM, nN, ns;
   int64_t mrows, mtiles, ntiles, kc;
+  int64_t tiles;                  // tiles of all instances
   float out_scale;                // undoes the terms' scale: 2^-30 (FP16) or 1
   uint8_t mO[GMAXB], nO[GMAXB], sO[GMAXB];
   // k_gemm_tc_conv: the M side read as complex64 from the operand itself
@@ -1710,72 +1717,121 @@ struct TcArgs {
 };
 
 __host__ __device__ constexpr int tc_plane_bytes(int rows) { return rows * 32; }
-// stages of the copy ring: up to four, within 220 KB (one CTA per SM) for
-// 256-column tiles and 110 KB (two CTAs per SM) for narrower ones
+// stages of the copy ring: as many as fit 200 KB, up to six
 __host__ __device__ constexpr int tc_stages(int nt, int planes) {
-  return (nt == 256 ? 220 : 110) * 1024 / (planes * tc_plane_bytes(TC_M + nt)) < 4
-             ? (nt == 256 ? 220 : 110) * 1024 / (planes * tc_plane_bytes(TC_M + nt))
-             : 4;
+  return 200 * 1024 / (planes * tc_plane_bytes(TC_M + nt)) < 6 ? 200 * 1024 / (planes * tc_plane_bytes(TC_M + nt)) : 6;
 }
-__host__ __device__ constexpr int tc_smem_bytes(int nt, int planes) {
-  return tc_stages(nt, planes) * planes * (tc_plane_bytes(TC_M) + tc_plane_bytes(nt));
-}
-// k_gemm_tc_conv: two plane stages (the converters write one while the MMAs
-// read the other), and as many stages of the raw ring (the M side's
-// complex64 rows of one chunk, 128 bytes per row) as fit in 220 KB, up to 8:
-// the copies run that many chunks ahead of the conversion, several
-// microseconds of MMA time, which covers the DRAM latency under load
-__host__ __device__ constexpr int tcc_stages(int nt, int planes) { return 2; }
+// With the M side converted in the kernel: two plane stages (the converters
+// write one while the MMAs read the other), and as many stages of the raw
+// ring (the M side's complex64 rows of one chunk, 128 bytes per row) as fit in
+// 212 KB, up to 8: the copies run that many chunks ahead of the conversion.
+// The offsets of the first 1024 summed entries follow.
+constexpr int TCC_STAGES = 2, TCC_KTAB = 1024;
 __host__ __device__ constexpr int tcc_raw_stages(int nt, int planes) {
-  return (220 * 1024 - tcc_stages(nt, planes) * planes * (tc_plane_bytes(TC_M) + tc_plane_bytes(nt))) /
-                     (TC_M * 128) < 8
-             ? (220 * 1024 - tcc_stages(nt, planes) * planes * (tc_plane_bytes(TC_M) + tc_plane_bytes(nt))) /
-                   (TC_M * 128)
+  return (212 * 1024 - TCC_STAGES * planes * tc_plane_bytes(TC_M + nt)) / (TC_M * 128) < 8
+             ? (212 * 1024 - TCC_STAGES * planes * tc_plane_bytes(TC_M + nt)) / (TC_M * 128)
              : 8;
 }
-__host__ __device__ constexpr int tcc_smem_bytes(int nt, int planes) {
-  return tcc_stages(nt, planes) * planes * (tc_plane_bytes(TC_M) + tc_plane_bytes(nt)) +
-         tcc_raw_stages(nt, planes) * TC_M * 128;
+__host__ __device__ constexpr int tc_smem_bytes(int nt, int planes, bool conv) {
+  return conv ? TCC_STAGES * planes * tc_plane_bytes(TC_M + nt) + tcc_raw_stages(nt, planes) * TC_M * 128 + TCC_KTAB * 8
+              : tc_stages(nt, planes) * planes * tc_plane_bytes(TC_M + nt);
 }
-static_assert(tcc_smem_bytes(256, 4) <= 220 * 1024 && tcc_smem_bytes(256, 6) <= 220 * 1024, "conv ring");
+static_assert(tc_smem_bytes(256, 4, true) <= 220 * 1024 && tc_smem_bytes(256, 6, true) <= 220 * 1024, "conv ring");
 
-template <int NT, int P>
-__global__ void __launch_bounds__(128, 1) k_gemm_tc(char *ws, const __grid_constant__ TcArgs a, Meta *meta,
-                                                    Header *hdr) {
-  constexpr int S = tc_stages(NT, P);
-  constexpr int ABYTES = P * tc_plane_bytes(TC_M), BBYTES = P * tc_plane_bytes(NT);
-  constexpr int SBYTES = ABYTES + BBYTES;
-  constexpr uint32_t COLS = 2 * NT < 32 ? 32 : 2 * NT;
-  static_assert(S >= 2, "at least two stages");
+// Half a converted row of a chunk (8 summed entries) into the stage's planes
+// (the layout k_split writes).
+template <int P>
+__device__ __forceinline__ void conv_put(uint8_t *stage, int r, int half, const float2 (&v)[8]) {
+  const int pb = tc_plane_bytes(TC_M);
+  uint8_t *base = stage + (r >> 3) * 256 + half * 128 + (r & 7) * 16;
+  if (P == 4) {
+    uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      split2h(v[2 * q].x, v[2 * q + 1].x, rh[q], rl[q]);
+      split2h(v[2 * q].y, v[2 * q + 1].y, ih[q], il[q]);
+    }
+    *reinterpret_cast<uint4 *>(base) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
+    *reinterpret_cast<uint4 *>(base + pb) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+    *reinterpret_cast<uint4 *>(base + 2 * pb) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
+    *reinterpret_cast<uint4 *>(base + 3 * pb) = make_uint4(il[0], il[1], il[2], il[3]);
+  } else {
+    uint32_t re[3][4], im[3][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      split3(v[2 * q].x, v[2 * q + 1].x, re[0][q], re[1][q], re[2][q]);
+      split3(v[2 * q].y, v[2 * q + 1].y, im[0][q], im[1][q], im[2][q]);
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      *reinterpret_cast<uint4 *>(base + t * pb) = make_uint4(re[t][0], re[t][1], re[t][2], re[t][3]);
+      *reinterpret_cast<uint4 *>(base + (3 + t) * pb) = make_uint4(im[t][0], im[t][1], im[t][2], im[t][3]);
+    }
+  }
+}
+
+// Where a tile lies: its instance (shared index, and batch entry when per
+// entry), M tile and N tile.  The batch entry runs fastest (per-entry products
+// of one tile write the same output sectors, which then merge in L2), then
+// the N tile, the M tile and the shared index; or the shared index before all
+// when its bits share output sectors.
+struct TcTile {
+  int64_t sidx, beta, tn, tm;
+};
+
+__device__ __forceinline__ TcTile tc_tile(const TcArgs &a, int64_t id) {
+  TcTile t{0, 0, 0, 0};
+  if (a.s_fast) {
+    t.sidx = id & ((1ll << a.ns) - 1);
+    id >>= a.ns;
+  }
+  if (a.perbeta) {
+    t.beta = id % a.Bp;
+    id /= a.Bp;
+  }
+  t.tn = id % a.ntiles;
+  id /= a.ntiles;
+  t.tm = id % a.mtiles;
+  if (!a.s_fast) t.sidx = id / a.mtiles;
+  return t;
+}
+
+// CONV: a folded step with the M side converted in the kernel.  When the batch
+// entries fold into the M side (one operand without a batch axis), that side
+// is the large operand streamed once; splitting it in a pass of its own would
+// read and write it once more.  Warps 4-11 convert: two threads copy row r of
+// each chunk (16 complex64 values through the operand's bit maps) into a raw
+// ring in shared memory with cp.async, RS - 1 chunks ahead, scale and split
+// it into the 16-bit planes of the stage, make the stores visible to the
+// tensor cores (fence.proxy.async) and arrive on the stage's "full" mbarrier,
+// which completes when the 256 converters and the N side's bytes are in.
+//
+// What bounds it (5x9 depth 40, K = 256): a 128 x 256 tile's MMAs take 12.3 us
+// of tensor time, and with the conversion's own traffic (raw values in and
+// out, planes in, planes read by the MMAs) shared memory is asked for more
+// than its 128 bytes a clock, so the MMAs of a converted tile last about
+// 16 us; then the epilogue of the one accumulator that fits, 5 to 7 us.  One
+// CTA per tile (the next CTA's allocation, tables and first chunk waiting for
+// the previous one's end) took 31 us a tile, 23 without conversion; walking
+// over tiles takes 24 and 22: M 2^15 x N 2^8 x 64 instances x 4 entries
+// 13.5 -> 10.3 ms, M 2^10 x N 2^8 x 2^10 x 4 7.05 -> 5.46, M 2^13 x N 2^12 x
+// 16 x 4 10.0 -> 9.6 (unconverted), N 2^9 in 128-column tiles with two
+// accumulators 2.40 -> 2.18; K = 16 (M 2^16 x N 2^8 x 16 x 4), all epilogue,
+// 4.53 -> 4.93.  A second warpgroup in the epilogue changed none of them.
+template <int NT, int P, bool CONV>
+__global__ void __launch_bounds__(CONV ? 512 : 256, 1) k_gemm_tc(char *ws, const __grid_constant__ TcArgs a, Meta *meta, Header *hdr) {
+  constexpr int S = CONV ? TCC_STAGES : tc_stages(NT, P), RS = CONV ? tcc_raw_stages(NT, P) : 3;
+  constexpr int ABYTES = P * tc_plane_bytes(TC_M), BBYTES = P * tc_plane_bytes(NT), SBYTES = ABYTES + BBYTES;
+  constexpr int NB = NT == 256 ? 1 : 2;                     // accumulators in tensor memory
+  constexpr uint32_t COLS = NB * 2 * NT < 32 ? 32 : NB * 2 * NT;
+  constexpr int THREADS = CONV ? 512 : 256;                 // the last four warps: epilogue
+  static_assert(S >= 2 && RS >= 3, "stages");
   extern __shared__ __align__(1024) uint8_t tsm[];
-  __shared__ __align__(8) uint64_t bar_full[S], bar_empty[S], bar_done;
+  __shared__ __align__(8) uint64_t bar_full[S], bar_empty[S], bar_acc[NB], bar_free[NB], bar_exit;
   __shared__ uint32_t tbase;
   __shared__ int abort_flag;
   __shared__ int64_t colO[NT];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // tile coordinates: the batch entry fastest (per-entry products of one
-  // tile write the same output sectors, which then merge in L2), then the N
-  // tile, the M tile and the shared index
-  int64_t bid = blockIdx.x;
-  int64_t beta = 0, sidx = 0;
-  if (a.s_fast) {
-    // the output's lowest index bits include a shared variable: the tiles of
-    // neighbouring instances fill the same sectors, so they run together
-    sidx = bid & ((1ll << a.ns) - 1);
-    bid >>= a.ns;
-  }
-  if (a.perbeta) {
-    beta = bid % a.Bp;
-    bid /= a.Bp;
-  }
-  const int64_t tn = bid % a.ntiles;
-  bid /= a.ntiles;
-  const int64_t tm = bid % a.mtiles;
-  if (!a.s_fast) sidx = bid / a.mtiles;
-  const int64_t inst = a.perbeta ? sidx * a.Bp + beta : sidx;
-  const int64_t uO = a.o_bat && !a.o_bout ? (int64_t)a.Bp * 8 : 8;
-  const int64_t bstrideO = a.o_bout ? ((int64_t)8 << a.o_rank) : 8;  // bytes between batch entries
-  for (int j = tid; j < NT; j += 128) colO[j] = lin_bits((uint64_t)(tn * NT + j), a.nO, a.nN) * uO;
   if (tid == 0) abort_flag = 0;
   float sa, sb;
   int ea, eb;
@@ -1790,42 +1846,63 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tc(char *ws, const __grid_const
   }
   if (tid == 0) {
     for (int i = 0; i < S; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_full[i])));
+      // the bulk copies (one arrival with their bytes), and 256 converters
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bar_full[i])), "r"(CONV ? 1 + 2 * TC_M : 1));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_empty[i])));
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_done)));
+    for (int i = 0; i < NB; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_acc[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bar_free[i])), "r"(TC_M));
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_exit)));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
+  // places of the tile's columns (its first column's is added per tile)
+  const int64_t uO = a.o_bat && !a.o_bout ? (int64_t)a.Bp * 8 : 8;
+  for (int j = tid; j < NT; j += THREADS) colO[j] = lin_bits((uint64_t)j, a.nO, a.nN) * uO;
+  const int64_t uA = a.a_batched && !a.a_bout ? (int64_t)a.Bp * 8 : 8;
+  int64_t *ktab = reinterpret_cast<int64_t *>(tsm + tc_smem_bytes(NT, P, CONV) - TCC_KTAB * 8);
+  if (CONV)
+    for (int k = tid; k < TCC_KTAB && k < (1 << a.nk); k += THREADS) ktab[k] = lin_bits((uint64_t)k, a.kA, a.nk) * uA;
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tbase;
   const uint32_t s0 = smem_u32(tsm);
-  const int64_t kc = a.kc;
+  const int kc = (int)a.kc;
+  // a wait that gives up, or sees another role's abort afterwards, ends the role
+  auto wait = [&](uint64_t *bar, uint32_t parity) {
+    if (!tc_wait(smem_u32(bar), parity)) atomicExch(&abort_flag, 1);
+    return *(volatile int *)&abort_flag == 0;
+  };
+  float lmax = 0.f;
   if (warp == 0) {
     if (lane == 0) {
-      // producer: one chunk (both operands' plane blocks) per stage
-      const char *srcA = ws + a.pm_off + (inst * a.mtiles + tm) * kc * ABYTES;
-      const char *srcB = ws + a.pn_off + (inst * a.ntiles + tn) * kc * BBYTES;
-      for (int64_t k = 0; k < kc; ++k) {
-        const int st = (int)(k % S);
-        if (k >= S && !tc_wait(smem_u32(&bar_empty[st]), (uint32_t)((k / S) - 1) & 1u)) {
-          atomicExch(&abort_flag, 1);
-          break;
+      uint32_t g = 0;  // chunks so far: stage g mod S, its use g / S
+      bool ok = true;
+      for (int64_t id = blockIdx.x; id < a.tiles && ok; id += gridDim.x) {
+        const TcTile t = tc_tile(a, id);
+        const int64_t inst = a.perbeta ? t.sidx * a.Bp + t.beta : t.sidx;
+        const char *srcA = ws + a.pm_off + (inst * a.mtiles + t.tm) * kc * ABYTES;
+        const char *srcB = ws + a.pn_off + (inst * a.ntiles + t.tn) * kc * BBYTES;
+        for (int k = 0; k < kc; ++k, ++g) {
+          const int st = (int)(g % S);
+          if (g >= S && !(ok = wait(&bar_empty[st], (g / S - 1) & 1u))) break;
+          const uint32_t fb = smem_u32(&bar_full[st]);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(CONV ? BBYTES : SBYTES)
+                       : "memory");
+          if (!CONV)
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                    s0 + st * SBYTES),
+                "l"(srcA + (int64_t)k * ABYTES), "r"(ABYTES), "r"(fb)
+                : "memory");
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                  s0 + st * SBYTES + ABYTES),
+              "l"(srcB + (int64_t)k * BBYTES), "r"(BBYTES), "r"(fb)
+              : "memory");
         }
-        if (*(volatile int *)&abort_flag) break;
-        const uint32_t fb = smem_u32(&bar_full[st]);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(SBYTES) : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                s0 + st * SBYTES),
-            "l"(srcA + k * ABYTES), "r"(ABYTES), "r"(fb)
-            : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                s0 + st * SBYTES + ABYTES),
-            "l"(srcB + k * BBYTES), "r"(BBYTES), "r"(fb)
-            : "memory");
       }
     }
     __syncwarp();
@@ -1838,362 +1915,165 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tc(char *ws, const __grid_const
       constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(NT >> 3) << 17) |
                                  ((uint32_t)(TC_M >> 4) << 24);
       constexpr uint32_t idesc_neg = idesc | (1u << 13);
-      for (int64_t k = 0; k < kc; ++k) {
-        const int st = (int)(k % S);
-        if (!tc_wait(smem_u32(&bar_full[st]), (uint32_t)(k / S) & 1u)) {
-          atomicExch(&abort_flag, 1);
-          break;
-        }
+      uint32_t g = 0, n = 0;  // chunks, tiles so far
+      bool ok = true;
+      for (int64_t id = blockIdx.x; id < a.tiles && ok; id += gridDim.x, ++n) {
+        const uint32_t b = n % NB, D = tmem + b * 2 * NT;
+        if (n >= NB && !(ok = wait(&bar_free[b], (n / NB - 1) & 1u))) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t sA = s0 + st * SBYTES, sB = sA + ABYTES;
-        uint32_t acc = k > 0 ? 1u : 0u;
-        if (P == 4) {
-          // planes: 0 re high, 1 re low, 2 im high, 3 im low; term pairs
-          // (h, h), (h, l), (l, h)
+        for (int k = 0; k < kc; ++k, ++g) {
+          const int st = (int)(g % S);
+          if (!(ok = wait(&bar_full[st], (g / S) & 1u))) break;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t sA = s0 + st * SBYTES, sB = sA + ABYTES;
+          uint32_t acc = k > 0 ? 1u : 0u;
+          if (P == 4) {
+            // planes: 0 re high, 1 re low, 2 im high, 3 im low; term pairs
+            // (h, h), (h, l), (l, h)
 #pragma unroll
-          for (int t = 0; t < 3; ++t) {
-            const int i = t == 2 ? 1 : 0, j = t == 1 ? 1 : 0;
-            const uint64_t ar = tc_desc(sA + i * tc_plane_bytes(TC_M)), ai = tc_desc(sA + (2 + i) * tc_plane_bytes(TC_M));
-            const uint64_t br = tc_desc(sB + j * tc_plane_bytes(NT)), bi = tc_desc(sB + (2 + j) * tc_plane_bytes(NT));
-            tc_mma(tmem, ar, br, idesc, acc);           // re += Ar Br
-            tc_mma(tmem, ai, bi, idesc_neg, 1u);        // re -= Ai Bi
-            tc_mma(tmem + NT, ar, bi, idesc, acc);      // im += Ar Bi
-            tc_mma(tmem + NT, ai, br, idesc, 1u);       // im += Ai Br
-            acc = 1u;
-          }
-        } else {
-          // planes: 0-2 re terms, 3-5 im terms; term pairs (i, j), i + j <= 2
+            for (int t = 0; t < 3; ++t) {
+              const int i = t == 2 ? 1 : 0, j = t == 1 ? 1 : 0;
+              const uint64_t ar = tc_desc(sA + i * tc_plane_bytes(TC_M)), ai = tc_desc(sA + (2 + i) * tc_plane_bytes(TC_M));
+              const uint64_t br = tc_desc(sB + j * tc_plane_bytes(NT)), bi = tc_desc(sB + (2 + j) * tc_plane_bytes(NT));
+              tc_mma(D, ar, br, idesc, acc);           // re += Ar Br
+              tc_mma(D, ai, bi, idesc_neg, 1u);        // re -= Ai Bi
+              tc_mma(D + NT, ar, bi, idesc, acc);      // im += Ar Bi
+              tc_mma(D + NT, ai, br, idesc, 1u);       // im += Ai Br
+              acc = 1u;
+            }
+          } else {
+            // planes: 0-2 re terms, 3-5 im terms; term pairs (i, j), i + j <= 2
 #pragma unroll
-          for (int t = 0; t < 6; ++t) {
-            const int i = t == 2 || t == 4 ? 1 : t == 5 ? 2 : 0;
-            const int j = t == 1 || t == 4 ? 1 : t == 3 ? 2 : 0;
-            const uint64_t ar = tc_desc(sA + i * tc_plane_bytes(TC_M)), ai = tc_desc(sA + (3 + i) * tc_plane_bytes(TC_M));
-            const uint64_t br = tc_desc(sB + j * tc_plane_bytes(NT)), bi = tc_desc(sB + (3 + j) * tc_plane_bytes(NT));
-            tc_mma(tmem, ar, br, idesc, acc);
-            tc_mma(tmem, ai, bi, idesc_neg, 1u);
-            tc_mma(tmem + NT, ar, bi, idesc, acc);
-            tc_mma(tmem + NT, ai, br, idesc, 1u);
-            acc = 1u;
+            for (int t = 0; t < 6; ++t) {
+              const int i = t == 2 || t == 4 ? 1 : t == 5 ? 2 : 0;
+              const int j = t == 1 || t == 4 ? 1 : t == 3 ? 2 : 0;
+              const uint64_t ar = tc_desc(sA + i * tc_plane_bytes(TC_M)), ai = tc_desc(sA + (3 + i) * tc_plane_bytes(TC_M));
+              const uint64_t br = tc_desc(sB + j * tc_plane_bytes(NT)), bi = tc_desc(sB + (3 + j) * tc_plane_bytes(NT));
+              tc_mma(D, ar, br, idesc, acc);
+              tc_mma(D, ai, bi, idesc_neg, 1u);
+              tc_mma(D + NT, ar, bi, idesc, acc);
+              tc_mma(D + NT, ai, br, idesc, 1u);
+              acc = 1u;
+            }
           }
+          tc_commit(smem_u32(&bar_empty[st]));
         }
-        tc_commit(smem_u32(&bar_empty[st]));
+        if (ok) tc_commit(smem_u32(&bar_acc[b]));
       }
-      // always: every MMA issued above completes before "done" does
-      tc_commit(smem_u32(&bar_done));
+      // always: every MMA issued above completes before "exit" does (they read
+      // only loaded stages, so they finish), and tensor memory is released
+      // after that
+      tc_commit(smem_u32(&bar_exit));
+      if (!tc_wait(smem_u32(&bar_exit), 0u)) tc_wait(smem_u32(&bar_exit), 0u);
     }
     __syncwarp();
-  }
-  // epilogue: thread r = tile row r = tensor-memory lane r
-  bool ok = tc_wait(smem_u32(&bar_done), 0u);
-  if (!ok) ok = tc_wait(smem_u32(&bar_done), 0u);  // MMAs read only loaded stages: they finish
-  ok = __all_sync(0xffffffffu, ok);                 // tcgen05.ld below is warp-collective
-  const bool valid_run = ok && !*(volatile int *)&abort_flag;
-  float lmax = 0.f;
-  if (ok) {
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const int64_t rho = tm * TC_M + tid;
-    const bool valid = valid_run && rho < a.mrows;
-    int64_t m = rho, b2 = beta;
-    if (a.fold) {
-      m = rho / a.Bp;
-      b2 = rho % a.Bp;
-    }
-    char *orow = ws + a.o_off + (lin_bits((uint64_t)sidx, a.sO, a.ns) + lin_bits((uint64_t)(valid ? m : 0), a.mO, a.nM)) * uO +
-                 (a.o_bat ? b2 * bstrideO : 0);
-    const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-    for (int c0 = 0; c0 < NT; c0 += 16) {
-      uint32_t re[16], im[16];
-      tc_ld16(tl + c0, re);
-      tc_ld16(tl + NT + c0, im);
-      if (valid) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float2 v = make_float2(__uint_as_float(re[j]) * a.out_scale, __uint_as_float(im[j]) * a.out_scale);
-          *reinterpret_cast<float2 *>(orow + colO[c0 + j]) = v;
-          lmax = fmax_nan(lmax, absmax2(v));
-        }
-      }
-    }
-  }
-  if (!valid_run && tid == 0 && hdr) atomicCAS(&hdr->status, 0, QGM_ERR_TIMEOUT);
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(COLS));
-  record_max(lmax, meta, a.o_meta);
-}
-
-// The folded tensor-core step with the M side converted in the kernel.  When
-// the batch entries fold into the M side (one operand without a batch axis),
-// that side is the large operand streamed once; splitting it in a separate
-// pass would read and write it once more.  Here 8 warps: warp 0 streams the
-// N side's planes (bulk copies, as k_gemm_tc), warp 1 issues the MMAs, warps
-// 4-7 convert: thread r copies row r of each chunk (16 complex64 values
-// through the operand's bit maps) into a raw ring in shared memory with
-// cp.async, RS - 1 chunks ahead, then scales and splits it into the 16-bit
-// planes of the stage (the layout k_split writes), makes the stores visible
-// to the tensor cores (fence.proxy.async) and arrives on the stage's "full"
-// mbarrier, which completes when the 128 converters and the N side's bytes
-// are in.  Warps 4-7 then read the accumulators back (TMEM lane quadrant =
-// warp % 4).  Waits are bounded as in k_gemm_tc.
-template <int P>
-__device__ __forceinline__ void conv_put(uint8_t *stage, int r, const float2 (&v)[16]) {
-  const int pb = tc_plane_bytes(TC_M);
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    uint8_t *base = stage + (r >> 3) * 256 + half * 128 + (r & 7) * 16;
-    if (P == 4) {
-      uint32_t rh[4], rl[4], ih[4], il[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        split2h(v[half * 8 + 2 * q].x, v[half * 8 + 2 * q + 1].x, rh[q], rl[q]);
-        split2h(v[half * 8 + 2 * q].y, v[half * 8 + 2 * q + 1].y, ih[q], il[q]);
-      }
-      *reinterpret_cast<uint4 *>(base) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
-      *reinterpret_cast<uint4 *>(base + pb) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
-      *reinterpret_cast<uint4 *>(base + 2 * pb) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
-      *reinterpret_cast<uint4 *>(base + 3 * pb) = make_uint4(il[0], il[1], il[2], il[3]);
-    } else {
-      uint32_t re[3][4], im[3][4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        split3(v[half * 8 + 2 * q].x, v[half * 8 + 2 * q + 1].x, re[0][q], re[1][q], re[2][q]);
-        split3(v[half * 8 + 2 * q].y, v[half * 8 + 2 * q + 1].y, im[0][q], im[1][q], im[2][q]);
-      }
-#pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        *reinterpret_cast<uint4 *>(base + t * pb) = make_uint4(re[t][0], re[t][1], re[t][2], re[t][3]);
-        *reinterpret_cast<uint4 *>(base + (3 + t) * pb) = make_uint4(im[t][0], im[t][1], im[t][2], im[t][3]);
-      }
-    }
-  }
-}
-
-template <int NT, int P>
-__global__ void __launch_bounds__(256, 1) k_gemm_tc_conv(char *ws, const __grid_constant__ TcArgs a, Meta *meta,
-                                                         Header *hdr) {
-  constexpr int S = tcc_stages(NT, P), RS = tcc_raw_stages(NT, P);
-  static_assert(RS >= 3, "raw ring");
-  constexpr int ABYTES = P * tc_plane_bytes(TC_M), BBYTES = P * tc_plane_bytes(NT);
-  constexpr int SBYTES = ABYTES + BBYTES;
-  constexpr uint32_t COLS = 2 * NT < 32 ? 32 : 2 * NT;
-  static_assert(S >= 2, "at least two stages");
-  extern __shared__ __align__(1024) uint8_t tsm[];
-  __shared__ __align__(8) uint64_t bar_full[S], bar_empty[S], bar_done;
-  __shared__ uint32_t tbase;
-  __shared__ int abort_flag;
-  __shared__ int64_t colO[NT];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int64_t bid = blockIdx.x;
-  int64_t sidx = 0;
-  if (a.s_fast) {
-    sidx = bid & ((1ll << a.ns) - 1);
-    bid >>= a.ns;
-  }
-  const int64_t tn = bid % a.ntiles;
-  bid /= a.ntiles;
-  const int64_t tm = bid % a.mtiles;
-  if (!a.s_fast) sidx = bid / a.mtiles;
-  const int64_t uO = a.o_bat && !a.o_bout ? (int64_t)a.Bp * 8 : 8;
-  const int64_t bstrideO = a.o_bout ? ((int64_t)8 << a.o_rank) : 8;
-  for (int j = tid; j < NT; j += 256) colO[j] = lin_bits((uint64_t)(tn * NT + j), a.nO, a.nN) * uO;
-  if (tid == 0) abort_flag = 0;
-  float sa, sb;
-  int ea, eb;
-  operand_scale(meta, a.a_meta, hdr, &sa, &ea);
-  operand_scale(meta, a.b_meta, hdr, &sb, &eb);
-  if (blockIdx.x == 0 && tid == 0)
-    meta[a.o_meta].exp = ea + eb + (a.a_meta >= 0 ? meta[a.a_meta].exp : 0) + (a.b_meta >= 0 ? meta[a.b_meta].exp : 0);
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tbase)),
-                 "r"(COLS));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    for (int i = 0; i < S; ++i) {
-      // the N side's bulk copy (one arrival with its bytes) and 128 converters
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bar_full[i])), "r"(1 + TC_M));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_empty[i])));
-    }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_done)));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = tbase;
-  const uint32_t s0 = smem_u32(tsm);
-  const int64_t kc = a.kc;
-  if (warp == 0) {
-    if (lane == 0) {
-      const char *srcB = ws + a.pn_off + (sidx * a.ntiles + tn) * kc * BBYTES;
-      for (int64_t k = 0; k < kc; ++k) {
-        const int st = (int)(k % S);
-        if (k >= S && !tc_wait(smem_u32(&bar_empty[st]), (uint32_t)((k / S) - 1) & 1u)) {
-          atomicExch(&abort_flag, 1);
-          break;
-        }
-        if (*(volatile int *)&abort_flag) break;
-        const uint32_t fb = smem_u32(&bar_full[st]);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(BBYTES) : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                s0 + st * SBYTES + ABYTES),
-            "l"(srcB + k * BBYTES), "r"(BBYTES), "r"(fb)
-            : "memory");
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t fmt = P == 4 ? 0u : 1u;
-      constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(NT >> 3) << 17) |
-                                 ((uint32_t)(TC_M >> 4) << 24);
-      constexpr uint32_t idesc_neg = idesc | (1u << 13);
-      for (int64_t k = 0; k < kc; ++k) {
-        const int st = (int)(k % S);
-        if (!tc_wait(smem_u32(&bar_full[st]), (uint32_t)(k / S) & 1u)) {
-          atomicExch(&abort_flag, 1);
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t sA = s0 + st * SBYTES, sB = sA + ABYTES;
-        uint32_t acc = k > 0 ? 1u : 0u;
-        if (P == 4) {
-#pragma unroll
-          for (int t = 0; t < 3; ++t) {
-            const int i = t == 2 ? 1 : 0, j = t == 1 ? 1 : 0;
-            const uint64_t ar = tc_desc(sA + i * tc_plane_bytes(TC_M)), ai = tc_desc(sA + (2 + i) * tc_plane_bytes(TC_M));
-            const uint64_t br = tc_desc(sB + j * tc_plane_bytes(NT)), bi = tc_desc(sB + (2 + j) * tc_plane_bytes(NT));
-            tc_mma(tmem, ar, br, idesc, acc);
-            tc_mma(tmem, ai, bi, idesc_neg, 1u);
-            tc_mma(tmem + NT, ar, bi, idesc, acc);
-            tc_mma(tmem + NT, ai, br, idesc, 1u);
-            acc = 1u;
-          }
-        } else {
-#pragma unroll
-          for (int t = 0; t < 6; ++t) {
-            const int i = t == 2 || t == 4 ? 1 : t == 5 ? 2 : 0;
-            const int j = t == 1 || t == 4 ? 1 : t == 3 ? 2 : 0;
-            const uint64_t ar = tc_desc(sA + i * tc_plane_bytes(TC_M)), ai = tc_desc(sA + (3 + i) * tc_plane_bytes(TC_M));
-            const uint64_t br = tc_desc(sB + j * tc_plane_bytes(NT)), bi = tc_desc(sB + (3 + j) * tc_plane_bytes(NT));
-            tc_mma(tmem, ar, br, idesc, acc);
-            tc_mma(tmem, ai, bi, idesc_neg, 1u);
-            tc_mma(tmem + NT, ar, bi, idesc, acc);
-            tc_mma(tmem + NT, ai, br, idesc, 1u);
-            acc = 1u;
-          }
-        }
-        tc_commit(smem_u32(&bar_empty[st]));
-      }
-      tc_commit(smem_u32(&bar_done));
-    }
-    __syncwarp();
-  } else if (warp >= 4) {
-    // converters: row r of the M tile.  The raw ring holds, per stage, the
-    // 16 complex64 values of each row for one chunk (128 bytes per row, its
-    // 16-byte pieces rotated by r mod 8 so a quarter-warp's reads hit
-    // distinct banks); each thread fills its own row with 8-byte cp.async
-    // copies RS - 1 chunks ahead, so only its own copy groups are waited on.
-    const int r = tid - 128;
-    const int64_t rho = tm * TC_M + r;
-    const bool live = rho < a.mrows;
-    const int64_t m = a.fold ? rho / a.Bp : rho, beta = a.fold ? rho % a.Bp : 0;
-    const int64_t uA = a.a_batched && !a.a_bout ? (int64_t)a.Bp * 8 : 8;
+  } else if (CONV && warp >= 4 && warp < 12) {
+    // converters: half h (8 summed entries) of row r of the M tile's chunks.
+    // The raw ring holds, per stage, the 16 complex64 values of each row for
+    // one chunk (128 bytes per row, its 16-byte pieces rotated by r mod 8 so a
+    // quarter-warp's reads hit distinct banks); each thread fills its own
+    // values with 8-byte cp.async copies RS - 1 chunks ahead, so only its own
+    // copy groups are waited on.
+    const int r = (tid - 128) & 127, h = (tid - 128) >> 7;
     const int64_t bstrideA = a.a_bout ? ((int64_t)8 << a.a_rank) : 8;
-    const char *rowA = ws + a.a_src_off +
-                       (lin_bits((uint64_t)sidx, a.sA, a.ns) + lin_bits((uint64_t)(live ? m : 0), a.mA, a.nM)) * uA +
-                       (a.a_batched ? beta * bstrideA : 0);
     const float sc = P == 4 ? sa * 32768.f : sa;
-    const int klow = a.nk < 4 ? a.nk : 4;  // summed variables inside a chunk of 16
     const int64_t K = (int64_t)1 << a.nk;
-    int64_t klo[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) klo[q] = q < (1 << klow) ? lin_bits((uint64_t)q, a.kA, klow) * uA : 0;
     uint8_t *raw = tsm + S * SBYTES + r * 128;
     const uint32_t raw_s = smem_u32(raw);
     const int rot = r & 7;
-    auto issue = [&](int64_t k) {
-      const int rs = (int)(k % RS);
-      const char *h = rowA + lin_bits((uint64_t)(k * 16), a.kA, a.nk) * uA;
+    uint32_t g = 0;
+    bool ok = true;
+    for (int64_t id = blockIdx.x; id < a.tiles && ok; id += gridDim.x) {
+      const TcTile t = tc_tile(a, id);
+      const int64_t rho = t.tm * TC_M + r;
+      const bool live = rho < a.mrows;
+      const int64_t m = a.fold ? rho / a.Bp : rho, beta = a.fold ? rho % a.Bp : 0;
+      const char *rowA = ws + a.a_src_off +
+                         (lin_bits((uint64_t)t.sidx, a.sA, a.ns) + lin_bits((uint64_t)(live ? m : 0), a.mA, a.nM)) * uA +
+                         (a.a_batched ? beta * bstrideA : 0);
+      auto issue = [&](int k) {
+        const int rs = k % RS;
+        const int64_t *kt = ktab + ((k * 16) & (TCC_KTAB - 1));
+        const char *src = rowA + (a.nk > 10 ? lin_bits((uint64_t)(k * 16) >> 10, a.kA + 10, a.nk - 10) * uA : 0);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int slot = rs * TC_M * 128 + (((q >> 1) ^ rot) << 4) + ((q & 1) << 3);
-        if (live && q < K) {
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(raw_s + slot), "l"(h + klo[q]) : "memory");
-        } else {
-          *reinterpret_cast<float2 *>(raw + slot) = make_float2(0.f, 0.f);
+        for (int u = 0; u < 8; ++u) {
+          const int q = h * 8 + u, slot = rs * TC_M * 128 + (((q >> 1) ^ rot) << 4) + ((q & 1) << 3);
+          if (live && q < K) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(raw_s + slot), "l"(src + kt[q]) : "memory");
+          } else {
+            *reinterpret_cast<float2 *>(raw + slot) = make_float2(0.f, 0.f);
+          }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+      for (int k = 0; k < RS - 1; ++k) {
+        if (k < kc) issue(k);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    for (int64_t k = 0; k < RS - 1; ++k) {
-      if (k < kc) issue(k);
-      else asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    for (int64_t k = 0; k < kc; ++k) {
-      if (k + RS - 1 < kc) issue(k + RS - 1);
-      else asm volatile("cp.async.commit_group;" ::: "memory");
-      // every group but the newest RS - 1 has landed: chunk k's row is in
-      asm volatile("cp.async.wait_group %0;" ::"n"(RS - 1) : "memory");
-      const int rs = (int)(k % RS);
-      float2 v[16];
+      for (int k = 0; k < kc; ++k, ++g) {
+        if (k + RS - 1 < kc) issue(k + RS - 1);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+        // every group but the newest RS - 1 has landed: chunk k's row is in
+        asm volatile("cp.async.wait_group %0;" ::"n"(RS - 1) : "memory");
+        const int rs = k % RS;
+        float2 v[8];
 #pragma unroll
-      for (int q2 = 0; q2 < 8; ++q2) {
-        const float4 w = *reinterpret_cast<const float4 *>(raw + rs * TC_M * 128 + ((q2 ^ rot) << 4));
-        v[2 * q2] = make_float2(w.x * sc, w.y * sc);
-        v[2 * q2 + 1] = make_float2(w.z * sc, w.w * sc);
+        for (int q2 = 0; q2 < 4; ++q2) {
+          const float4 w = *reinterpret_cast<const float4 *>(raw + rs * TC_M * 128 + (((h * 4 + q2) ^ rot) << 4));
+          v[2 * q2] = make_float2(w.x * sc, w.y * sc);
+          v[2 * q2 + 1] = make_float2(w.z * sc, w.w * sc);
+        }
+        const int st = (int)(g % S);
+        if (g >= S && !(ok = wait(&bar_empty[st], (g / S - 1) & 1u))) break;
+        conv_put<P>(tsm + st * SBYTES, r, h, v);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_full[st])) : "memory");
       }
-      const int st = (int)(k % S);
-      if (k >= S && !tc_wait(smem_u32(&bar_empty[st]), (uint32_t)((k / S) - 1) & 1u)) {
-        atomicExch(&abort_flag, 1);
-        break;
-      }
-      conv_put<P>(tsm + st * SBYTES, r, v);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_full[st])) : "memory");
+      // no copy of this thread is left in flight when its slots are reused,
+      // or the CTA ends
+      asm volatile("cp.async.wait_all;" ::: "memory");
     }
-    // no copy of this thread is left in flight when the CTA ends
-    asm volatile("cp.async.wait_all;" ::: "memory");
-  }
-  // epilogue: warps 4-7, thread tid - 128 = tile row = tensor-memory lane
-  bool ok = tc_wait(smem_u32(&bar_done), 0u);
-  if (!ok) ok = tc_wait(smem_u32(&bar_done), 0u);
-  ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld below is warp-collective
-  const bool valid_run = ok && !*(volatile int *)&abort_flag;
-  float lmax = 0.f;
-  if (ok && warp >= 4) {
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const int64_t rho = tm * TC_M + (tid - 128);
-    const bool valid = valid_run && rho < a.mrows;
-    int64_t m = rho, b2 = 0;
-    if (a.fold) {
-      m = rho / a.Bp;
-      b2 = rho % a.Bp;
-    }
-    char *orow = ws + a.o_off +
-                 (lin_bits((uint64_t)sidx, a.sO, a.ns) + lin_bits((uint64_t)(valid ? m : 0), a.mO, a.nM)) * uO +
-                 (a.o_bat ? b2 * bstrideO : 0);
-    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  } else if (warp >= THREADS / 32 - 4) {
+    // epilogue: tile row = tensor-memory lane = 32 (warp mod 4) + lane
+    const int64_t bstrideO = a.o_bout ? ((int64_t)8 << a.o_rank) : 8;  // bytes between batch entries
+    const int row = tid & 127;
+    uint32_t n = 0;
+    for (int64_t id = blockIdx.x; id < a.tiles; id += gridDim.x, ++n) {
+      const TcTile t = tc_tile(a, id);
+      const int64_t rho = t.tm * TC_M + row;
+      const bool valid = rho < a.mrows;
+      const int64_t m = a.fold ? rho / a.Bp : rho, b2 = a.fold ? rho % a.Bp : t.beta;
+      char *orow = ws + a.o_off +
+                   (lin_bits((uint64_t)t.sidx, a.sO, a.ns) + lin_bits((uint64_t)(valid ? m : 0), a.mO, a.nM) +
+                    lin_bits((uint64_t)(t.tn * NT), a.nO, a.nN)) *
+                       uO +
+                   (a.o_bat ? b2 * bstrideO : 0);
+      const uint32_t b = n % NB;
+      // (warp-uniform: the loads below are warp-collective)
+      if (!__all_sync(0xffffffffu, wait(&bar_acc[b], (n / NB) & 1u))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const uint32_t tl = tmem + b * 2 * NT + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-    for (int c0 = 0; c0 < NT; c0 += 16) {
-      uint32_t re[16], im[16];
-      tc_ld16(tl + c0, re);
-      tc_ld16(tl + NT + c0, im);
-      if (valid) {
+      for (int c0 = 0; c0 < NT; c0 += 16) {
+        uint32_t re[16], im[16];
+        tc_ld16(tl + c0, re);
+        tc_ld16(tl + NT + c0, im);
+        if (valid) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float2 v = make_float2(__uint_as_float(re[j]) * a.out_scale, __uint_as_float(im[j]) * a.out_scale);
-          *reinterpret_cast<float2 *>(orow + colO[c0 + j]) = v;
-          lmax = fmax_nan(lmax, absmax2(v));
+          for (int j = 0; j < 16; ++j) {
+            const float2 v = make_float2(__uint_as_float(re[j]) * a.out_scale, __uint_as_float(im[j]) * a.out_scale);
+            *reinterpret_cast<float2 *>(orow + colO[c0 + j]) = v;
+            lmax = fmax_nan(lmax, absmax2(v));
+          }
         }
       }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_free[b])) : "memory");
     }
   }
-  if (!valid_run && tid == 0 && hdr) atomicCAS(&hdr->status, 0, QGM_ERR_TIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
+  if (tid == 0 && *(volatile int *)&abort_flag && hdr) atomicCAS(&hdr->status, 0, QGM_ERR_TIMEOUT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(COLS));
   record_max(lmax, meta, a.o_meta);
 }
@@ -2922,36 +2802,21 @@ static void launch_gemm_tc(char *ws, int sms, int Bp, GemmDesc g, const TcCfg &c
   std::memcpy(a.mA, g.mA, GMAXB);
   std::memcpy(a.kA, g.kA, GMAXB);
   std::memcpy(a.sA, g.sA, GMAXB);
-  const unsigned grid = (unsigned)(c.inst * c.mtiles * c.ntiles);
-  if (conv) {
-#define QGM_TC_CONV(NT_, P_) \
-  k_gemm_tc_conv<NT_, P_><<<grid, 256, tcc_smem_bytes(NT_, P_), st>>>(ws, a, meta, hdr)
-    if (P == 4) {
-      if (c.nt == 256) QGM_TC_CONV(256, 4);
-      else if (c.nt == 128) QGM_TC_CONV(128, 4);
-      else if (c.nt == 64) QGM_TC_CONV(64, 4);
-      else QGM_TC_CONV(32, 4);
-    } else {
-      if (c.nt == 256) QGM_TC_CONV(256, 6);
-      else if (c.nt == 128) QGM_TC_CONV(128, 6);
-      else if (c.nt == 64) QGM_TC_CONV(64, 6);
-      else QGM_TC_CONV(32, 6);
-    }
-#undef QGM_TC_CONV
-    return;
-  }
-#define QGM_TC_LAUNCH(NT_, P_) \
-  k_gemm_tc<NT_, P_><<<grid, 128, tc_smem_bytes(NT_, P_), st>>>(ws, a, meta, hdr)
+  a.tiles = c.inst * c.mtiles * c.ntiles;
+  const unsigned grid = (unsigned)std::min<int64_t>(a.tiles, sms);
+#define QGM_TC_LAUNCH(NT_, P_)                                                                                        \
+  if (conv) k_gemm_tc<NT_, P_, true><<<grid, 512, tc_smem_bytes(NT_, P_, true), st>>>(ws, a, meta, hdr);              \
+  else k_gemm_tc<NT_, P_, false><<<grid, 256, tc_smem_bytes(NT_, P_, false), st>>>(ws, a, meta, hdr);
   if (P == 4) {
-    if (c.nt == 256) QGM_TC_LAUNCH(256, 4);
-    else if (c.nt == 128) QGM_TC_LAUNCH(128, 4);
-    else if (c.nt == 64) QGM_TC_LAUNCH(64, 4);
-    else QGM_TC_LAUNCH(32, 4);
+    if (c.nt == 256) { QGM_TC_LAUNCH(256, 4) }
+    else if (c.nt == 128) { QGM_TC_LAUNCH(128, 4) }
+    else if (c.nt == 64) { QGM_TC_LAUNCH(64, 4) }
+    else { QGM_TC_LAUNCH(32, 4) }
   } else {
-    if (c.nt == 256) QGM_TC_LAUNCH(256, 6);
-    else if (c.nt == 128) QGM_TC_LAUNCH(128, 6);
-    else if (c.nt == 64) QGM_TC_LAUNCH(64, 6);
-    else QGM_TC_LAUNCH(32, 6);
+    if (c.nt == 256) { QGM_TC_LAUNCH(256, 6) }
+    else if (c.nt == 128) { QGM_TC_LAUNCH(128, 6) }
+    else if (c.nt == 64) { QGM_TC_LAUNCH(64, 6) }
+    else { QGM_TC_LAUNCH(32, 6) }
   }
 #undef QGM_TC_LAUNCH
 }
@@ -2979,30 +2844,21 @@ static cudaError_t mm_set_smem(int device) {
 // Raise the dynamic shared-memory limit of every tensor-core kernel.
 static cudaError_t tc_set_smem() {
   cudaError_t e = cudaSuccess;
-#define QGM_TC_ATTR(NT_, P_)                                                                                  \
-  if (e == cudaSuccess)                                                                                       \
-  e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes(NT_, P_))
-  QGM_TC_ATTR(256, 4);
-  QGM_TC_ATTR(128, 4);
-  QGM_TC_ATTR(64, 4);
-  QGM_TC_ATTR(32, 4);
-  QGM_TC_ATTR(256, 6);
-  QGM_TC_ATTR(128, 6);
-  QGM_TC_ATTR(64, 6);
-  QGM_TC_ATTR(32, 6);
-#undef QGM_TC_ATTR
-#define QGM_TC_ATTR(NT_, P_)                                                                                  \
-  if (e == cudaSuccess)                                                                                       \
-  e = cudaFuncSetAttribute(k_gemm_tc_conv<NT_, P_>, cudaFuncAttributeMaxDynamicSharedMemorySize,              \
-                           tcc_smem_bytes(NT_, P_))
-  QGM_TC_ATTR(256, 4);
-  QGM_TC_ATTR(128, 4);
-  QGM_TC_ATTR(64, 4);
-  QGM_TC_ATTR(32, 4);
-  QGM_TC_ATTR(256, 6);
-  QGM_TC_ATTR(128, 6);
-  QGM_TC_ATTR(64, 6);
-  QGM_TC_ATTR(32, 6);
+#define QGM_TC_ATTR(NT_, P_)                                                                                          \
+  if (e == cudaSuccess)                                                                                               \
+    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,                  \
+                             tc_smem_bytes(NT_, P_, false));                                                          \
+  if (e == cudaSuccess)                                                                                               \
+    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,                   \
+                             tc_smem_bytes(NT_, P_, true));
+  QGM_TC_ATTR(256, 4)
+  QGM_TC_ATTR(128, 4)
+  QGM_TC_ATTR(64, 4)
+  QGM_TC_ATTR(32, 4)
+  QGM_TC_ATTR(256, 6)
+  QGM_TC_ATTR(128, 6)
+  QGM_TC_ATTR(64, 6)
+  QGM_TC_ATTR(32, 6)
 #undef QGM_TC_ATTR
   return e;
 }

@@ -129,6 +129,30 @@ def test_in_kernel_conversion_matches_split_pass(precision):
     assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("rows,cols,depth,B,trees", [(4, 6, 34, 1, None), (4, 7, 40, 32, None), (5, 5, 40, 3, True)])
+def test_tile_counts_around_the_grid(rows, cols, depth, B, trees, precision):
+    # the product kernel's CTAs walk over the tiles: fewer tiles than CTAs
+    # (4x6, one entry), one to seven per CTA with a ragged last round (4x7,
+    # 2^9 to 2^12 rows x 32 entries; 5x5, 2^14 rows per entry of an odd
+    # batch), each N tile with and without conversion, 4 to 512 summed entries (zero-padded
+    # chunks, rings shorter and longer than a tile).  Against the FP32 kernels:
+    # a split product is off by at most 2^-21 of its terms' magnitudes, five
+    # steps by 2.4e-6, the FP32 sums by about as much again.
+    q = Q()
+    m = q.Model(q.Circuit.grid(rows, cols, depth, 0))
+    bits = qi.bitstrings(rows * cols, B, 0)
+    p = q.Plan(m, order_kind=1, batch=B, executor=1, trees=trees, max_fuse=10, precision=precision).bind()
+    ref = q.Plan(m, order_kind=1, batch=B, executor=1, trees=trees, precision="fp32").bind().amplitudes_host(bits)
+    assert p.info.n_gemm_tc_steps >= 2
+    for nt in (64, 128, 256):
+        for conv in (0, 1):
+            p.set_tuning([{"step": g["step"], "nt_cap": nt, "conv": conv} for g in p.gemm_shapes()])
+            a = p.amplitudes_host(bits)
+            assert p.status() == 0
+            assert np.max(np.abs(a - ref)) <= 1e-5 * np.max(np.abs(ref)), (nt, conv)
+
+
 def test_repeat_calls_are_identical():
     # the planes are rewritten on every call: two calls give the same bits
     q = Q()

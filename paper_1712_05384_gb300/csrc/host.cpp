@@ -1401,7 +1401,8 @@ static void forward_program(qgm_plan *p) {
 // found by its offset.
 static void gradient_program(qgm_plan *p) {
   Program &P = p->gprog;
-  P.all = p->gfwd;
+  P.all.reserve(p->gfwd.size() + p->gbwd.size());
+  P.all.insert(P.all.end(), p->gfwd.begin(), p->gfwd.end());
   P.all.insert(P.all.end(), p->gbwd.begin(), p->gbwd.end());
   P.prod.assign(P.all.size(), {});
   std::map<int64_t, int> producer;

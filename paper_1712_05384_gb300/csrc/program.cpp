@@ -44,17 +44,14 @@ PIn make_in(const InDesc &in, int w, int64_t off_meta) {
   p.off = in.off;
   p.meta = in.meta >= 0 ? off_meta + 8 * (int64_t)in.meta : -1;
   p.batched = in.batched;
-  std::vector<uint32_t> row, term;
+  uint32_t term[MAXRUN];
   for (int q = 0; q < in.nruns; ++q) {
     const int s = in.src[q], l = in.len[q], d = in.dst[q];
     const int nr = std::max(0, std::min(l, w - s));
-    if (nr > 0) row.push_back((uint32_t)(s | nr << 8 | d << 16));
-    if (nr < l) term.push_back((uint32_t)((s + nr - w) | (l - nr) << 8 | (d + nr) << 16));
+    if (nr > 0) p.run[p.nrow++] = (uint32_t)(s | nr << 8 | d << 16);
+    if (nr < l) term[p.nterm++] = (uint32_t)((s + nr - w) | (l - nr) << 8 | (d + nr) << 16);
   }
-  p.nrow = (int16_t)row.size();
-  p.nterm = (int16_t)term.size();
-  std::copy(row.begin(), row.end(), p.run);
-  std::copy(term.begin(), term.end(), p.run + row.size());
+  std::copy(term, term + p.nterm, p.run + p.nrow);
   return p;
 }
 
@@ -80,6 +77,7 @@ bool program_alone(const StepDesc &d, int Bp) {
 void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char> &alone) {
   const int n = (int)P.all.size();
   P.steps.clear();
+  P.steps.reserve(n + n / 4 + 8);
   P.tasks.clear();
   P.ops.clear();
   P.n_segments = 0;
@@ -111,6 +109,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
     int chain = -1;
   };
   std::vector<Node> nodes;
+  nodes.reserve(n + n / 4 + 8);
   std::vector<int> node_of(n, -1);
   std::vector<std::vector<int>> readers;
   auto add = [&](Node &&nd) {

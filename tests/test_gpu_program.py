@@ -110,3 +110,27 @@ def test_register_tiled_steps_match_the_general_kernel(q, rows, cols, depth, B, 
     assert p.status() == 0
     # two FP32 evaluations of the same sums, each within 1e-5 of the largest
     assert torch.max(torch.abs(a - b)).item() <= 2e-5 * torch.max(torch.abs(b)).item()
+
+
+@pytest.mark.parametrize("rows,cols,depth,div", [(3, 3, 8, 0), (4, 6, 30, 0), (3, 4, 20, 4)])
+def test_outputs_are_written_whole(q, rows, cols, depth, div):
+    # a pass of one slice stores its amplitudes over whatever the output
+    # holds, launched directly (3x3) or as a graph (4x6); with slices it adds
+    # to zeros; new buffers on every call, and a pass between that leaves the
+    # slice counter elsewhere
+    c = qi.grid_circuit(rows, cols, depth, 6)
+    m = q.Model(q.Circuit.grid(rows, cols, depth, 6))
+    kw = {}
+    if div:
+        kw["mem_budget_bytes"] = q.Plan(m, batch=7, executor=q.EXEC_STEPWISE).info.arena_bytes // div
+    p = q.Plan(m, batch=7, executor=q.EXEC_STEPWISE, **kw).bind()
+    bits = qi.bitstrings(c.n, 7, 3)
+    ref = sv.amplitudes(c, bits)
+    for B in (7, 3):
+        for _ in range(2):
+            out = torch.full((2 * 7,), float("nan"), dtype=torch.float64, device="cuda")
+            p.amplitudes(torch.from_numpy(bits[:B].view(np.int64)).cuda(), out, B=B)
+            a = torch.view_as_complex(out.view(7, 2)).cpu().numpy()
+            assert p.status() == 0 and np.all(np.isnan(a[B:].real))
+            e = errmeasure.measures(a[:B], ref[:B], c.n)
+            assert e["rel"] < TOL and e["abs"] < TOL, e

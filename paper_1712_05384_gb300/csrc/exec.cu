@@ -2198,18 +2198,19 @@ __global__ void k_grad_reduce(const char *ws, const GradParam *gp, const uint64_
 // by the 16 bytes per amplitude, so work is spread over SMs and kept to a few
 // FP64 operations per amplitude.  Statistics of 65536 amplitudes and 10000
 // samples of them: 889 us with one CTA per sum and a logarithm per amplitude,
-// 65 us as below (k_xeb 27, the three k_cdf kernels 12, k_sample 8.5, the
+// 60 us as below (k_xeb 22, the three k_cdf kernels 12, k_sample 8.5, the
 // rest the host's wait for the statistics).
 //
-// The statistics run as one thread-block cluster of SET_CTAS CTAs (the
-// largest portable cluster) whose partial results meet in distributed shared
-// memory: no scratch beyond the caller's four doubles, a fixed order of every
-// sum.  Sum of log p over the set = log of the product: each thread
+// The statistics run as one thread-block cluster whose partial results meet in
+// distributed shared memory: no scratch beyond the caller's four doubles, a
+// fixed order of every sum.  They are bound by the FP64 rate of the SMs that
+// take part: sixteen CTAs (eight is the portable limit) 65 -> 60 us for the
+// whole case.  Sum of log p over the set = log of the product: each thread
 // multiplies the significands (renormalised to [1, 2) after every factor, a
 // relative rounding of 2^-53 each, below the rounding of adding logarithms)
 // and adds the binary exponents as integers; only the whole product's
 // logarithm (about 45 FP64 operations) is taken.
-constexpr int SET_CTAS = 8, SET_THREADS = 1024;
+constexpr int SET_CTAS = 16, SET_THREADS = 1024;  // (8 where the device places no larger cluster)
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -2251,7 +2252,7 @@ __global__ void __launch_bounds__(SET_THREADS) k_xeb(const double2 *a, int64_t B
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   LogSum L{1.0, 0};
   double sx = 0, s1 = 0, s2 = 0;
-  for (int64_t b = (int64_t)blockIdx.x * SET_THREADS + tid; b < B; b += SET_CTAS * SET_THREADS) {
+  for (int64_t b = (int64_t)blockIdx.x * SET_THREADS + tid; b < B; b += (int64_t)gridDim.x * SET_THREADS) {
     const double p = a[b].x * a[b].x + a[b].y * a[b].y;
     const int64_t bits = __double_as_longlong(p);
     const uint32_t x = (uint32_t)(bits >> 52);  // p >= 0 (or NaN): sign and exponent
@@ -2294,7 +2295,7 @@ __global__ void __launch_bounds__(SET_THREADS) k_xeb(const double2 *a, int64_t B
   }
   cluster_sync();
   if (cluster_rank() == 0 && wid == 0) {
-    const bool have = lane < SET_CTAS;
+    const bool have = lane < (int)gridDim.x;
     L = {have ? cluster_peek(&part[0], lane) : 1.0, have ? (int64_t)cluster_peek(&part[1], lane) : 0};
     sx = have ? cluster_peek(&part[2], lane) : 0.0;
     s1 = have ? cluster_peek(&part[3], lane) : 0.0;
@@ -2405,20 +2406,35 @@ __global__ void __launch_bounds__(256) k_sample(const double *cdf, int64_t t, in
   }
 }
 
-// Launch of a one-cluster kernel of SET_CTAS CTAs
-template <typename... A>
-cudaError_t launch_set(void (*k)(A...), cudaStream_t st, A... args) {
+// k_xeb as one cluster of SET_CTAS CTAs, or of eight (the portable size)
+static cudaError_t launch_xeb(const double2 *a, int64_t B, double N, double *sums, cudaStream_t st) {
+  static std::atomic<int> size[128];  // per device: CTAs of the cluster, 0 not known yet
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(SET_CTAS);
   cfg.blockDim = dim3(SET_THREADS);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = SET_CTAS;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, args...);
+  int n = dev < 128 ? size[dev].load() : 0;
+  if (n == 0) {
+    n = SET_CTAS;
+    cfg.gridDim = dim3(n);
+    at[0].val.clusterDim.x = n;
+    int fit = 0;
+    if (cudaFuncSetAttribute(k_xeb, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&fit, k_xeb, &cfg) != cudaSuccess || fit < 1)
+      n = 8;
+    cudaGetLastError();
+    if (dev < 128) size[dev] = n;
+  }
+  cfg.gridDim = dim3(n);
+  at[0].val.clusterDim.x = n;
+  return cudaLaunchKernelEx(&cfg, k_xeb, a, B, N, sums);
 }
 
 // FP32 peak microbenchmark: independent FMA chains per thread (enough of
@@ -3912,7 +3928,7 @@ int qgm_xeb_stats(const double *d_amps, int64_t B, int n_qubits, double *d_scrat
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const double N = std::ldexp(1.0, n_qubits);
-  CK(launch_set(k_xeb, st, reinterpret_cast<const double2 *>(d_amps), B, N, d_scratch));
+  CK(launch_xeb(reinterpret_cast<const double2 *>(d_amps), B, N, d_scratch, st));
   double h[3];
   CK(cudaMemcpyAsync(h, d_scratch, sizeof h, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));

@@ -1705,6 +1705,8 @@ struct TcArgs {
   int32_t o_bat, fold, perbeta, Bp;
   int32_t o_bout, o_rank;         // output batch entry outermost (2^o_rank complex64 per entry)
   int32_t s_fast;                 // shared index fastest in the grid (its bits share output sectors)
+  int32_t pair;                   // a tile holds both instances of the lowest shared bit
+  int32_t pair_n;                 // and the columns' lowest bit is the output's next one
   int32_t nM, nN, ns;
   int64_t mrows, mtiles, ntiles, kc;
   int64_t tiles;                  // tiles of all instances
@@ -1781,9 +1783,10 @@ struct TcTile {
 
 __device__ __forceinline__ TcTile tc_tile(const TcArgs &a, int64_t id) {
   TcTile t{0, 0, 0, 0};
+  const int ns = a.ns - a.pair;
   if (a.s_fast) {
-    t.sidx = id & ((1ll << a.ns) - 1);
-    id >>= a.ns;
+    t.sidx = id & ((1ll << ns) - 1);
+    id >>= ns;
   }
   if (a.perbeta) {
     t.beta = id % a.Bp;
@@ -1793,6 +1796,7 @@ __device__ __forceinline__ TcTile tc_tile(const TcArgs &a, int64_t id) {
   id /= a.ntiles;
   t.tm = id % a.mtiles;
   if (!a.s_fast) t.sidx = id / a.mtiles;
+  t.sidx <<= a.pair;
   return t;
 }
 
@@ -1816,14 +1820,23 @@ __device__ __forceinline__ TcTile tc_tile(const TcArgs &a, int64_t id) {
 // over tiles takes 24 and 22: M 2^15 x N 2^8 x 64 instances x 4 entries
 // 13.5 -> 10.3 ms, M 2^10 x N 2^8 x 2^10 x 4 7.05 -> 5.46, M 2^13 x N 2^12 x
 // 16 x 4 10.0 -> 9.6 (unconverted), N 2^9 in 128-column tiles with two
-// accumulators 2.40 -> 2.18; K = 16 (M 2^16 x N 2^8 x 16 x 4), all epilogue,
-// 4.53 -> 4.93.  A second warpgroup in the epilogue changed none of them.
-template <int NT, int P, bool CONV>
+// accumulators 2.40 -> 2.18.  A second warpgroup in the epilogue changed none
+// of them.
+//
+// G = 2: a short product writes far more than its MMAs take, and where a shared
+// variable is the output's lowest index bit (no batch axis below it) every
+// value of one instance is a quarter or a half of a 32-byte sector, which L2
+// then writes as often.  A tile holds both instances of that variable, in
+// accumulators side by side, and a thread stores whole sectors (the next bit a
+// column's) or halves (a row's, in the neighbouring lane): M 2^16 x N 2^8 x
+// K 16 x 16 x 4 entries, 8.6 GB written, 4.93 -> 1.77 ms (one CTA per tile and
+// instance 4.53).
+template <int NT, int P, bool CONV, int G>
 __global__ void __launch_bounds__(CONV ? 512 : 256, 1) k_gemm_tc(char *ws, const __grid_constant__ TcArgs a, Meta *meta, Header *hdr) {
   constexpr int S = CONV ? TCC_STAGES : tc_stages(NT, P), RS = CONV ? tcc_raw_stages(NT, P) : 3;
   constexpr int ABYTES = P * tc_plane_bytes(TC_M), BBYTES = P * tc_plane_bytes(NT), SBYTES = ABYTES + BBYTES;
-  constexpr int NB = NT == 256 ? 1 : 2;                     // accumulators in tensor memory
-  constexpr uint32_t COLS = NB * 2 * NT < 32 ? 32 : NB * 2 * NT;
+  constexpr int NB = G * NT >= 256 ? 1 : 2;                 // accumulators in tensor memory
+  constexpr uint32_t COLS = NB * G * 2 * NT < 32 ? 32 : NB * G * 2 * NT;
   constexpr int THREADS = CONV ? 512 : 256;                 // the last four warps: epilogue
   static_assert(S >= 2 && RS >= 3, "stages");
   extern __shared__ __align__(1024) uint8_t tsm[];
@@ -1882,10 +1895,11 @@ __global__ void __launch_bounds__(CONV ? 512 : 256, 1) k_gemm_tc(char *ws, const
       bool ok = true;
       for (int64_t id = blockIdx.x; id < a.tiles && ok; id += gridDim.x) {
         const TcTile t = tc_tile(a, id);
-        const int64_t inst = a.perbeta ? t.sidx * a.Bp + t.beta : t.sidx;
-        const char *srcA = ws + a.pm_off + (inst * a.mtiles + t.tm) * kc * ABYTES;
-        const char *srcB = ws + a.pn_off + (inst * a.ntiles + t.tn) * kc * BBYTES;
-        for (int k = 0; k < kc; ++k, ++g) {
+        for (int q = 0; q < G * kc; ++q, ++g) {  // (the second instance's chunks after the first's)
+          const int i = G == 1 ? 0 : q / kc, k = q - i * kc;
+          const int64_t inst = a.perbeta ? (t.sidx + i) * a.Bp + t.beta : t.sidx + i;
+          const char *srcA = ws + a.pm_off + (inst * a.mtiles + t.tm) * kc * ABYTES;
+          const char *srcB = ws + a.pn_off + (inst * a.ntiles + t.tn) * kc * BBYTES;
           const int st = (int)(g % S);
           if (g >= S && !(ok = wait(&bar_empty[st], (g / S - 1) & 1u))) break;
           const uint32_t fb = smem_u32(&bar_full[st]);
@@ -1918,10 +1932,12 @@ __global__ void __launch_bounds__(CONV ? 512 : 256, 1) k_gemm_tc(char *ws, const
       uint32_t g = 0, n = 0;  // chunks, tiles so far
       bool ok = true;
       for (int64_t id = blockIdx.x; id < a.tiles && ok; id += gridDim.x, ++n) {
-        const uint32_t b = n % NB, D = tmem + b * 2 * NT;
+        const uint32_t b = n % NB;
         if (n >= NB && !(ok = wait(&bar_free[b], (n / NB - 1) & 1u))) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        for (int k = 0; k < kc; ++k, ++g) {
+        for (int q = 0; q < G * kc; ++q, ++g) {
+          const int i = G == 1 ? 0 : q / kc, k = q - i * kc;
+          const uint32_t D = tmem + (b * G + i) * 2 * NT;
           const int st = (int)(g % S);
           if (!(ok = wait(&bar_full[st], (g / S) & 1u))) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
@@ -2052,9 +2068,37 @@ __global__ void __launch_bounds__(CONV ? 512 : 256, 1) k_gemm_tc(char *ws, const
       // (warp-uniform: the loads below are warp-collective)
       if (!__all_sync(0xffffffffu, wait(&bar_acc[b], (n / NB) & 1u))) break;
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint32_t tl = tmem + b * 2 * NT + ((uint32_t)((warp & 3) * 32) << 16);
+      const uint32_t tl = tmem + b * G * 2 * NT + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll 1
-      for (int c0 = 0; c0 < NT; c0 += 16) {
+      for (int c0 = 0; G == 2 && c0 < NT; c0 += 16) {
+        uint32_t r0[16], i0[16], r1[16], i1[16];
+        tc_ld16(tl + c0, r0);
+        tc_ld16(tl + NT + c0, i0);
+        tc_ld16(tl + 2 * NT + c0, r1);
+        tc_ld16(tl + 3 * NT + c0, i1);
+        if (valid) {
+          float4 v[16];  // both instances' entries of a column: neighbours in the output
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            v[j] = make_float4(__uint_as_float(r0[j]) * a.out_scale, __uint_as_float(i0[j]) * a.out_scale,
+                               __uint_as_float(r1[j]) * a.out_scale, __uint_as_float(i1[j]) * a.out_scale);
+            lmax = fmax_nan(lmax, fmax_nan(absmax2(make_float2(v[j].x, v[j].y)), absmax2(make_float2(v[j].z, v[j].w))));
+          }
+          if (a.pair_n) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 2)
+              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(orow + colO[c0 + j]), "f"(v[j].x),
+                           "f"(v[j].y), "f"(v[j].z), "f"(v[j].w), "f"(v[j + 1].x), "f"(v[j + 1].y), "f"(v[j + 1].z),
+                           "f"(v[j + 1].w)
+                           : "memory");
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) *reinterpret_cast<float4 *>(orow + colO[c0 + j]) = v[j];
+          }
+        }
+      }
+#pragma unroll 1
+      for (int c0 = 0; G == 1 && c0 < NT; c0 += 16) {
         uint32_t re[16], im[16];
         tc_ld16(tl + c0, re);
         tc_ld16(tl + NT + c0, im);
@@ -2747,6 +2791,14 @@ static void launch_leaves(qgm_plan *p, const uint64_t *d_bits, int64_t B, cudaSt
 // kernels can walk rows by table increments.
 // Tensor-core form of a GEMM-shaped step: split both operands into planes,
 // then the product (see k_split and k_gemm_tc).
+// Two instances a tile (k_gemm_tc, G = 2): the lowest shared variable is the
+// output's lowest index bit, with no batch axis below it, and the product is
+// short.  Both instances' MMAs of 64 columns take about 0.6 us a chunk of 16
+// summed entries, the tile's stores 3 us: up to four chunks hide behind them.
+static bool tc_pair(const GemmDesc &g) {
+  return g.ns > 0 && g.sO[0] == 0 && !(g.o_bat && !g.o_bout) && g.nk <= 6;
+}
+
 static void launch_gemm_tc(char *ws, int sms, int Bp, GemmDesc g, const TcCfg &c, int64_t planes_off, int P,
                            Meta *meta, Header *hdr, cudaStream_t st, cudaEvent_t mid = nullptr, bool conv = false) {
   if (c.swap) gemm_swap_roles(g);
@@ -2798,8 +2850,10 @@ static void launch_gemm_tc(char *ws, int sms, int Bp, GemmDesc g, const TcCfg &c
   // a shared variable among the output's two lowest index bits (one 32-byte
   // sector of complex64) when no batch axis lies below them: instances fastest
   a.s_fast = 0;
+  a.pair = !conv && tc_pair(g) && c.nt <= 128 ? 1 : 0;
+  a.pair_n = a.pair && g.nO[0] == 1 ? 1 : 0;
   if (g.ns > 0 && !(g.o_bat && !g.o_bout))
-    for (int b = 0; b < g.ns; ++b)
+    for (int b = a.pair; b < g.ns; ++b)
       if (g.sO[b] < 2) a.s_fast = 1;
   a.o_rank = g.nm + g.nn + g.ns;
   a.nM = g.nm;
@@ -2821,11 +2875,22 @@ static void launch_gemm_tc(char *ws, int sms, int Bp, GemmDesc g, const TcCfg &c
   std::memcpy(a.mA, g.mA, GMAXB);
   std::memcpy(a.kA, g.kA, GMAXB);
   std::memcpy(a.sA, g.sA, GMAXB);
-  a.tiles = c.inst * c.mtiles * c.ntiles;
+  a.tiles = (c.inst >> a.pair) * c.mtiles * c.ntiles;
   const unsigned grid = (unsigned)std::min<int64_t>(a.tiles, sms);
 #define QGM_TC_LAUNCH(NT_, P_)                                                                                        \
-  if (conv) k_gemm_tc<NT_, P_, true><<<grid, 512, tc_smem_bytes(NT_, P_, true), st>>>(ws, a, meta, hdr);              \
-  else k_gemm_tc<NT_, P_, false><<<grid, 256, tc_smem_bytes(NT_, P_, false), st>>>(ws, a, meta, hdr);
+  if (conv) k_gemm_tc<NT_, P_, true, 1><<<grid, 512, tc_smem_bytes(NT_, P_, true), st>>>(ws, a, meta, hdr);           \
+  else k_gemm_tc<NT_, P_, false, 1><<<grid, 256, tc_smem_bytes(NT_, P_, false), st>>>(ws, a, meta, hdr);
+#define QGM_TC_PAIR(NT_, P_) k_gemm_tc<NT_, P_, false, 2><<<grid, 256, tc_smem_bytes(NT_, P_, false), st>>>(ws, a, meta, hdr);
+  if (a.pair) {
+    if (P == 4 && c.nt == 128) { QGM_TC_PAIR(128, 4) }
+    else if (P == 4 && c.nt == 64) { QGM_TC_PAIR(64, 4) }
+    else if (P == 4) { QGM_TC_PAIR(32, 4) }
+    else if (c.nt == 128) { QGM_TC_PAIR(128, 6) }
+    else if (c.nt == 64) { QGM_TC_PAIR(64, 6) }
+    else { QGM_TC_PAIR(32, 6) }
+    return;
+  }
+#undef QGM_TC_PAIR
   if (P == 4) {
     if (c.nt == 256) { QGM_TC_LAUNCH(256, 4) }
     else if (c.nt == 128) { QGM_TC_LAUNCH(128, 4) }
@@ -2865,16 +2930,27 @@ static cudaError_t tc_set_smem() {
   cudaError_t e = cudaSuccess;
 #define QGM_TC_ATTR(NT_, P_)                                                                                          \
   if (e == cudaSuccess)                                                                                               \
-    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,                  \
+    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,               \
                              tc_smem_bytes(NT_, P_, false));                                                          \
   if (e == cudaSuccess)                                                                                               \
-    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,                   \
+    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
                              tc_smem_bytes(NT_, P_, true));
   QGM_TC_ATTR(256, 4)
   QGM_TC_ATTR(128, 4)
   QGM_TC_ATTR(64, 4)
   QGM_TC_ATTR(32, 4)
   QGM_TC_ATTR(256, 6)
+  QGM_TC_ATTR(128, 6)
+  QGM_TC_ATTR(64, 6)
+  QGM_TC_ATTR(32, 6)
+#undef QGM_TC_ATTR
+#define QGM_TC_ATTR(NT_, P_)                                                                                          \
+  if (e == cudaSuccess)                                                                                               \
+    e = cudaFuncSetAttribute(k_gemm_tc<NT_, P_, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,               \
+                             tc_smem_bytes(NT_, P_, false));
+  QGM_TC_ATTR(128, 4)
+  QGM_TC_ATTR(64, 4)
+  QGM_TC_ATTR(32, 4)
   QGM_TC_ATTR(128, 6)
   QGM_TC_ATTR(64, 6)
   QGM_TC_ATTR(32, 6)
@@ -2894,7 +2970,7 @@ static cudaError_t tc_set_smem() {
 static bool tc_step(const StepDesc &d, const GemmDesc *gemms, int Bp, int planes, bool bound, const StepTune *tn, TcCfg *c) {
   if (d.gemm < 0 || (tn && tn->ps)) return false;
   const GemmDesc &g = gemms[d.gemm];
-  *c = tc_config(g, Bp, planes, tn && tn->nt_cap ? tn->nt_cap : 256);
+  *c = tc_config(g, Bp, planes, tn && tn->nt_cap ? tn->nt_cap : tc_pair(g) && !(tn && tn->conv) ? 64 : 256);
   if (!c->ok) return false;
   MmStep mm;
   const bool outer = g.a_bout || g.b_bout || g.o_bout, forced = tn && tn->nt_cap;

@@ -154,7 +154,7 @@ inline TcCfg tc_config(const GemmDesc &g, int Bp, int planes, int nt_cap = 256) 
   if (c.mrows < TC_M) return c;
   c.mtiles = (c.mrows + TC_M - 1) / TC_M;
   c.nt = c.nN >= 8 ? 256 : (1 << c.nN);
-  if (c.nt > nt_cap && nt_cap >= 32) c.nt = nt_cap;  // narrower N tiles: two CTAs per SM
+  if (c.nt > nt_cap && nt_cap >= 32) c.nt = nt_cap;  // narrower N tiles: two accumulators in tensor memory
   c.ntiles = ((int64_t)1 << c.nN) / c.nt;
   c.kc = (((int64_t)1 << g.nk) + 15) / 16;  // fewer than 16 summed entries: one chunk, zero-padded
   c.inst = ((int64_t)1 << g.ns) * (c.perbeta ? Bp : 1);
@@ -168,7 +168,7 @@ inline TcCfg tc_config(const GemmDesc &g, int Bp, int planes, int nt_cap = 256) 
 // Launch parameters of one step chosen by the autotuner (qgm_plan_opts.autotune)
 // by timing its candidates on the bound device; zeros are the fixed rules.
 struct StepTune {
-  int32_t nt_cap = 0;     // tensor-core GEMM: N tile at most 256, 128 or 64 (0: 256)
+  int32_t nt_cap = 0;     // tensor-core GEMM: N tile at most 256, 128 or 64 (0: the rule)
   int32_t T = 0;          // batched product-sum: term groups per row (0: rule)
   int32_t conv = 0;       // folded tensor-core step: 1 converts the M side in the product kernel
   int32_t U = 0;          // batched product-sum: terms in flight per thread (4 or 8, else 2)

@@ -153,6 +153,26 @@ def test_tile_counts_around_the_grid(rows, cols, depth, B, trees, precision):
             assert np.max(np.abs(a - ref)) <= 1e-5 * np.max(np.abs(ref)), (nt, conv)
 
 
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("rows,cols,depth,B,fuse", [(5, 5, 40, 3, 8), (5, 6, 36, 2, 5)])
+def test_pairs_of_instances(rows, cols, depth, B, fuse, precision):
+    # short products (K = 8) whose output has a shared variable at its lowest
+    # index bit take both its instances into one tile: the next bit a row's
+    # (5x5: half sectors from neighbouring lanes, 64 columns) or a column's
+    # (5x6: whole sectors, 32 columns).  Bound as in
+    # test_tile_counts_around_the_grid.
+    q = Q()
+    m = q.Model(q.Circuit.grid(rows, cols, depth, 0))
+    bits = qi.bitstrings(rows * cols, B, 0)
+    p = q.Plan(m, order_kind=1, batch=B, executor=1, max_fuse=fuse, precision=precision).bind()
+    assert any(g["tc"] and g["o_bout"] and g["nk"] == 3 for g in p.gemm_shapes())
+    a = p.amplitudes_host(bits)
+    assert p.status() == 0
+    del p
+    ref = q.Plan(m, order_kind=1, batch=B, executor=1, max_fuse=fuse, precision="fp32").bind().amplitudes_host(bits)
+    assert np.max(np.abs(a - ref)) <= 1e-5 * np.max(np.abs(ref))
+
+
 def test_repeat_calls_are_identical():
     # the planes are rewritten on every call: two calls give the same bits
     q = Q()

@@ -1712,7 +1712,7 @@ struct TcArgs {
   int64_t tiles;                  // tiles of all instances
   float out_scale;                // undoes the terms' scale: 2^-30 (FP16) or 1
   uint8_t mO[GMAXB], nO[GMAXB], sO[GMAXB];
-  // k_gemm_tc_conv: the M side read as complex64 from the operand itself
+  // converting form: the M side read as complex64 from the operand itself
   int64_t a_src_off;
   int32_t a_batched, a_bout, a_rank, nk;
   uint8_t mA[GMAXB], kA[GMAXB], sA[GMAXB];

@@ -3386,7 +3386,7 @@ static int upload_image(qgm_plan *p, const ResidentLayout &L, cudaStream_t st) {
       const int64_t d = j.dst - shift;
       x->image_leaf.push_back({4 * (int64_t)place[(uint32_t)(d / 16)] + d % 16 / 4, 2 * (int64_t)j.src - p->off_base / 4});
     }
-    for (const auto &sb : static_bounds(L)) {
+    for (const auto &sb : static_bounds(p, L)) {
       const uint32_t bits = (uint32_t)(127 + sb.second.k) << 23;
       const int32_t ex = sb.second.exp_known ? sb.second.exp : 0;
       std::memcpy(&x->image[2 * (size_t)sb.first], &bits, 4);  // (the metadata's chunks come first)

@@ -396,21 +396,38 @@ struct ResidentLayout {
 // Shared-memory bytes of the work lists, which sit between the metadata and
 // the tensors (the compiled kernel has no work lists and drops them).
 inline int64_t worklist_bytes(const ResidentLayout &L) { return ((int64_t)L.wlist.size() * 4 + 15) & ~int64_t(15); }
+// Parametrised gates each tensor of the elimination is formed from.
+std::vector<int> rotations(const qgm_plan *p);
 // Steps of the compiled resident kernel with a static bound on their output:
 // inputs are scaled to maxima at most 1 (gate tables have entries of modulus
 // at most 1), so |out| <= 2^k for k summed variables.  That bound serves as
 // the recorded maximum (no run-time reduction, and a constant scale in the
 // consumer).  Powers of two cost no precision; what a loose bound gives away
-// is headroom towards FP32's smallest values, so it is counted (k bits and one
-// per scaled input, added along the tree) and a step whose bound may be more
-// than 2^48 above its values is measured instead, as is always the final
-// tensor (non-finite values reach it and set the status there).
+// is headroom towards FP32's smallest values, as the consumer multiplies raw
+// values.
+//
+// The slack is counted along the tree: k bits and one per scaled input (fixed
+// gates have entries of modulus 1: a step's values are sums of phases), and
+// ROTATION_BITS for every parametrised gate, whose table (the plan is kept over
+// new angles) may have entries as small as one likes.  It is an estimate (sums
+// may cancel further, angles be smaller), so it stays far from the range:
+// tensors are measured instead such that no step's output, and no step's inputs
+// together, have more than SLACK_BITS; of the inputs, the one with the fewest
+// entries that suffices.  Behind a rotation, a product of measured tensors may
+// be small everywhere (large entries of one meeting small ones of the other):
+// a step that reads one measured is itself measured, as is the final tensor
+// (non-finite values reach it and set the status there).
+//
+// Over grids of up to 28 qubits and depths of 8 to 60 the largest product of
+// raw values of any step is above 2^-65 (2^-133, out of range, when only a
+// step's own output was held to 48 bits).
+constexpr int SLACK_BITS = 40, ROTATION_BITS = 8;
 struct StaticBound {
   int k = 0;               // |out| <= 2^k
   bool exp_known = false;  // every input's exponent is known too:
   int exp = 0;             //   the output's, else it is formed at run time
 };
-std::map<int, StaticBound> static_bounds(const ResidentLayout &L);  // by metadata slot
+std::map<int, StaticBound> static_bounds(const qgm_plan *p, const ResidentLayout &L);  // by metadata slot
 // 16-byte chunks of the compiled resident kernel's initial shared memory that
 // hold something (tensor metadata, bitstring-independent leaf rows); the
 // others are written before they are read

@@ -14,10 +14,9 @@
 //
 // Arithmetic follows the generic kernel: per-tensor power-of-two exponents
 // (the producer records max |re|,|im|; the consumer scales by 2^-e), one
-// combined scale per output entry when the inputs' exponents sum to a
-// representable power of two, the inputs rescaled in place otherwise.  Three
-// additions.  Most steps take a static bound as their recorded maximum
-// (static_bounds): their consumers' scales are constants and nothing is
+// combined scale per output entry while raw products stay clear of both ends
+// of FP32's range, the inputs rescaled in place otherwise.  Three additions.
+// Most steps take a static bound as their recorded maximum (static_bounds): their consumers' scales are constants and nothing is
 // measured.  In wide steps a thread forms two or four entries that share
 // loads and addresses (emit_tile).  Shared memory starts from the chunks of a
 // plan image that hold something, built at bind.
@@ -98,11 +97,11 @@ __device__ __forceinline__ void cmac(float2 &a, float2 x, float2 y) {
   a.y = fmaf(x.x, y.y, a.y);
   a.y = fmaf(x.y, y.x, a.y);
 }
-__device__ __forceinline__ void opscale(const Meta *meta, int slot, float &s, int &e, int &esum) {
+__device__ __forceinline__ void opscale(const Meta *meta, int slot, float &s, int &lo, int &hi, int &esum) {
   const unsigned bits = meta[slot].maxbits;
   const int E = (int)((bits >> 23) & 0xff);
   s = 1.f;
-  e = 0;
+  int e = 0;
   // Inf or NaN (E = 0xff) stays unscaled: it reaches the final tensor,
   // whose check sets the status
   if (E != 0 && E != 0xff) {
@@ -110,6 +109,8 @@ __device__ __forceinline__ void opscale(const Meta *meta, int slot, float &s, in
     if (e > 126) e = 126;
     s = __int_as_float((127 - e) << 23);
   }
+  lo += min(e, 0);
+  hi += max(e, 0);
   esum += e + meta[slot].exp;
 }
 )";
@@ -371,30 +372,84 @@ void emit_body(std::ostringstream &o, const qgm_plan *p, const ResidentLayout &L
 
 }  // namespace
 
-std::map<int, StaticBound> static_bounds(const ResidentLayout &L) {
-  constexpr int kMost = 48;  // bits a bound may lie above the values
+std::vector<int> rotations(const qgm_plan *p) {
+  std::vector<int> n(p->sim.tensors.size(), 0);
+  for (size_t li = 0; li < p->leaves.size(); ++li)
+    for (int fi : p->leaves[li].members) n[li] += p->model.gates[p->model.factors[fi].gate].kind == QGM_GATE_RXY;
+  for (const StepRec &st : p->sim.steps)
+    for (int id : st.inputs) n[st.out] += n[id];
+  return n;
+}
+
+std::map<int, StaticBound> static_bounds(const qgm_plan *p, const ResidentLayout &L) {
   std::map<int, StaticBound> bound;
-  std::map<int, int> loose;  // metadata slot -> bits
-  for (const RStep &r : L.steps) {
+  struct Slack {
+    int bits;
+    int64_t entries;
+  };
+  std::map<int, Slack> loose;  // by metadata slot
+  const std::vector<int> rot = rotations(p);
+  for (size_t q = 0; q < L.steps.size(); ++q) {
+    const RStep &r = L.steps[q];
+    const StepRec &st = p->sim.steps[L.src_step[q]];
+    const int64_t entries = ((int64_t)1 << r.w_out) * (r.batched_out ? L.chunk : 1);
+    // slack of the leaves and of the inputs with a static bound; inputs scaled
+    int leaf = 0, slack = 0, scaled = 0;
+    for (int i = 0; i < r.m; ++i) {
+      if (r.in[i].meta < 0) leaf += ROTATION_BITS * rot[st.inputs[i]];
+      else ++scaled;
+      if (bound.count(r.in[i].meta)) slack += loose[r.in[i].meta].bits;
+    }
+    // the smallest input whose slack leaves at most `most` without it, the
+    // loosest where there is none (-1: no input has slack)
+    auto pick = [&](int most) {
+      int best = -1;
+      bool enough = false;
+      for (int i = 0; i < r.m; ++i) {
+        if (!bound.count(r.in[i].meta)) continue;
+        const Slack &s = loose[r.in[i].meta];
+        const bool e = slack - s.bits <= most;
+        const bool better = best < 0 || e > enough ||
+                            (e == enough && (e ? s.entries < loose[r.in[best].meta].entries
+                                               : s.bits > loose[r.in[best].meta].bits));
+        if (better) {
+          best = i;
+          enough = e;
+        }
+      }
+      return best;
+    };
+    auto measure = [&](int i) {
+      slack -= loose[r.in[i].meta].bits;
+      bound.erase(r.in[i].meta);
+    };
+    while (slack > 0 && leaf + slack > SLACK_BITS) measure(pick(SLACK_BITS - leaf));
+    if (r.out_meta == L.final_meta) continue;
+    const int own = r.k + scaled + leaf;
+    if (own + slack > SLACK_BITS) {
+      // measure one input in place of the output where that is less work
+      const int i = pick(SLACK_BITS - own);
+      if (i < 0 || slack - loose[r.in[i].meta].bits > SLACK_BITS - own || loose[r.in[i].meta].entries >= entries) continue;
+      measure(i);
+    }
     StaticBound s;
     s.k = r.k;
     s.exp_known = true;
-    int bits = r.k;
+    bool ok = true;
     for (int i = 0; i < r.m; ++i) {
       if (r.in[i].meta < 0) continue;
-      bits += 1;
       auto it = bound.find(r.in[i].meta);
       if (it == bound.end()) {
         s.exp_known = false;  // measured at run time
+        ok = ok && rot[st.inputs[i]] == 0;
         continue;
       }
-      bits += loose[r.in[i].meta];
       s.exp_known = s.exp_known && it->second.exp_known;
       s.exp += it->second.k + 1 + it->second.exp;  // scale exponent k+1, recorded exponent
     }
-    if (r.out_meta == L.final_meta || bits > kMost) continue;
+    if (!ok) continue;
     bound[r.out_meta] = s;
-    loose[r.out_meta] = bits;
+    loose[r.out_meta] = {own + slack, entries};
   }
   return bound;
 }
@@ -477,7 +532,8 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
   }
   o << "  __syncthreads();\n";
   // recorded maxima known before the run: steps with a static bound
-  const std::map<int, StaticBound> static_k = static_bounds(L);
+  const std::map<int, StaticBound> static_k = static_bounds(p, L);
+  const std::vector<int> rot = rotations(p);
   // steps in level order; inside a level grouped by first warp, so that
   // each warp's code for the level is contiguous
   std::vector<size_t> emit_order(L.steps.size());
@@ -517,26 +573,29 @@ std::string resident_source(const qgm_plan *p, const ResidentLayout &L, const st
         if (it->second.exp_known) esum_static += it->second.exp;
         else esum_late += " + meta[" + std::to_string(r.in[i].meta) + "].exp";
       }
-    o << "    int es = " << es_static << ", esum = " << esum_static << ";\n";
+    // exponents of the inputs: the negative ones (how small raw products may
+    // be) and the others apart
+    o << "    int lo = 0, hi = " << es_static << ", esum = " << esum_static << ";\n";
     for (int i = 0; i < d.m; ++i) {
       if (r.in[i].meta < 0) continue;
       auto it = static_k.find(r.in[i].meta);
       if (it != static_k.end())
         o << "    const float s" << i << " = __int_as_float(" << (126 - it->second.k) << " << 23);\n";
       else
-        o << "    float s" << i << "; { int e; opscale(meta, " << r.in[i].meta << ", s" << i
-          << ", e, esum); es += e; }\n";
+        o << "    float s" << i << "; opscale(meta, " << r.in[i].meta << ", s" << i << ", lo, hi, esum);\n";
     }
-    // scales: one combined factor per entry when the inputs' exponents sum
-    // to a representable power of two; otherwise the intermediate inputs are
-    // rescaled in place first (each feeds this step only) and the factor is 1
+    // scales: one combined factor per entry while products of raw values stay
+    // clear of both ends of FP32's range (by more where small entries matter,
+    // behind rotations); otherwise the intermediate inputs are rescaled in
+    // place first (each feeds this step only) and the factor is 1
     bool any_meta = false;
+    const int least = rot[p->sim.steps[L.src_step[q]].out] ? -16 : -40;
     for (int i = 0; i < d.m; ++i) any_meta |= r.in[i].meta >= 0;
     o << "    float comb = 1.f;\n";
-    if (any_meta && !any_dynamic && es_static >= -120 && es_static <= 120) {
+    if (any_meta && !any_dynamic && es_static <= 60) {
       o << "    comb = __int_as_float(" << (127 - es_static) << " << 23);\n";
     } else if (any_meta) {
-      o << "    if (es >= -120 && es <= 120) comb = __int_as_float((127 - es) << 23);\n";
+      o << "    if (lo >= " << least << " && hi <= 60) comb = __int_as_float((127 - lo - hi) << 23);\n";
       o << "    else {\n";
       for (int i = 0; i < d.m; ++i) {
         if (r.in[i].meta < 0) continue;

@@ -589,6 +589,16 @@ __global__ void __launch_bounds__(STEP_THREADS)
   record_max(lmax, meta, d.out_meta);
 }
 
+// One factor on a step's sum, 2^-(e_1 + .. + e_m), gives the same values as
+// scaling every input by its 2^-e_i (powers of two) while no product of
+// unscaled values leaves FP32's range.  At the top their exponents bound it;
+// at the bottom entries far below their tensor's maximum (rotations by small
+// angles) count as well, so next to nothing is given away there: in circuits
+// of ordinary angles the negative exponents of a step's inputs sum to -5 at
+// least (with -60 allowed, 4x5 with five layers of rotations by 6e-6 was off
+// by 0.5%).  es, big: sums of e and |e| over the inputs.
+__device__ __forceinline__ bool one_factor(int es, int big) { return big - es <= 2 * 8 && big + es <= 2 * 60; }
+
 // Index from packed runs (see PIn).
 __device__ __forceinline__ int64_t run_index64(const uint32_t *run, int n, uint32_t x) {
   int64_t r = 0;
@@ -714,8 +724,7 @@ __global__ void __launch_bounds__(STEP_THREADS, 3)
     meta[d.out_meta].exp = e[0] + e[1] + (d.in[0].meta >= 0 ? meta[d.in[0].meta].exp : 0) +
                            (d.in[1].meta >= 0 ? meta[d.in[1].meta].exp : 0);
   __syncthreads();
-  // one factor on each sum, as prog_comb
-  const bool one = (e[0] < 0 ? -e[0] : e[0]) + (e[1] < 0 ? -e[1] : e[1]) <= 60;
+  const bool one = one_factor(e[0] + e[1], abs(e[0]) + abs(e[1]));
   const float lmax = one ? reg_items<TM, TN, false>(d, ws, tab, scale, __int_as_float((127 - e[0] - e[1]) << 23), Bp)
                          : reg_items<TM, TN, true>(d, ws, tab, scale, 1.f, Bp);
   record_max(lmax, meta, d.out_meta);
@@ -944,9 +953,8 @@ __global__ void __launch_bounds__(256, NEST ? 1 : 2)
   }
   if (blockIdx.x == 0 && tid == 0) meta[d.out_meta].exp = esum;
   __syncthreads();
-  // one factor on each sum, as prog_comb
   float lmax;
-  if (big <= 60) lmax = mm_tiles<MGB, NGB, NEST, false>(d, ws, mms, tab, scale, __int_as_float((127 - es) << 23), Bp);
+  if (one_factor(es, big)) lmax = mm_tiles<MGB, NGB, NEST, false>(d, ws, mms, tab, scale, __int_as_float((127 - es) << 23), Bp);
   else lmax = mm_tiles<MGB, NGB, NEST, true>(d, ws, mms, tab, scale, 1.f, Bp);
   record_max(lmax, meta, d.out_meta);
 }
@@ -1128,13 +1136,12 @@ __device__ __forceinline__ int prog_scale_exp(uint32_t bits) {
   return E == 0xff || E == 0 ? 0 : (E - 126 > 126 ? 126 : E - 126);
 }
 
-// The factor on the sum: 2^-(e_1 + .. + e_m) gives the same values as scaling
-// every input (powers of two) while no product of unscaled inputs leaves
-// FP32's range; 0 where that is not sure (exponents above 60 in all).
+// The factor on the sum; 0 where the inputs have to be scaled one by one
+// (one_factor).
 __device__ __forceinline__ float prog_comb(ProgMeta q) {
   const int e = prog_scale_exp(q.bits);
   const int es = __reduce_add_sync(0xffffffffu, e), big = __reduce_add_sync(0xffffffffu, e < 0 ? -e : e);
-  return big <= 60 ? __int_as_float((127 - es) << 23) : 0.f;
+  return one_factor(es, big) ? __int_as_float((127 - es) << 23) : 0.f;
 }
 
 // Items [i0, i1) of a step of M inputs, U terms in flight per thread.  PAIR:

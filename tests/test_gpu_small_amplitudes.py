@@ -57,6 +57,18 @@ def test_small_rotations(q, rows, cols, layers, theta, executor):
         assert np.max(np.abs(a - ref)) < 1e-5 * abs(ref), (a, ref)
 
 
+def test_tiny_rotations_stepwise(q):
+    # inputs near 2^-50 each and table entries of 2^-18: in range one by one
+    # with every input scaled first, not as raw products (2^-340 in all)
+    c = _near_identity(4, 5, 5, 6.3e-6, 3)
+    x = (1 << c.n) - 1
+    p = q.Plan(q.Model(q.Circuit.from_gates(c.n, c.gates)), batch=4, executor=q.EXEC_STEPWISE).bind()
+    ref = vec.amplitude(c, x)
+    a = p.amplitudes_host(np.full(4, x, dtype=np.uint64))
+    assert p.status() == 0
+    assert np.max(np.abs(a - ref)) < 1e-5 * abs(ref), (a, ref)
+
+
 @pytest.mark.parametrize("executor", EXECS)
 @pytest.mark.parametrize("rows,cols,depth,seed", [(4, 4, 28, 1), (4, 4, 28, 4), (4, 5, 23, 0), (4, 4, 36, 2), (3, 4, 40, 0)])
 def test_deep_circuits_of_fixed_gates(q, rows, cols, depth, seed, executor):

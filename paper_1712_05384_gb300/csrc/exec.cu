@@ -2361,14 +2361,18 @@ __global__ void __launch_bounds__(SET_THREADS) k_xeb(const double2 *a, int64_t B
   cluster_sync();  // a CTA's shared memory stays until it has been read
 }
 
-// Inclusive scan over a block of 256 of one value per thread; *sum = total.
+// Scan over a block of 256 of one value per thread: the sum of the values
+// before a thread's own; *sum = total.
 __device__ __forceinline__ double block_scan(double v, double *sum) {
   __shared__ double wsum[8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double ex = 0;
   for (int o = 1; o < 32; o <<= 1) {
     const double u = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += u;
   }
+  ex = __shfl_up_sync(0xffffffffu, v, 1);
+  if (lane == 0) ex = 0;
   __syncthreads();  // the previous call's wsum is read
   if (lane == 31) wsum[wid] = v;
   __syncthreads();
@@ -2379,14 +2383,50 @@ __device__ __forceinline__ double block_scan(double v, double *sum) {
     all += wsum[w];
   }
   *sum = all;
-  return before + v;
+  return before + ex;
+}
+
+// Sums of p as their bits: non-negative values order like them, NaN above all
+// (integer maxima, as FP64 arithmetic is scarce).
+typedef unsigned long long SumBits;
+__device__ __forceinline__ SumBits sum_bits(double v) { return (SumBits)__double_as_longlong(v); }
+
+// Maximum of `first` and the values before a thread's own, over a block of
+// 256; *all = that of every value.
+__device__ __forceinline__ SumBits block_max_scan(SumBits v, SumBits first, SumBits *all) {
+  __shared__ SumBits wmax[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const SumBits u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v = max(u, v);
+  }
+  SumBits ex = __shfl_up_sync(0xffffffffu, v, 1);
+  if (lane == 0) ex = first;
+  __syncthreads();  // the previous call's wmax is read
+  if (lane == 31) wmax[wid] = v;
+  __syncthreads();
+  SumBits before = max(first, ex), m = first;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w < wid) before = max(before, wmax[w]);
+    m = max(m, wmax[w]);
+  }
+  *all = m;
+  return before;
 }
 
 // Cumulative sums of p_j = |a_j|^2 over chunks of CDF_CHUNK values, one block
 // each, on all SMs (one cluster would be bound by its FP64 units): the
 // chunk's total goes to the chunk's first entry of cdf, one block turns these
-// into the sums before each chunk, and each block then reads its own and
-// writes its chunk.
+// into the sums before and after each chunk, and each block then reads its own
+// and writes its chunk.
+//
+// Sums formed in a tree are not monotone to the last bit.  A search needs an
+// order, and an entry of probability zero must have its predecessor's sum, or
+// it could be drawn: every sum is therefore the largest of the tree's sums up
+// to it over the entries (chunks) that are not zero, held below the chunk's
+// last sum, which the chunk's last such entry takes and the next chunk starts
+// from.
 constexpr int CDF_CHUNK = 512;
 __device__ __forceinline__ double p_of(const double2 *a, int64_t j, int64_t t) {
   return j < t ? a[j].x * a[j].x + a[j].y * a[j].y : 0.0;
@@ -2403,25 +2443,48 @@ __global__ void __launch_bounds__(256) k_cdf_before(int64_t n, double *cdf) {
     const int64_t c = c0 + threadIdx.x;
     const double v = c < n ? cdf[c * CDF_CHUNK] : 0.0;
     double all;
-    const double s = block_scan(v, &all);
-    if (c < n) cdf[c * CDF_CHUNK] = run + (s - v);
-    run += all;
+    const double s = run + (block_scan(v, &all) + v);
+    const SumBits own = sum_bits(v != 0.0 ? s : run);
+    SumBits last;
+    const SumBits before = block_max_scan(own, sum_bits(run), &last);
+    if (c < n) cdf[c * CDF_CHUNK] = __longlong_as_double(before);
+    if (c < n - 1) cdf[c * CDF_CHUNK + 1] = __longlong_as_double(max(before, own));  // (all but the last chunk are full)
+    run = __longlong_as_double(last);
   }
 }
 __global__ void __launch_bounds__(256) k_cdf_chunks(const double2 *a, int64_t t, double *cdf) {
-  const int64_t j = (int64_t)blockIdx.x * CDF_CHUNK + 2 * threadIdx.x;
+  __shared__ int wlast[8];
+  const int tid = threadIdx.x;
+  const int64_t j0 = (int64_t)blockIdx.x * CDF_CHUNK, j = j0 + 2 * tid;
   const double p0 = p_of(a, j, t), p1 = p_of(a, j + 1, t);
-  const double run = cdf[(int64_t)blockIdx.x * CDF_CHUNK];
-  double all;
-  const double s = run + block_scan(p0 + p1, &all);  // its barriers order the read before the writes
-  if (j < t) cdf[j] = s - p1;
-  if (j + 1 < t) cdf[j + 1] = s;
+  const bool full = blockIdx.x + 1 < gridDim.x;
+  const double run = cdf[j0];
+  const SumBits start = sum_bits(run), end = sum_bits(full ? cdf[j0 + 1] : 0.0);
+  // the chunk's last entry that is not zero
+  const int wl = __reduce_max_sync(0xffffffffu, p1 != 0.0 ? 2 * tid + 1 : p0 != 0.0 ? 2 * tid : -1);
+  if ((tid & 31) == 0) wlast[tid >> 5] = wl;
+  double total;
+  const double ex = block_scan(p0 + p1, &total);  // its barriers order the reads before the writes
+  int last = -1;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) last = max(last, wlast[w]);
+  SumBits c0 = sum_bits(run + (ex + p0)), c1 = sum_bits(run + (ex + p0 + p1)), all;
+  if (full) {
+    c0 = 2 * tid == last ? end : min(c0, end);
+    c1 = 2 * tid + 1 == last ? end : min(c1, end);
+  }
+  if (p0 == 0.0) c0 = start;
+  if (p1 == 0.0) c1 = start;
+  const SumBits before = block_max_scan(max(c0, c1), start, &all);
+  c0 = max(before, c0);
+  if (j < t) cdf[j] = __longlong_as_double(c0);
+  if (j + 1 < t) cdf[j + 1] = __longlong_as_double(max(c0, c1));
 }
 
 // Draw i: u = the i-th output of SplitMix64(seed) (counter form: the state
 // after i + 1 golden-ratio increments, then the two mixing rounds), top 53
-// bits; index = first j with cdf[j] / total > u.  The search runs on
-// cdf[j] > u * total, its first levels over SAMPLE_COARSE entries staged in
+// bits; index = first j with cdf[j] / total > u (cdf never falls, and rises at
+// entries that are not zero only).  The search runs on cdf[j] > u * total, its first levels over SAMPLE_COARSE entries staged in
 // shared memory (a search in global memory is a chain of L2 latencies), and
 // the defining quotient is checked around the place found.
 constexpr int SAMPLE_COARSE = 512;

@@ -64,3 +64,27 @@ def test_irregular_probabilities(q):
     a[99] = np.nan
     st = q._lib.xeb_stats(_device(a), 5000, 20, torch.zeros(4, dtype=torch.float64, device="cuda"))
     assert np.isnan(st["cross_entropy"]) and np.isnan(st["mean_Np"])
+
+
+@pytest.mark.parametrize("t", [1, 2, 511, 512, 513, 1024, 1025, 5000, 131073, 300001])
+def test_cumulative_sums_are_ordered(q, t):
+    # never falling, and an entry of probability zero has its predecessor's
+    # sum, so that no draw can find it: zeros strewn about and in stretches
+    # over the ends of the kernels' chunks, values of every size
+    rng = np.random.default_rng(t)
+    a = _set(t, t) * 2.0 ** rng.integers(-30, 1, t)
+    a[rng.random(t) < 0.4] = 0
+    for s in range(0, t, 512 * 7):
+        a[max(0, s - 300):s + 700] = 0
+    if t > 2000:
+        a[-3:] = 0
+    a[t // 2] = 1e-3
+    p = a.real * a.real + a.imag * a.imag
+    cdf = torch.zeros(t, dtype=torch.float64, device="cuda")
+    idx = torch.full((20000,), -1, dtype=torch.int64, device="cuda")
+    q._lib.sample_from_set(_device(a), t, 20000, 7, cdf, idx)
+    c = np.concatenate([[0.0], cdf.cpu().numpy()])
+    step = np.diff(c)
+    assert np.all(step >= 0) and np.all(step[p == 0] == 0)
+    assert np.max(np.abs(c[1:] - np.cumsum(p))) <= 1e-12 * c[-1]
+    assert np.all(p[idx.cpu().numpy()] > 0)

@@ -171,13 +171,15 @@ __device__ __forceinline__ int64_t run_bit(const InDesc &in, int b) {
 // Increment tables of one launch (every input index is linear in the bits of
 // the union index): when a thread's row counter carries into bit t the byte
 // address of input i moves by rowtab[i][t]; when its term counter carries into
-// bit t, by etab[i][t].  Rows advance by 2^r0, terms by 2^lt.
-constexpr int ROWTAB = 32, ETAB = 16;
+// bit t, by etab[i][t].  Rows advance by 2^r0, terms by 2^lt.  A forward step
+// sums at most ETAB variables, an adjoint step (k_step_batched) at most ADJTAB.
+constexpr int ROWTAB = 32, ETAB = 16, ADJTAB = ADJOINT_K;
 
+template <int NE>
 __device__ void build_tables(const StepDesc &d, int r0, int lt, int Bp, int64_t (*rowtab)[ROWTAB],
-                             int64_t (*etab)[ETAB], int tid, int nthreads) {
-  for (int x = tid; x < MAXIN * (ROWTAB + ETAB); x += nthreads) {
-    const int i = x / (ROWTAB + ETAB), t = x - i * (ROWTAB + ETAB);
+                             int64_t (*etab)[NE], int tid, int nthreads) {
+  for (int x = tid; x < MAXIN * (ROWTAB + NE); x += nthreads) {
+    const int i = x / (ROWTAB + NE), t = x - i * (ROWTAB + NE);
     if (i >= d.m) continue;
     const InDesc &in = d.in[i];
     const int64_t unit = in.batched ? (int64_t)Bp * 8 : 8;
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(512)
     k_step_batched(char *ws, const StepDesc d, Meta *meta, Header *hdr, int Bp, int logP) {
   __shared__ float4 part[512];
   __shared__ int64_t rowtab[MAXIN][ROWTAB];
-  __shared__ int64_t etab[MAXIN][ETAB];
+  __shared__ int64_t etab[MAXIN][ADJTAB];
   const int tx = threadIdx.x, ty = threadIdx.y, T = blockDim.y;
   const int tid = ty * STEP_THREADS + tx;
   // wide batch (logP < 0): a row spans gridDim.x blocks of pairs; narrow

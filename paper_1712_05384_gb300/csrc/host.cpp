@@ -1961,6 +1961,10 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
         d.k = (int)summed.size();
         d.w_out = (int)it.vars.size();
         d.batched_out = 1;
+        if (d.k > ADJOINT_K) {
+          set_error("qgm_plan_order: an adjoint step sums %d variables, at most %d are possible", d.k, ADJOINT_K);
+          return QGM_ERR_ARG;
+        }
         adj_off[id] = gtake(pow2(d.w_out) * Bp * 8);
         adj_meta[id] = next_meta++;
         d.out_off = adj_off[id];

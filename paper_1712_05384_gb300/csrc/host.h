@@ -51,6 +51,7 @@ struct Model {
 // ------------------------------------------------------------------- plan
 constexpr int MAXIN = 8;    // tensors multiplied in one step
 constexpr int MAXRUN = 16;  // contiguous bit runs of an index map
+constexpr int ADJOINT_K = 30;  // most variables an adjoint step sums
 constexpr int MAXLEAFV = 4; // variables of a leaf factor (internal+slice+output)
 constexpr int RES_WARPS = 8; // warps of a resident CTA
 

@@ -166,3 +166,33 @@ def test_gradient_needs_gradient_plan(q):
     bits = torch.zeros(4, dtype=torch.int64, device="cuda")
     with pytest.raises(q.QgmError):
         plan.amplitude_grad(bits, d, d)
+
+
+def test_long_adjoint_sums_over_wide_tensors(q):
+    # an adjoint step that sums 18 variables and reads a tensor of 2 GiB runs
+    # on its own (its offsets pass the step program's): the gradient of one
+    # batch of 512 against the sum of the gradients of eight of 64, whose
+    # steps all run in the program
+    rows, cols, depth, B, part = 4, 6, 34, 512, 64
+    m = q.Model(q.Circuit.grid(rows, cols, depth, 0, True))
+    if torch.cuda.mem_get_info()[0] < 48 << 30:
+        pytest.skip("needs 48 GiB")
+    bits = qi.bitstrings(rows * cols, B, 1)
+    d_bits = torch.from_numpy(bits.astype(np.int64)).cuda()
+    w = np.random.default_rng(3).standard_normal(2 * B)
+    d_w = torch.from_numpy(w).cuda()
+    n = 2 * len(m.circuit.param_gates())
+    grads = []
+    for size in (B, part):
+        p = q.Plan(m, batch=size, gradients=True, executor=q.EXEC_STEPWISE).bind()
+        total = np.zeros(n)
+        for b0 in range(0, B, size):
+            g = torch.zeros(n, dtype=torch.float64, device="cuda")
+            p.amplitude_grad(d_bits[b0:b0 + size].clone(), d_w[2 * b0:2 * (b0 + size)].clone(), g)
+            total += g.cpu().numpy()
+        assert p.status() == 0
+        grads.append(total)
+        del p
+        torch.cuda.empty_cache()
+    # two FP32 evaluations of the same sums, each within 1e-5 of the largest
+    assert np.max(np.abs(grads[0] - grads[1])) <= 2e-5 * np.max(np.abs(grads[1]))

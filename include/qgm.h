@@ -433,6 +433,14 @@ int qgm_measure_fp32_peak(double *tflops, void *stream);
  * context stays usable either way.  Host int32 out; synchronises. */
 int qgm_selftest_wait_timeout(int64_t limit_ns, int32_t arrive, int32_t *status_out, void *stream);
 
+/* The same for the waits between the steps that share a launch (a segment of
+ * the stepwise pass): one segment of a bound plan runs without the step it
+ * starts with, so that those which read it wait in vain, for limit_ns (1 us ..
+ * 2 s; a pass allows a second and more).  *status_out = QGM_ERR_TIMEOUT (read
+ * and cleared); the plan's next pass is a whole one.  QGM_ERR_ARG where no two
+ * steps of the plan share a launch that way.  Synchronises. */
+int qgm_selftest_program_timeout(qgm_plan *p, int64_t limit_ns, int32_t *status_out, void *stream);
+
 /* Executor chosen at bind time:/* Executor chosen at bind time: *kind (QGM_EXEC_STEPWISE, _RESIDENT or
  * _COMPILED), the bitstrings per CTA *chunk and the dynamic shared memory per
  * CTA (resident and compiled). */

@@ -101,6 +101,7 @@ _SIGS = {
     "qgm_plan_profile_gemm": [_P, _P, C.c_int64, _P, C.POINTER(C.c_float), C.POINTER(C.c_float), _P],
     "qgm_measure_fp32_peak": [C.POINTER(C.c_double), _P],
     "qgm_selftest_wait_timeout": [C.c_int64, C.c_int32, _I32P, _P],
+    "qgm_selftest_program_timeout": [_P, C.c_int64, _I32P, _P],
     "qgm_plan_step_stats": [_P, C.POINTER(C.c_uint32), _I32P, C.c_int64, _P],
     "qgm_plan_free": [_P],
     "qgm_plan_bind": [_P, _P, C.c_size_t, _P],
@@ -523,6 +524,14 @@ def selftest_wait_timeout(limit_ns, arrive=False, stream=None):
     the kernel wrote (QGM_ERR_TIMEOUT or 0)."""
     st = C.c_int32(1)
     check(lib().qgm_selftest_wait_timeout(int(limit_ns), 1 if arrive else 0, C.byref(st), _stream(stream)))
+    return st.value
+
+
+def selftest_program_timeout(plan, limit_ns, stream=None):
+    """Run a segment of the plan's stepwise pass without the step others wait
+    for; returns the status (QGM_ERR_TIMEOUT)."""
+    st = C.c_int32(1)
+    check(lib().qgm_selftest_program_timeout(plan._h, int(limit_ns), C.byref(st), _stream(stream)))
     return st.value
 
 

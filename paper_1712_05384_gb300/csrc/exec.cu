@@ -1054,8 +1054,8 @@ __global__ void __launch_bounds__(256)
 // Units are numbered producers first, and a CTA takes one unit at a time: the
 // unfinished unit of the lowest number never waits for an unfinished one, so
 // the segment always advances, whatever the number of resident CTAs.  Waits
-// are bounded all the same (one second); one that runs out raises the abort
-// word, every CTA leaves, and the status is QGM_ERR_TIMEOUT.
+// are bounded all the same (ProgramOp::wait_ns); one that runs out raises the
+// abort word, every CTA leaves, and the status is QGM_ERR_TIMEOUT.
 //
 // Data written by other CTAs of the launch is read with ordinary loads after
 // an acquire of the counter (no read-only path).
@@ -1067,12 +1067,12 @@ __device__ __forceinline__ int ld_acquire(const int *p) {
   return v;
 }
 
-__device__ __forceinline__ bool prog_wait(const int *done, int need, const int *abort_word) {
+__device__ __forceinline__ bool prog_wait(const int *done, int need, const int *abort_word, uint64_t limit_ns) {
   if (ld_acquire(done) >= need) return true;
   const uint64_t t0 = gtimer();
   while (ld_acquire(done) < need) {
     __nanosleep(40);
-    if (gtimer() - t0 > 1000000000ull || *(const volatile int *)abort_word) return false;
+    if (gtimer() - t0 > limit_ns || *(const volatile int *)abort_word) return false;
   }
   return true;
 }
@@ -1271,7 +1271,7 @@ __device__ __forceinline__ uint32_t prog_items_u(const PStep &S, char *ws, const
 
 __global__ void __launch_bounds__(PROG_THREADS, 2)
     k_program(char *ws, const PStep *steps, const PTask *tasks, int n_tasks, int *sync, int ticket, int done0, Header *hdr,
-              int Bp) {
+              int Bp, uint64_t limit_ns) {
   __shared__ PStep desc[2];
   __shared__ int eoff[MAXIN * 256];
   __shared__ uint32_t red[PROG_THREADS / 32];
@@ -1302,7 +1302,7 @@ __global__ void __launch_bounds__(PROG_THREADS, 2)
       }
       bool ok = true;
       if (wid == 0) {
-        if (lane < S.n_deps) ok = prog_wait(sync + done0 + S.dep[lane], S.dep_units[lane], sync);
+        if (lane < S.n_deps) ok = prog_wait(sync + done0 + S.dep[lane], S.dep_units[lane], sync, limit_ns);
         ok = __all_sync(0xffffffffu, ok);
       }
       const int Kt = k < 8 ? 1 << k : 256;
@@ -3296,6 +3296,15 @@ static void launch_accumulate(qgm_plan *p, double2 *d_out, int64_t n_out, int64_
       c.imag(), p->open_in_batch, p->Bp, only ? 1 : 0);
 }
 
+// One segment; ticket: its word among the sync words.
+static void launch_segment(qgm_plan *p, const Program &P, const ProgramOp &op, int ticket, int64_t wait_ns, cudaStream_t st) {
+  char *ws = p->exec->ws;
+  k_program<<<std::min(op.tasks, 2 * p->exec->sms), PROG_THREADS, 0, st>>>(
+      ws, reinterpret_cast<const PStep *>(ws + P.off_steps), reinterpret_cast<const PTask *>(ws + P.off_tasks) + op.task0,
+      op.tasks, reinterpret_cast<int *>(ws + P.off_sync), ticket, (int)P.done_word(),
+      reinterpret_cast<Header *>(ws + p->off_header), p->Bp, (uint64_t)wait_ns);
+}
+
 // Enqueue a step program: its segments, and its large steps on their own (with
 // the tuner's parameters for the forward pass).
 static void launch_program(qgm_plan *p, const Program &P, cudaStream_t st) {
@@ -3304,14 +3313,11 @@ static void launch_program(qgm_plan *p, const Program &P, cudaStream_t st) {
   Header *hdr = reinterpret_cast<Header *>(ws + p->off_header);
   int ticket = 1;  // sync word 0 is the abort word
   for (const ProgramOp &op : P.ops) {
-    if (op.big >= 0) {
+    if (op.big >= 0)
       launch_step_ws(ws, p->exec->sms, p->Bp, P.all[op.big], P.gemms.data(), meta, hdr, st, p->gemm_tc, p->off_planes,
                      p->tc_planes, nullptr, &P == &p->fprog ? &p->tune[op.big] : nullptr);
-    } else {
-      k_program<<<std::min(op.tasks, 2 * p->exec->sms), PROG_THREADS, 0, st>>>(
-          ws, reinterpret_cast<const PStep *>(ws + P.off_steps), reinterpret_cast<const PTask *>(ws + P.off_tasks) + op.task0,
-          op.tasks, reinterpret_cast<int *>(ws + P.off_sync), ticket++, (int)P.done_word(), hdr, p->Bp);
-    }
+    else
+      launch_segment(p, P, op, ticket++, op.wait_ns, st);
   }
 }
 
@@ -4036,6 +4042,38 @@ int qgm_selftest_wait_timeout(int64_t limit_ns, int32_t arrive, int32_t *status_
   CK(cudaMemcpyFromSymbolAsync(status_out, g_selftest_status, sizeof(int32_t), 0, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return QGM_OK;
+}
+
+int qgm_selftest_program_timeout(qgm_plan *p, int64_t limit_ns, int32_t *status_out, void *stream) {
+  int rc = check_bound(p, "qgm_selftest_program_timeout");
+  if (rc) return rc;
+  if (!status_out || limit_ns < 1000 || limit_ns > 2000000000ll) {
+    set_error("qgm_selftest_program_timeout: need status_out and 1 us <= limit_ns <= 2 s");
+    return QGM_ERR_ARG;
+  }
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const Program &P = p->fprog;
+  int ticket = 1;
+  for (const ProgramOp &op : P.ops) {
+    if (op.big >= 0) continue;
+    // the tasks of the segment's first step are left out (the ticket counter
+    // starts behind them) where a step waits for it
+    const PTask &t = P.tasks[op.task0];
+    const PStep &s = P.steps[t.step + t.count - 1];
+    const int skip = P.steps[t.step].n_units;
+    if (s.signal && skip < op.tasks) {
+      launch_leaves(p, reinterpret_cast<const uint64_t *>(p->exec->ws + p->off_bits), 0, st, &P);
+      CK(cudaMemcpyAsync(p->exec->ws + P.off_sync + 4 * (int64_t)ticket, &skip, 4, cudaMemcpyHostToDevice, st));
+      launch_segment(p, P, op, ticket, limit_ns, st);
+      CK(cudaGetLastError());
+      CK(cudaStreamSynchronize(st));
+      *status_out = qgm_status(p, stream);
+      return QGM_OK;
+    }
+    ++ticket;
+  }
+  set_error("qgm_selftest_program_timeout: no step of the plan waits for another in one launch");
+  return QGM_ERR_ARG;
 }
 
 int qgm_measure_fp32_peak(double *tflops, void *stream) {

@@ -233,6 +233,7 @@ struct PTask {
 struct ProgramOp {
   int32_t big;          // >= 0: index of a step launched on its own; -1: a segment
   int32_t task0, tasks; // the segment's tasks
+  int64_t wait_ns;      // longest wait of a unit for another step
 };
 
 struct Program {

@@ -227,6 +227,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
   size_t o = 0;
   for (int ph = 0; ph <= (int)big_of.size(); ++ph) {
     const int task0 = (int)P.tasks.size();
+    double loads = 0;
     for (; o < order.size() && nodes[order[o]].phase == ph; ++o) {
       const int i0 = order[o];
       PTask t{(int)P.steps.size(), 0, 0, 0};
@@ -240,6 +241,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
             s.dep_units[s.n_deps++] = nodes[q].s.n_units;
           }
         for (int r : readers[i]) s.signal |= r != next[i];
+        loads += std::ldexp((double)s.items * s.m, s.k);
         P.steps.push_back(s);
         ++t.count;
       }
@@ -250,10 +252,13 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
       }
     }
     if ((int)P.tasks.size() > task0) {
-      P.ops.push_back({-1, task0, (int)P.tasks.size() - task0});
+      // a wait lasts at most as long as the segment: a second, and a
+      // nanosecond for each of its loads (some hundred times their time), up
+      // to a minute
+      P.ops.push_back({-1, task0, (int)P.tasks.size() - task0, 1000000000 + (int64_t)std::min(loads, 6e10)});
       P.n_segments += 1;
     }
-    if (ph < (int)big_of.size()) P.ops.push_back({big_of[ph], 0, 0});
+    if (ph < (int)big_of.size()) P.ops.push_back({big_of[ph], 0, 0, 0});
   }
 }
 

@@ -134,3 +134,20 @@ def test_outputs_are_written_whole(q, rows, cols, depth, div):
             assert p.status() == 0 and np.all(np.isnan(a[B:].real))
             e = errmeasure.measures(a[:B], ref[:B], c.n)
             assert e["rel"] < TOL and e["abs"] < TOL, e
+
+
+@pytest.mark.parametrize("rows,cols,depth,B", [(3, 3, 10, 5), (4, 6, 30, 4)])
+def test_wait_between_steps_gives_up(q, rows, cols, depth, B):
+    # a segment whose first step never runs: the units that wait for it give
+    # up after 2 ms and the launch ends with a status; the next passes (one
+    # launch after another, or a graph) are whole
+    c = qi.grid_circuit(rows, cols, depth, 3)
+    p = q.Plan(q.Model(q.Circuit.grid(rows, cols, depth, 3)), batch=B, executor=q.EXEC_STEPWISE).bind()
+    bits = qi.bitstrings(c.n, B, 4)
+    before = p.amplitudes_host(bits)
+    for _ in range(2):
+        assert q._lib.selftest_program_timeout(p, 2_000_000) == -4
+        assert p.status() == 0
+        assert np.array_equal(p.amplitudes_host(bits), before) and p.status() == 0
+    with pytest.raises(q.QgmError):
+        q._lib.selftest_program_timeout(p, 10)  # limit out of range

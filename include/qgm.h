@@ -251,7 +251,8 @@ typedef struct {
   int64_t n_slices;           /* 2^n_slice_vars */
   int64_t max_tensor_entries; /* largest intermediate, complex64 entries */
   int64_t workspace_bytes;    /* device workspace qgm_plan_bind needs */
-  int64_t arena_bytes;        /* of which live intermediates */
+  int64_t arena_bytes;        /* of which live intermediates: the most that are at
+                                 once, however the steps are launched */
   double bytes_per_slice;     /* algorithmic bytes (inputs read + output written) */
   double flops_per_slice;     /* algorithmic real flops of the products and sums */
   double max_step_bytes;      /* algorithmic bytes of the largest step */

@@ -1335,12 +1335,72 @@ int plan_set_params(qgm_plan *p, const double *params) {
   return QGM_OK;
 }
 
-// The forward pass as a step program.  Small steps run in any order their
-// inputs allow, so their outputs leave the arena (whose reuse of memory
-// assumes the plan's order) for a region of their own, where a block is only
-// reused along a tensor's descent: what step s frees goes to the one step
-// that reads s's output, which cannot start before s is done.
-static void forward_program(qgm_plan *p) {
+// Places the tensors of the forward pass for the phases of its program: times
+// are phases (segment, then large step), a tensor lives from its producer's to
+// its one reader's.  Inside a segment the steps run in any order their inputs
+// allow, so there two tensors share memory only along a tensor's descent: what
+// a step reads last may be written by the steps its output leads to.  off: the
+// places, from 0 on; returns the extent.
+static int64_t place_tensors(const qgm_plan *p, const Program &P, std::vector<int64_t> &off) {
+  const SimResult &S = p->sim;
+  const int n = (int)P.all.size();
+  // the elimination is a tree: first[s] .. s in reader order is its subtree
+  // (post[s]: place in a post-order, lo[s]: the lowest place below s)
+  std::vector<int> reader(n, -1), post(n, -1), lo(n, 0), size(n, 1);
+  for (int s = 0; s < n; ++s)
+    for (int q : P.prod[s])
+      if (q >= 0) {
+        reader[q] = s;
+        size[s] += size[q];
+      }
+  // places from the roots down (readers come after their inputs in the order)
+  int next = 0;
+  std::vector<int> fill(n, 0);
+  for (int s = n - 1; s >= 0; --s) {
+    if (reader[s] < 0) {
+      lo[s] = next;
+      next += size[s];
+    } else {
+      lo[s] = fill[reader[s]];
+      fill[reader[s]] += size[s];
+    }
+    post[s] = lo[s] + size[s] - 1;
+    fill[s] = lo[s];
+  }
+  auto below = [&](int a, int b) { return a != b && lo[b] <= post[a] && post[a] < post[b]; };  // b needs a
+  // step a is over before step b starts
+  auto before = [&](int a, int b) {
+    const int ta = P.time(a), tb = P.time(b);
+    return ta < tb || (ta == tb && below(a, b));
+  };
+  std::vector<int> idx(n);
+  std::iota(idx.begin(), idx.end(), 0);
+  auto bytes = [&](int s) { return (S.tensors[S.steps[s].out].entries * 8 + 255) & ~int64_t(255); };
+  std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return bytes(a) > bytes(b); });
+  off.assign(n, 0);
+  int64_t extent = 0;
+  std::vector<int> by_off;  // placed steps, lowest place first
+  for (int s : idx) {
+    const int64_t need = bytes(s);
+    int64_t at = 0;
+    for (int q : by_off) {
+      if (off[q] >= at + need) break;
+      if ((reader[q] >= 0 && before(reader[q], s)) || (reader[s] >= 0 && before(reader[s], q))) continue;
+      at = std::max(at, off[q] + bytes(q));
+    }
+    off[s] = at;
+    extent = std::max(extent, at + need);
+    by_off.insert(std::upper_bound(by_off.begin(), by_off.end(), s, [&](int a, int b) { return off[a] < off[b]; }), s);
+  }
+  return extent;
+}
+
+// The forward pass as a step program.  Its tensors have places of their own
+// over those of the plan's order (which passes step by step use: never both at
+// once).  Small steps side by side keep more tensors live than the plan's
+// order does; where that would pass the memory budget, segments are cut short,
+// down to a step each at the plan's own places.
+static void forward_program(qgm_plan *p, int64_t budget) {
   const SimResult &S = p->sim;
   const int n = (int)p->steps.size();
   Program &P = p->fprog;
@@ -1349,51 +1409,34 @@ static void forward_program(qgm_plan *p) {
   P.prod.assign(n, {});
   std::vector<int> producer(S.tensors.size(), -1);
   for (int s = 0; s < n; ++s) producer[S.steps[s].out] = s;
-  using Block = std::pair<int64_t, int64_t>;  // size, offset
-  std::vector<std::vector<Block>> pool(n);
-  std::vector<int64_t> off(S.tensors.size());
-  std::vector<char> moved(S.tensors.size(), 0);
-  for (size_t t = 0; t < S.tensors.size(); ++t) off[t] = S.tensors[t].off;
-  int64_t top = p->ws_bytes - 256;
-  for (int s = 0; s < n; ++s) {
-    const StepRec &st = S.steps[s];
-    StepDesc &d = P.all[s];
-    for (size_t i = 0; i < st.inputs.size(); ++i) {
-      const int q = producer[st.inputs[i]];
-      P.prod[s].push_back(q);
-      d.in[i].off = off[st.inputs[i]];
-      if (q >= 0) {
-        pool[s].insert(pool[s].end(), pool[q].begin(), pool[q].end());
-        pool[q].clear();
+  for (int s = 0; s < n; ++s)
+    for (int id : S.steps[s].inputs) P.prod[s].push_back(producer[id]);
+  std::vector<int64_t> off;
+  for (int run : {0, 16, 1, -1}) {
+    const bool own = run >= 0;  // else the plan's places
+    program_phases(P, p->Bp, own ? run : 1);
+    int64_t extent = S.arena_peak;
+    if (own) extent = place_tensors(p, P, off);
+    else
+      for (int s = 0; s < n; ++s) off[s] = p->steps[s].out_off - p->off_arena;
+    for (int s = 0; s < n; ++s) {
+      StepDesc &d = P.all[s];
+      d.out_off = p->off_arena + off[s];
+      for (int i = 0; i < d.m; ++i)
+        if (P.prod[s][i] >= 0) d.in[i].off = p->off_arena + off[P.prod[s][i]];
+      if (d.gemm >= 0) {
+        GemmDesc &g = P.gemms[d.gemm];
+        g.a_off = d.in[0].off;
+        g.b_off = d.in[1].off;
+        g.o_off = d.out_off;
       }
     }
-    if (!program_alone(d, p->Bp)) {
-      const int64_t bytes = (S.tensors[st.out].entries * 8 + 255) & ~int64_t(255);
-      int best = -1;
-      for (int b = 0; b < (int)pool[s].size(); ++b)
-        if (pool[s][b].first >= bytes && (best < 0 || pool[s][b].first < pool[s][best].first)) best = b;
-      if (best >= 0) {
-        off[st.out] = pool[s][best].second;
-        pool[s][best].first -= bytes;
-        pool[s][best].second += bytes;
-      } else {
-        off[st.out] = top;
-        top += bytes;
-      }
-      moved[st.out] = 1;
-      d.out_off = off[st.out];
-    }
-    for (int id : st.inputs)
-      if (moved[id]) pool[s].push_back({(S.tensors[id].entries * 8 + 255) & ~int64_t(255), off[id]});
-    if (d.gemm >= 0) {
-      GemmDesc &g = P.gemms[d.gemm];
-      g.a_off = off[st.inputs[0]];
-      g.b_off = off[st.inputs[1]];
-    }
+    build_program(P, p->Bp, p->off_meta, own);
+    p->live_bytes = std::max(S.arena_peak, extent + P.tmp_bytes);
+    if (p->live_bytes <= budget) break;
   }
-  p->f_final_off = off[S.final_tensor];
-  build_program(P, p->Bp, p->off_meta, std::vector<char>(n, 0));
-  p->ws_bytes = place_program(P, top) + 256;
+  p->f_final_off = producer[S.final_tensor] >= 0 ? P.all[producer[S.final_tensor]].out_off : p->final_off;
+  p->prog_end = p->off_arena + ((std::max(S.arena_peak, p->live_bytes - P.tmp_bytes) + 255) & ~int64_t(255));
 }
 
 // The gradient pass (forward keeping every intermediate, then the adjoint
@@ -1413,7 +1456,8 @@ static void gradient_program(qgm_plan *p) {
     }
     producer[P.all[s].out_off] = (int)s;
   }
-  build_program(P, p->Bp, p->off_meta, std::vector<char>(P.all.size(), 0));
+  program_phases(P, p->Bp, 0);
+  build_program(P, p->Bp, p->off_meta, true);
   p->ws_bytes = place_program(P, p->ws_bytes - 256) + 256;
 }
 
@@ -1886,17 +1930,18 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
     if (s1 - s0 >= 2) p->plain_group[s0] = (int32_t)(s1 - s0);
     s0 = s1 > s0 ? s1 : s0 + 1;
   }
-  // the split operand planes of the largest tensor-core step, after the arena
+  // the split operand planes of the largest tensor-core step, after the
+  // tensors (of either layout), then the step program's tables
   p->ws_fwd_bytes = p->ws_bytes;
+  forward_program(p, budget);
   p->planes_bytes = 0;
   if (p->gemm_tc)
     for (const GemmDesc &g : p->gemms) {
       const TcCfg c = tc_config(g, (int)Bp, p->tc_planes);
       if (c.ok) p->planes_bytes = std::max(p->planes_bytes, c.bytesM + c.bytesN);
     }
-  p->off_planes = p->ws_bytes - 256;
-  p->ws_bytes = p->off_planes + p->planes_bytes + 256;
-  forward_program(p);
+  p->off_planes = p->prog_end;
+  p->ws_bytes = place_program(p->fprog, p->off_planes + p->planes_bytes) + 256;
   build_resident(p);
   if (p->grad) {
     // ------------------------------------------- adjoint elimination layout
@@ -2364,7 +2409,7 @@ int qgm_plan_get_info(const qgm_plan *p, qgm_plan_info *info) {
   info->n_slices = (int64_t)1 << p->slice_vars.size();
   info->max_tensor_entries = p->sim.max_entries;
   info->workspace_bytes = p->ws_bytes;
-  info->arena_bytes = p->sim.arena_peak;
+  info->arena_bytes = p->live_bytes;
   info->bytes_per_slice = p->sim.bytes;
   info->flops_per_slice = p->sim.flops;
   info->max_step_bytes = p->sim.max_step_bytes;

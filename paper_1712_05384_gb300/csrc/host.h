@@ -240,6 +240,10 @@ struct Program {
   std::vector<StepDesc> all;     // every step, offsets as the program uses them
   std::vector<GemmDesc> gemms;
   std::vector<std::vector<int>> prod;  // producer step of each input (-1: a leaf or another pass's tensor)
+  // phase by phase: a segment of small steps, then (if any) one large step
+  std::vector<char> big;           // per step: launched on its own
+  std::vector<int> phase, big_at;  // phase of each step; the large step of each phase (-1: none)
+  int time(int s) const { return 2 * phase[s] + big[s]; }
   std::vector<PStep> steps;
   std::vector<PTask> tasks;
   std::vector<ProgramOp> ops;
@@ -560,6 +564,8 @@ struct qgm_plan {
   std::vector<int32_t> plain_group;
   qgm::Program fprog, gprog;  // the forward and the gradient pass as step programs
   int64_t f_final_off = 0;    // the forward program's final tensor
+  int64_t prog_end = 0;       // end of the tensors' region (both layouts)
+  int64_t live_bytes = 0;     // live intermediates of the larger layout, split sums' temporaries included
   // per leaf: table layout (internal | slice | output variables), offset of
   // its base table and of its derivative tables (floats), its RXY member
   std::vector<std::vector<int>> leaf_layout;
@@ -581,9 +587,14 @@ struct qgm_plan {
 namespace qgm {
 int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p);
 int plan_set_params(qgm_plan *p, const double *params);
+// The phases of P.all (program.cpp): run = 0 gives every small step the first
+// segment after its producers; else the steps keep their order, at most `run`
+// small ones to a segment (less memory is live then).
+void program_phases(Program &P, int Bp, int run);
 // Cut P.all into segments of small steps and large steps launched on their
-// own (program.cpp).  alone[s]: launch step s on its own whatever its size.
-void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char> &alone);
+// own, by its phases.  split: long sums over few outputs in two, through a
+// temporary.
+void build_program(Program &P, int Bp, int64_t off_meta, bool split);
 // Whether a step is launched on its own by its size and form.
 bool program_alone(const StepDesc &d, int Bp);
 // The register-tiled form of a step, where it has one that pays.

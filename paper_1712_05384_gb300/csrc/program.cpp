@@ -74,7 +74,33 @@ bool program_alone(const StepDesc &d, int Bp) {
   return d.gemm >= 0 || (items >= kAloneItems && d.k <= 16 && std::ldexp(items * d.m, d.k) >= kAlone) || !fits(d, Bp);
 }
 
-void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char> &alone) {
+void program_phases(Program &P, int Bp, int run) {
+  const int n = (int)P.all.size();
+  P.big.assign(n, 0);
+  P.phase.assign(n, 0);
+  P.big_at.clear();
+  int in_run = 0;  // small steps in the present segment (run > 0)
+  for (int s = 0; s < n; ++s) {
+    P.big[s] = program_alone(P.all[s], Bp);
+    if (P.big[s] || (run > 0 && in_run == run)) {
+      // the present phase ends, with this step or without a large one
+      P.big_at.push_back(P.big[s] ? s : -1);
+      in_run = 0;
+      if (P.big[s]) {
+        P.phase[s] = (int)P.big_at.size() - 1;
+        continue;
+      }
+    }
+    ++in_run;
+    if (run > 0) P.phase[s] = (int)P.big_at.size();
+    else
+      for (int q : P.prod[s])
+        if (q >= 0) P.phase[s] = std::max(P.phase[s], P.big[q] ? P.phase[q] + 1 : P.phase[q]);
+  }
+  P.big_at.push_back(-1);
+}
+
+void build_program(Program &P, int Bp, int64_t off_meta, bool split) {
   const int n = (int)P.all.size();
   P.steps.clear();
   P.steps.reserve(n + n / 4 + 8);
@@ -83,21 +109,9 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
   P.n_segments = 0;
   P.n_tmp = 0;
   P.tmp_bytes = 0;
-  // phase of a step: a large step b of the launch order belongs to phase b
-  // (after segment b), a small one to the first segment after its producers
-  std::vector<int> phase(n, 0), big_of;
-  std::vector<char> big(n, 0);
-  for (int s = 0; s < n; ++s) {
-    const StepDesc &d = P.all[s];
-    big[s] = alone[s] || program_alone(d, Bp);
-    if (big[s]) {
-      phase[s] = (int)big_of.size();
-      big_of.push_back(s);
-    } else {
-      for (int q : P.prod[s])
-        if (q >= 0) phase[s] = std::max(phase[s], big[q] ? phase[q] + 1 : phase[q]);
-    }
-  }
+  const std::vector<char> &big = P.big;
+  const std::vector<int> &phase = P.phase;
+  std::vector<int64_t> tmp(P.big_at.size(), 0);  // bytes of temporaries, which a later segment reuses
   // small steps as PSteps; a long sum over few outputs is split in two: the
   // sum over its low summed variables for every value of the high ones, into
   // a temporary, then the sum over those
@@ -139,7 +153,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
         nd.deps.push_back(node_of[q]);
     set_units(t);
     int hi = 0;  // summed variables left to the second step
-    while (t.k - hi - t.lg > 5 && ((int64_t)t.items << (t.lg + hi)) < kLanes) ++hi;
+    while (split && t.k - hi - t.lg > 5 && ((int64_t)t.items << (t.lg + hi)) < kLanes) ++hi;
     if (hi < 2) {
       for (int i = 0; i < d.m; ++i) t.in[i] = make_in(d.in[i], d.w_out, off_meta);
       node_of[s] = add(std::move(nd));
@@ -176,7 +190,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
       std::copy(term.begin(), term.end(), p.run + row.size());
       t.in[i] = p;
     }
-    t.out_off = -1 - P.tmp_bytes;  // placed by place_program
+    t.out_off = -1 - tmp[nd.phase];  // placed by place_program
     t.out_meta = -1 - P.n_tmp;
     set_units(t);
     PStep &u = second.s;
@@ -190,7 +204,8 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
     u.in[0].run[u.in[0].nrow] = (uint32_t)(0 | hi << 8 | w << 16);
     u.in[0].nterm = 1;
     set_units(u);
-    P.tmp_bytes += ((rows << hi) * (d.batched_out ? Bp : 1) * 8 + 255) & ~int64_t(255);
+    tmp[nd.phase] += ((rows << hi) * (d.batched_out ? Bp : 1) * 8 + 255) & ~int64_t(255);
+    P.tmp_bytes = std::max(P.tmp_bytes, tmp[nd.phase]);
     P.n_tmp += 1;
     second.deps.push_back(add(std::move(nd)));
     node_of[s] = add(std::move(second));
@@ -225,7 +240,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
   });
   std::vector<int> at(nn, -1);  // node -> index in P.steps
   size_t o = 0;
-  for (int ph = 0; ph <= (int)big_of.size(); ++ph) {
+  for (int ph = 0; ph < (int)P.big_at.size(); ++ph) {
     const int task0 = (int)P.tasks.size();
     double loads = 0;
     for (; o < order.size() && nodes[order[o]].phase == ph; ++o) {
@@ -258,7 +273,7 @@ void build_program(Program &P, int Bp, int64_t off_meta, const std::vector<char>
       P.ops.push_back({-1, task0, (int)P.tasks.size() - task0, 1000000000 + (int64_t)std::min(loads, 6e10)});
       P.n_segments += 1;
     }
-    if (ph < (int)big_of.size()) P.ops.push_back({big_of[ph], 0, 0, 0});
+    if (P.big_at[ph] >= 0) P.ops.push_back({P.big_at[ph], 0, 0, 0});
   }
 }
 

@@ -151,3 +151,22 @@ def test_wait_between_steps_gives_up(q, rows, cols, depth, B):
         assert np.array_equal(p.amplitudes_host(bits), before) and p.status() == 0
     with pytest.raises(q.QgmError):
         q._lib.selftest_program_timeout(p, 10)  # limit out of range
+
+
+@pytest.mark.parametrize("rows,cols,depth,B,budget", [(4, 4, 20, 8, 20000), (4, 5, 24, 16, 400000), (4, 5, 28, 9, 1 << 20)])
+def test_passes_share_their_memory(q, rows, cols, depth, B, budget):
+    # a pass in program order, one step by step (profile) and one for a fixed
+    # assignment use the same memory in turn, in different layouts; the first
+    # plan's budget holds only with a step to a launch
+    c = qi.grid_circuit(rows, cols, depth, 2)
+    bits = qi.bitstrings(c.n, B, 5)
+    d_bits = torch.from_numpy(bits.astype(np.int64)).cuda()
+    p = q.Plan(q.Model(q.Circuit.grid(rows, cols, depth, 2)), batch=B, mem_budget_bytes=budget, executor=q.EXEC_STEPWISE).bind()
+    assert p.info.arena_bytes <= budget
+    ref = sv.amplitudes(c, bits)
+    for _ in range(2):
+        e = errmeasure.measures(p.amplitudes_host(bits), ref, c.n)
+        assert p.status() == 0 and e["rel"] < TOL and e["abs"] < TOL, e
+        p.profile(d_bits, torch.empty(2 * B, dtype=torch.float64, device="cuda"))
+        raw, ex = p.eliminate_fixed([int(bits[1]) >> j & 1 for j in range(c.n)])
+        assert abs(raw[0] * 2.0 ** ex - ref[1]) * 2.0 ** (c.n / 2) < TOL

@@ -387,3 +387,18 @@ def test_folded_steps_are_the_convertible_ones(rows, cols, depth, batch):
     for g in gs:
         fold = g["tc"] and g["o_bat"] and (g["a_bat"] != g["b_bat"]) and batch > 1
         assert g["conv_ok"] == int(bool(fold)), g
+
+
+@pytest.mark.parametrize("rows,cols,depth,batch,budget", [(4, 4, 24, 1000, 16 << 20), (5, 6, 28, 8, 32 << 20),
+                                                          (5, 6, 30, 16, 128 << 20), (4, 4, 20, 8, 20000),
+                                                          (4, 6, 26, 4, 60000)])
+def test_workspace_keeps_to_the_memory_budget(rows, cols, depth, batch, budget):
+    # the budget caps the live intermediates of a pass however its steps are
+    # launched: beside them the workspace holds the leaves, the bitstrings and
+    # amplitudes, the plan's tables (256 KiB and a few KiB a step) and the
+    # operand planes of tensor-core steps (none without them)
+    m = Q.Model(Q.Circuit.grid(rows, cols, depth, 0))
+    p = Q.Plan(m, batch=batch, mem_budget_bytes=budget, executor=Q.EXEC_STEPWISE, precision="fp32")
+    assert p.info.arena_bytes <= budget
+    leaves = m.info.n_factors * 4 * 8 * p.info.batch_padded
+    assert p.info.workspace_bytes <= budget + leaves + 48 * p.info.batch_padded + (256 << 10) + 4096 * p.info.n_steps

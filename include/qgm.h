@@ -232,7 +232,9 @@ typedef struct {
 enum {
   QGM_EXEC_AUTO = 0,      /* compiled resident, else resident, when a chunk's live
                              set fits in shared memory; else stepwise */
-  QGM_EXEC_STEPWISE = 1,  /* one kernel per step over the whole batch (CUDA graph) */
+  QGM_EXEC_STEPWISE = 1,  /* step by step over the whole batch: a launch per large
+                             step, small steps sharing launches (CUDA graph,
+                             where a pass has more than a few launches) */
   QGM_EXEC_RESIDENT = 2,  /* one persistent launch: each CTA runs all steps for a
                              chunk of bitstrings out of shared memory, reading a
                              descriptor per step */
@@ -256,8 +258,9 @@ typedef struct {
   double bytes_per_slice;     /* algorithmic bytes (inputs read + output written) */
   double flops_per_slice;     /* algorithmic real flops of the products and sums */
   double max_step_bytes;      /* algorithmic bytes of the largest step */
-  int32_t n_gemm_steps;       /* steps run by the tiled GEMM kernel */
-  int32_t n_tile_steps;       /* batched steps run with a register tile */
+  int32_t n_gemm_steps;       /* GEMM-shaped steps */
+  int32_t n_tile_steps;       /* batched steps whose outputs share their largest
+                                 input's values */
   int32_t n_nested_steps;     /* steps whose compiled form sums some variables
                                  in an inner loop over part of the inputs */
   int32_t n_gemm_tc_steps;    /* of the GEMM steps, those with a tensor-core
@@ -278,11 +281,14 @@ int qgm_plan_get_slice_vars(const qgm_plan *p, int32_t *vars, int64_t cap, int64
  * variables of the output), k[s] (variables summed), n_in[s], batched[s]. */
 int qgm_plan_get_steps(const qgm_plan *p, int32_t *out_rank, int32_t *k, int32_t *n_in,
                        int32_t *batched, int64_t cap);
-/* Kernel that runs step s in the stepwise executor: 0 product-sum without a
- * batch axis, 1 batched product-sum, 2 batched with a register tile, 3 tiled
- * GEMM, 4 a small step without a batch axis among neighbours of the same
- * kind.  Small steps of any kind share a launch (a segment of the pass's step
- * program); large ones run with the kernel named here. */
+/* Shape of step s, as the stepwise executor sorts its steps: 0 product-sum
+ * without a batch axis, 1 batched product-sum, 2 batched, with outputs that
+ * share their largest input's values, 3 GEMM-shaped, 4 a small step without a
+ * batch axis among neighbours of the same kind.  The shape does not name the
+ * kernel: steps below a size share a launch (a segment of the pass's step
+ * program) whatever their shape, and larger ones of shape 1 to 3 run register-
+ * tiled, on the tensor cores or with the plain kernel of their shape by size,
+ * precision and tuning. */
 int qgm_plan_get_step_kernels(const qgm_plan *p, int32_t *kind, int64_t cap);
 
 /* Algorithmic cost of step s: bytes[s] (inputs read once + output written,
@@ -345,8 +351,8 @@ int qgm_plan_bind(qgm_plan *p, void *d_workspace, size_t ws_bytes, void *stream)
  * with <x_b|C|0^n> for b < B.  With k = popcount(opts.open_mask) > 0, d_out
  * holds B * 2^k amplitudes: entry b * 2^k + c is x_b with its open qubits
  * set from c (bit i of c = the i-th lowest open qubit).  Runs every step of the plan, all slices, on
- * `stream` (asynchronous; the first call with a given pointer set also
- * builds a CUDA graph).  Requires QGM_OUT_BATCH and a bound workspace.
+ * `stream` (asynchronous; the first call with a given pointer set may also
+ * build a CUDA graph).  Requires QGM_OUT_BATCH and a bound workspace.
  * Errors: QGM_ERR_ARG (mode, B, unbound), QGM_ERR_CUDA. */
 int qgm_amplitudes(qgm_plan *p, const uint64_t *d_bitstrings, int64_t B, double *d_out,
                    void *stream);

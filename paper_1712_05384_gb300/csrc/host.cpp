@@ -1917,19 +1917,6 @@ int build_plan(const Model &m, const qgm_plan_opts &o, qgm_plan *p) {
     }
   }
   p->tune.assign(p->steps.size(), StepTune{});
-  // runs of at least two consecutive small batch-free product-sum steps (at
-  // most 2^12 outputs and 2^16 products each), as step reports list them
-  p->plain_group.assign(p->steps.size(), 0);
-  for (size_t s0 = 0; s0 < p->steps.size();) {
-    auto small = [&](size_t s) {
-      const StepDesc &d = p->steps[s];
-      return d.gemm < 0 && !d.batched_out && d.w_out <= 12 && d.w_out + d.k <= 16;
-    };
-    size_t s1 = s0;
-    while (s1 < p->steps.size() && small(s1)) ++s1;
-    if (s1 - s0 >= 2) p->plain_group[s0] = (int32_t)(s1 - s0);
-    s0 = s1 > s0 ? s1 : s0 + 1;
-  }
   // the split operand planes of the largest tensor-core step, after the
   // tensors (of either layout), then the step program's tables
   p->ws_fwd_bytes = p->ws_bytes;
@@ -2470,9 +2457,15 @@ int qgm_plan_get_step_kernels(const qgm_plan *p, int32_t *kind, int64_t cap) {
     const StepDesc &d = p->steps[s];
     kind[s] = d.gemm >= 0 ? 3 : (d.tile_t > 0 ? 2 : (d.batched_out ? 1 : 0));
   }
-  // steps inside a run of small batch-free steps
-  for (size_t s = 0; s < p->plain_group.size(); ++s)
-    for (int32_t j = 0; j < p->plain_group[s] && (int64_t)(s + j) < cap; ++j) kind[s + j] = 4;
+  // runs of at least two consecutive small batch-free product-sum steps (at
+  // most 2^12 outputs and 2^16 products each)
+  auto small = [&](int64_t s) {
+    const StepDesc &d = p->steps[s];
+    return d.gemm < 0 && !d.batched_out && d.w_out <= 12 && d.w_out + d.k <= 16;
+  };
+  const int64_t n = (int64_t)p->steps.size();
+  for (int64_t s = 0; s < std::min(cap, n); ++s)
+    if (small(s) && ((s > 0 && small(s - 1)) || (s + 1 < n && small(s + 1)))) kind[s] = 4;
   return QGM_OK;
 }
 

@@ -559,9 +559,6 @@ struct qgm_plan {
   int64_t planes_bytes = 0; // its size (the largest tensor-core step's two operands)
   int64_t ws_fwd_bytes = 0; // workspace the forward pass needs without that region
   std::vector<qgm::StepTune> tune;  // per step of `steps` (autotuner choices)
-  // runs of consecutive small steps without a batch axis:
-  // plain_group[s] = steps in the run starting at s (0: none)
-  std::vector<int32_t> plain_group;
   qgm::Program fprog, gprog;  // the forward and the gradient pass as step programs
   int64_t f_final_off = 0;    // the forward program's final tensor
   int64_t prog_end = 0;       // end of the tensors' region (both layouts)

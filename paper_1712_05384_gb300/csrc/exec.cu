@@ -2865,8 +2865,11 @@ static void launch_leaves(qgm_plan *p, const uint64_t *d_bits, int64_t B, cudaSt
 // then the product (see k_split and k_gemm_tc).
 // Two instances a tile (k_gemm_tc, G = 2): the lowest shared variable is the
 // output's lowest index bit, with no batch axis below it, and the product is
-// short.  Both instances' MMAs of 64 columns take about 0.6 us a chunk of 16
-// summed entries, the tile's stores 3 us: up to four chunks hide behind them.
+// short: both instances' MMAs take less time than the tile's stores for up to
+// four chunks of 16 summed entries.  Tiles of 128 columns (one pair of
+// accumulators) and of 64 (two): M 2^16 x N 2^8 x K 16 x 16 x 4 entries 1.52
+// and 1.61 ms, 2^10 x 2^9 x 4 x 4 x 8 0.035 and 0.044, 2^11 x 2^6 x 32 x 32 x 2
+// the same tiles; 128 by rule.
 static bool tc_pair(const GemmDesc &g) {
   return g.ns > 0 && g.sO[0] == 0 && !(g.o_bat && !g.o_bout) && g.nk <= 6;
 }
@@ -3042,7 +3045,7 @@ static cudaError_t tc_set_smem() {
 static bool tc_step(const StepDesc &d, const GemmDesc *gemms, int Bp, int planes, bool bound, const StepTune *tn, TcCfg *c) {
   if (d.gemm < 0 || (tn && tn->ps)) return false;
   const GemmDesc &g = gemms[d.gemm];
-  *c = tc_config(g, Bp, planes, tn && tn->nt_cap ? tn->nt_cap : tc_pair(g) && !(tn && tn->conv) ? 64 : 256);
+  *c = tc_config(g, Bp, planes, tn && tn->nt_cap ? tn->nt_cap : tc_pair(g) && !(tn && tn->conv) ? 128 : 256);
   if (!c->ok) return false;
   MmStep mm;
   const bool outer = g.a_bout || g.b_bout || g.o_bout, forced = tn && tn->nt_cap;

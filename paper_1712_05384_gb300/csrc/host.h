@@ -417,17 +417,16 @@ std::vector<int> rotations(const qgm_plan *p);
 // ROTATION_BITS for every parametrised gate, whose table (the plan is kept over
 // new angles) may have entries as small as one likes.  It is an estimate (sums
 // may cancel further, angles be smaller), so it stays far from the range:
-// tensors are measured instead such that no step's output, and no step's inputs
-// together, have more than SLACK_BITS; of the inputs, the one with the fewest
-// entries that suffices.  Behind a rotation, a product of measured tensors may
+// tensors are measured instead, the loosest first, such that no step's output,
+// and no step's inputs together, have more than SLACK_BITS.  Behind a rotation, a product of measured tensors may
 // be small everywhere (large entries of one meeting small ones of the other):
 // a step that reads one measured is itself measured, as is the final tensor
 // (non-finite values reach it and set the status there).
 //
 // Over grids of up to 28 qubits and depths of 8 to 60 the largest product of
-// raw values of any step is above 2^-65 (2^-133, out of range, when only a
+// raw values of any step is above 2^-70 (2^-133, out of range, when only a
 // step's own output was held to 48 bits).
-constexpr int SLACK_BITS = 40, ROTATION_BITS = 8;
+constexpr int SLACK_BITS = 48, ROTATION_BITS = 9;
 struct StaticBound {
   int k = 0;               // |out| <= 2^k
   bool exp_known = false;  // every input's exponent is known too:

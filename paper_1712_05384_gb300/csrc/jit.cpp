@@ -400,35 +400,22 @@ std::map<int, StaticBound> static_bounds(const qgm_plan *p, const ResidentLayout
       else ++scaled;
       if (bound.count(r.in[i].meta)) slack += loose[r.in[i].meta].bits;
     }
-    // the smallest input whose slack leaves at most `most` without it, the
-    // loosest where there is none (-1: no input has slack)
-    auto pick = [&](int most) {
+    auto loosest = [&]() {
       int best = -1;
-      bool enough = false;
-      for (int i = 0; i < r.m; ++i) {
-        if (!bound.count(r.in[i].meta)) continue;
-        const Slack &s = loose[r.in[i].meta];
-        const bool e = slack - s.bits <= most;
-        const bool better = best < 0 || e > enough ||
-                            (e == enough && (e ? s.entries < loose[r.in[best].meta].entries
-                                               : s.bits > loose[r.in[best].meta].bits));
-        if (better) {
-          best = i;
-          enough = e;
-        }
-      }
+      for (int i = 0; i < r.m; ++i)
+        if (bound.count(r.in[i].meta) && (best < 0 || loose[r.in[i].meta].bits > loose[r.in[best].meta].bits)) best = i;
       return best;
     };
     auto measure = [&](int i) {
       slack -= loose[r.in[i].meta].bits;
       bound.erase(r.in[i].meta);
     };
-    while (slack > 0 && leaf + slack > SLACK_BITS) measure(pick(SLACK_BITS - leaf));
+    while (slack > 0 && leaf + slack > SLACK_BITS) measure(loosest());
     if (r.out_meta == L.final_meta) continue;
     const int own = r.k + scaled + leaf;
     if (own + slack > SLACK_BITS) {
-      // measure one input in place of the output where that is less work
-      const int i = pick(SLACK_BITS - own);
+      // measure an input in place of the output where that is less work
+      const int i = loosest();
       if (i < 0 || slack - loose[r.in[i].meta].bits > SLACK_BITS - own || loose[r.in[i].meta].entries >= entries) continue;
       measure(i);
     }

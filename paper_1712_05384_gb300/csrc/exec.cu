@@ -2364,28 +2364,29 @@ __global__ void __launch_bounds__(SET_THREADS) k_xeb(const double2 *a, int64_t B
 }
 
 // Scan over a block of 256 of one value per thread: the sum of the values
-// before a thread's own; *sum = total.
+// before a thread's own; *sum = total.  (The warps' sums are added up by one
+// warp: FP64 additions by every thread cost more than the barrier.)
 __device__ __forceinline__ double block_scan(double v, double *sum) {
-  __shared__ double wsum[8];
+  __shared__ double wsum[8], wpre[9];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  double ex = 0;
   for (int o = 1; o < 32; o <<= 1) {
     const double u = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += u;
   }
-  ex = __shfl_up_sync(0xffffffffu, v, 1);
+  double ex = __shfl_up_sync(0xffffffffu, v, 1);
   if (lane == 0) ex = 0;
-  __syncthreads();  // the previous call's wsum is read
   if (lane == 31) wsum[wid] = v;
-  __syncthreads();
-  double before = 0, all = 0;
+  __syncthreads();  // (and the previous call's wpre is read)
+  if (threadIdx.x < 9) {
+    double before = 0;
 #pragma unroll
-  for (int w = 0; w < 8; ++w) {
-    before += w < wid ? wsum[w] : 0.0;
-    all += wsum[w];
+    for (int w = 0; w < 8; ++w)
+      if (w < (int)threadIdx.x) before += wsum[w];
+    wpre[threadIdx.x] = before;
   }
-  *sum = all;
-  return before + ex;
+  __syncthreads();
+  *sum = wpre[8];
+  return wpre[wid] + ex;
 }
 
 // Sums of p as their bits: non-negative values order like them, NaN above all

@@ -22,10 +22,10 @@
 // plan image that hold something, built at bind.
 //
 // What bounds it: one CTA alone, the chain of dependency levels (5x5 depth 20:
-// 17 levels, 16.6 us before these additions, 10.4 now; 4x4 depth 12: 3.9 and
-// 2.4 us); a full SM (7 CTAs, shared memory), instruction issue: 1024
-// bitstrings of 5x5 depth 20 26.9 -> 21.0 M warp instructions, 47% of them
-// FP32 arithmetic, 37.2 -> 28.5 us (20 -> 26 TFLOP/s).
+// 17 levels, 27.9 us before these additions, 20.5 now, caches cold; 4x4 depth
+// 12: 7.1 and 5.7 us); a full SM (7 CTAs, shared memory), instruction issue:
+// 1024 bitstrings of 5x5 depth 20 26.9 -> 21.5 M warp instructions, 36.5 ->
+// 28.7 us (20 -> 26 TFLOP/s).
 #include <cuda_runtime.h>
 #include <dlfcn.h>
 
